@@ -584,9 +584,10 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
     cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned) * launches.size(), cs);
     bool cap_ok = true;
     std::vector<int> ibs;
-    for (const Ordered& o : ordered) {
+    for (Ordered& o : ordered) {
         int ib = 0;
-        cap_ok = cap_ok && launch_point_sort(o.user.x, o.user.y, o.user.z, o.user.n, order_level, o.pairs, &ib, cs) == OT_OK;
+        cap_ok = cap_ok && launch_point_sort(o.user.x, o.user.y, o.user.z, o.user.n, order_level, o.pairs, &ib,
+                                             &o.pairs, cs) == OT_OK;
         ibs.push_back(ib);
         k_gather_points<<<grid_b(o.user.n), 256, 0, cs>>>(o.pairs, o.user.n, (1ULL << ib) - 1, o.user.x, o.user.y,
                                                           o.user.z, o.xs, o.ys, o.zs);

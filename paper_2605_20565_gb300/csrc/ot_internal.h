@@ -79,28 +79,18 @@ ot_status scan_u32_ws(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t
 // Stable LSD radix sort of n uint64 by bits [bit0, bit1) (8-bit digits).  d_tmp: n uint64
 // scratch.  Result in d_keys.  Temporaries (histograms) are stream-ordered allocations.
 ot_status radix_sort_u64(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, cudaStream_t s);
-// Workspace bytes of radix_sort_u64_ws / radix_sort_u64_dn (histograms, offsets and the
-// scan's temporaries): with it those sorts allocate nothing.
+// The same sort with caller workspace of radix_ws_bytes(n) bytes: nothing is allocated.
+// d_n (nullable): the key count in device memory, at most n.  *result (nullable): the buffer
+// (d_keys or d_tmp) left with the sorted keys; without it they are in d_keys.
 size_t radix_ws_bytes(int64_t n);
-// Sort of the first *d_n (device value, <= n_max) keys with workspace of radix_ws_bytes(n_max)
-// bytes; *result is the buffer (d_keys or d_tmp) holding the sorted keys.
-ot_status radix_sort_u64_dn(uint64_t* d_keys, uint64_t* d_tmp, int64_t n_max, const uint32_t* d_n, int bit0,
-                            int bit1, void* ws, uint64_t** result, cudaStream_t s);
-// Same sort with caller-provided workspace (no allocation): ws of radix_ws_bytes(n) bytes.
 ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
-                            cudaStream_t s);
+                            cudaStream_t s, const uint32_t* d_n = nullptr, uint64_t** result = nullptr);
 // Compaction: out[j] = in[i] for the i with flag[i] != 0, in order; *h_count on the host
 // (synchronises).  d_scan: n uint32 scratch.
 ot_status compact_u64(const uint64_t* d_in, const uint32_t* d_flag, uint32_t* d_scan, int64_t n, uint64_t* d_out,
                       int64_t* h_count, cudaStream_t s);
 // Sorted input -> unique values in place; *h_count on the host (synchronises).
 ot_status unique_u64(uint64_t* d_keys, int64_t n, int64_t* h_count, cudaStream_t s);
-
-// Allocation-free scan / radix sort: temporaries in caller scratch.
-ot_status scan_u32_noalloc(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* tmp, cudaStream_t s);
-size_t radix_noalloc_bytes(int64_t n);
-ot_status radix_sort_u64_noalloc(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
-                                 cudaStream_t s);
 
 // builder (ot_build.cu) ------------------------------------------------------------------------
 ot_status build_tree(const ot_sphere* h_spheres, int n, const ot_build_params* p, cudaStream_t s, ot_octree* t);
@@ -149,7 +139,7 @@ bool mates_fit(const ot_octree* t);
 size_t order_ws_bytes(int64_t n);
 bool order_fits(int64_t n, int level);
 ot_status launch_point_sort(const double* x, const double* y, const double* z, int64_t n, int level,
-                            uint64_t* pairs, int* ib_out, cudaStream_t s);
+                            uint64_t* pairs, int* ib_out, uint64_t** sorted, cudaStream_t s);
 
 // spreading (ot_spread.cu) ---------------------------------------------------------------------
 size_t spread_ws_bytes(const ot_octree* t, int kernel, int64_t n);

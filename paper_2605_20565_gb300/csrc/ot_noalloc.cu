@@ -21,6 +21,9 @@ namespace {
 // address: the address comes from cudaGetSymbolAddress, once per device and context.
 static __device__ __align__(256) unsigned char g_spread_scratch[OT_NOALLOC_SCRATCH_BYTES];
 
+// The documented limits of octtrack.h (pairs, sort buffer and tile counts must fit the array).
+constexpr int64_t kMaxMarkersPeskin4 = 150635, kMaxMarkersRoma3 = 508394;
+
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_scratch_ptr[kMaxDevices] = {};
@@ -86,7 +89,9 @@ extern "C" ot_status ot_spread_noalloc(const ot_octree* t, int kernel, const dou
     if (t->lmax < 1) return OT_ERR_ARG;
     if (n == 0) return OT_OK;
     if (n * 64 >= (1LL << 32)) return OT_ERR_LIMIT;
-    if (ot::spread_noalloc_bytes(kernel, n) > (size_t)OT_NOALLOC_SCRATCH_BYTES) return OT_ERR_LIMIT;
+    if (n > (kernel == OT_PESKIN4 ? kMaxMarkersPeskin4 : kMaxMarkersRoma3) ||
+        ot::spread_noalloc_bytes(kernel, n) > (size_t)OT_NOALLOC_SCRATCH_BYTES)
+        return OT_ERR_LIMIT;
     void* scratch = nullptr;
     cudaError_t e = scratch_address(&scratch);
     if (e != cudaSuccess) return ot::cuda_status(e);

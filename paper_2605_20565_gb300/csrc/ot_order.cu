@@ -47,18 +47,18 @@ size_t order_ws_bytes(int64_t n) { return 2 * sizeof(uint64_t) * (size_t)n + rad
 
 bool order_fits(int64_t n, int level) { return level >= 1 && level <= MAXLEVEL && 3 * level + index_bits(n) <= 64; }
 
-// Sorts (cell key << ib | index) pairs of the n points into `pairs` (workspace: pairs, tmp and
-// the radix histograms, order_ws_bytes(n) bytes from `pairs`); the low ib bits of each sorted
-// pair are a point index.  Capturable in a CUDA graph.
+// Sorts (cell key << ib | index) pairs of the n points in the workspace from `pairs` (pairs, tmp
+// and the radix histograms, order_ws_bytes(n) bytes); *sorted: where they are left, and the low
+// ib bits of each are a point index.  Capturable in a CUDA graph.
 ot_status launch_point_sort(const double* x, const double* y, const double* z, int64_t n, int level,
-                            uint64_t* pairs, int* ib_out, cudaStream_t s) {
+                            uint64_t* pairs, int* ib_out, uint64_t** sorted, cudaStream_t s) {
     const int ib = index_bits(n);
     *ib_out = ib;
     uint64_t* tmp = pairs + n;
     void* rws = tmp + n;
     k_point_keys<<<grid_o(n), 256, 0, s>>>(x, y, z, n, level, ib, pairs);
     count_launch();
-    return radix_sort_u64_ws(pairs, tmp, n, ib, ib + 3 * level, rws, s);
+    return radix_sort_u64_ws(pairs, tmp, n, ib, ib + 3 * level, rws, s, nullptr, sorted);
 }
 
 } // namespace ot
@@ -81,15 +81,11 @@ extern "C" ot_status ot_points_morton_order(const double* d_x, const double* d_y
         ws_bytes < order_ws_bytes(n))
         return OT_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    uint64_t* pairs = static_cast<uint64_t*>(d_workspace);
-    uint64_t* tmp = pairs + n;
-    void* rws = tmp + n;
-    const int ib = index_bits(n);
-    k_point_keys<<<grid_o(n), 256, 0, s>>>(d_x, d_y, d_z, n, level, ib, pairs);
-    count_launch();
-    ot_status st = radix_sort_u64_ws(pairs, tmp, n, ib, ib + 3 * level, rws, s);
+    uint64_t* sorted = nullptr;
+    int ib = 0;
+    ot_status st = launch_point_sort(d_x, d_y, d_z, n, level, static_cast<uint64_t*>(d_workspace), &ib, &sorted, s);
     if (st != OT_OK) return st;
-    k_pair_index<<<grid_o(n), 256, 0, s>>>(pairs, n, ((uint64_t)1 << ib) - 1, d_perm);
+    k_pair_index<<<grid_o(n), 256, 0, s>>>(sorted, n, ((uint64_t)1 << ib) - 1, d_perm);
     count_launch();
     OT_CUDA(cudaGetLastError());
     return OT_OK;

@@ -139,92 +139,167 @@ ot_status scan_u32(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* d
 }
 
 // ------------------------------------------------------------------------------------------
-// Stable LSD radix sort of uint64 keys, 8-bit digits.  A tile is RT threads x RI rounds; in
-// round r thread t owns element r*RT + t, so (round, warp, lane) order is input order and the
-// scatter ranks each element after every earlier element of the tile with the same digit.
+// Stable LSD radix sort of uint64 keys, digits of up to 8 bits (the bits are split evenly over
+// the passes).  A pass is three launches: digit counts per tile, one block per digit scanning
+// that digit's row of tile counts, and the scatter.  A tile is RT threads x RI keys; warp w owns
+// the tile's keys [w, w + 1) RTILE / RW, 32 at a time, so (warp, round, lane) order is input
+// order.
+// The scatter is bound by its stores: written straight from the ranking rounds, 256 keys go to
+// 256 digits, 8 bytes to a 32-byte sector each, with four block barriers per round.  Instead a
+// warp ranks its keys against its own digit counters (no block barrier), the tile is put in
+// digit order in shared memory and written out in order: 16 consecutive keys per digit on
+// average, 128-byte runs.
 // ------------------------------------------------------------------------------------------
 constexpr int RT = 256, RI = 16, RTILE = RT * RI, RW = RT / 32;
 
 // d_n (nullable): the element count in device memory, at most n (tiles past it stay empty).
-__global__ void k_radix_hist(const uint64_t* __restrict__ in, int64_t n, int shift, uint32_t mask,
-                             uint32_t* __restrict__ hist, int ntiles, const uint32_t* __restrict__ d_n) {
+__global__ void __launch_bounds__(RT) k_radix_hist(const uint64_t* __restrict__ in, int64_t n, int shift,
+                                                   uint32_t mask, uint32_t* __restrict__ hist, int ntiles,
+                                                   const uint32_t* __restrict__ d_n) {
     __shared__ uint32_t cnt[256];
     cnt[threadIdx.x] = 0;
     if (d_n) n = min(n, (int64_t)*d_n);
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * RTILE;
+    if (base + RTILE <= n) {  // a whole tile: every load issued before the first count
+        uint32_t d[RI];
 #pragma unroll
-    for (int r = 0; r < RI; ++r) {
-        int64_t i = base + r * RT + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(uint32_t)(in[i] >> shift) & mask], 1u);
+        for (int r = 0; r < RI; ++r) d[r] = (uint32_t)(__ldg(in + base + r * RT + threadIdx.x) >> shift) & mask;
+#pragma unroll
+        for (int r = 0; r < RI; ++r) atomicAdd(&cnt[d[r]], 1u);
+    } else {
+        for (int r = 0; r < RI; ++r) {
+            const int64_t i = base + r * RT + threadIdx.x;
+            if (i < n) atomicAdd(&cnt[(uint32_t)(in[i] >> shift) & mask], 1u);
+        }
     }
     __syncthreads();
     hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
 }
 
-__global__ void k_radix_scatter(const uint64_t* __restrict__ in, uint64_t* __restrict__ out, int64_t n, int shift,
-                                uint32_t mask, const uint32_t* __restrict__ offs, int ntiles,
-                                const uint32_t* __restrict__ d_n) {
-    __shared__ uint32_t s_base[256];
-    __shared__ uint32_t s_w[RW][256];
+// Block d: exclusive scan of digit d's row of tile counts in place; its total to totals[d].
+constexpr int ROW_T = 512, ROW_I = 4;
+__global__ void __launch_bounds__(ROW_T) k_radix_rows(uint32_t* __restrict__ hist, int ntiles,
+                                                      uint32_t* __restrict__ totals) {
+    __shared__ uint32_t s_warp[33];
+    uint32_t* row = hist + (int64_t)blockIdx.x * ntiles;
+    uint32_t carry = 0;
+    for (int base = 0; base < ntiles; base += ROW_T * ROW_I) {
+        const int i0 = base + (int)threadIdx.x * ROW_I;
+        uint32_t v[ROW_I], sum = 0;
+#pragma unroll
+        for (int k = 0; k < ROW_I; ++k) {
+            v[k] = i0 + k < ntiles ? row[i0 + k] : 0u;
+            sum += v[k];
+        }
+        uint32_t tot;
+        uint32_t run = carry + block_exclusive_scan(sum, s_warp, &tot);
+#pragma unroll
+        for (int k = 0; k < ROW_I; ++k) {
+            if (i0 + k < ntiles) row[i0 + k] = run;
+            run += v[k];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
+}
+
+__global__ void __launch_bounds__(RT) k_radix_scatter(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
+                                                      int64_t n, int shift, uint32_t mask,
+                                                      const uint32_t* __restrict__ offs, int ntiles,
+                                                      const uint32_t* __restrict__ totals,
+                                                      const uint32_t* __restrict__ d_n) {
+    __shared__ uint64_t s_key[RTILE];
+    __shared__ uint32_t s_cnt[RW][256];  // per warp: digit counts, then the warp's first place per digit
+    // per warp and digit, the lanes of the current round (used before the keys are placed)
+    uint32_t (*s_grp)[256] = reinterpret_cast<uint32_t (*)[256]>(s_key);
+    __shared__ uint32_t s_base[256];     // digit: its place in out, less its place in the tile
+    __shared__ uint32_t s_warp[33];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (d_n) n = min(n, (int64_t)*d_n);
-    if ((int64_t)blockIdx.x * RTILE >= n) return;  // block-uniform
-    const unsigned lt = (1u << lane) - 1u;
-    s_base[tid] = offs[(int64_t)tid * ntiles + blockIdx.x];
     const int64_t base = (int64_t)blockIdx.x * RTILE;
+    if (base >= n) return;  // block-uniform
+    const int cnt = (int)min((int64_t)RTILE, n - base);
+    const int first = warp * (RTILE / RW) + lane;
+    uint64_t v[RI];
+#pragma unroll
+    for (int r = 0; r < RI; ++r) v[r] = first + 32 * r < cnt ? __ldg(in + base + first + 32 * r) : 0ULL;
+    const uint32_t toff = offs[(int64_t)tid * ntiles + blockIdx.x], tot = totals[tid];
+#pragma unroll
+    for (int w = 0; w < RW; ++w) s_cnt[w][tid] = 0, s_grp[w][tid] = 0;
+    __syncthreads();
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t rank[RI];
+#pragma unroll
     for (int r = 0; r < RI; ++r) {
-#pragma unroll
-        for (int w = 0; w < RW; ++w) s_w[w][tid] = 0;
-        __syncthreads();
-        const int64_t i = base + r * RT + tid;
-        const bool valid = i < n;
-        uint64_t v = valid ? in[i] : 0ULL;
-        uint32_t d = valid ? ((uint32_t)(v >> shift) & mask) : 256u;
-        unsigned grp = __match_any_sync(0xffffffffu, d);
-        uint32_t rank = __popc(grp & lt);
-        if (valid && rank == 0) s_w[warp][d] = __popc(grp);
-        __syncthreads();
-        {  // digit tid: exclusive prefix over the warps of this round
-            uint32_t run = s_base[tid];
-#pragma unroll
-            for (int w = 0; w < RW; ++w) {
-                uint32_t c = s_w[w][tid];
-                s_w[w][tid] = run;
-                run += c;
-            }
-            s_base[tid] = run;
+        const bool valid = first + 32 * r < cnt;
+        const uint32_t d = (uint32_t)(v[r] >> shift) & mask;
+        // the lanes with this lane's digit: all valid ones when the digits agree (coherent
+        // input), else gathered by an OR in shared memory
+        unsigned grp = __ballot_sync(0xffffffffu, valid);
+        const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);  // every lane takes part
+        if (__any_sync(0xffffffffu, valid && d != d0)) {      // warp-uniform
+            if (valid) atomicOr(&s_grp[warp][d], 1u << lane);
+            __syncwarp();
+            if (valid) grp = s_grp[warp][d];
         }
-        __syncthreads();
-        if (valid) out[s_w[warp][d] + rank] = v;
-        __syncthreads();
+        const uint32_t before = __popc(grp & lt);
+        uint32_t old = 0;
+        if (valid) old = s_cnt[warp][d];
+        __syncwarp();
+        if (valid && before == 0) s_cnt[warp][d] = old + __popc(grp), s_grp[warp][d] = 0;
+        __syncwarp();
+        rank[r] = old + before;
+    }
+    __syncthreads();
+    // digit tid: the warps' places within the digit, the digit's place within the tile and in out
+    uint32_t run = 0, unused;
+#pragma unroll
+    for (int w = 0; w < RW; ++w) {
+        const uint32_t c = s_cnt[w][tid];
+        s_cnt[w][tid] = run;
+        run += c;
+    }
+    const uint32_t start = block_exclusive_scan(run, s_warp, &unused);
+    const uint32_t dig = block_exclusive_scan(tot, s_warp, &unused);
+#pragma unroll
+    for (int w = 0; w < RW; ++w) s_cnt[w][tid] += start;
+    s_base[tid] = dig + toff - start;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RI; ++r)
+        if (first + 32 * r < cnt) s_key[s_cnt[warp][(uint32_t)(v[r] >> shift) & mask] + rank[r]] = v[r];
+    __syncthreads();
+    for (int i = tid; i < cnt; i += RT) {
+        const uint64_t k = s_key[i];
+        out[s_base[(uint32_t)(k >> shift) & mask] + (uint32_t)i] = k;
     }
 }
 
-// Histograms and offsets (256 per tile each), then the scan's temporaries.
+// Tile counts (256 per tile) and the digits' totals.
 size_t radix_ws_bytes(int64_t n) {
-    int64_t nt = (n + RTILE - 1) / RTILE;
-    if (nt < 1) nt = 1;
-    return (size_t)(2 * 256 * nt) * sizeof(uint32_t) + scan_ws_bytes(256 * nt) + 256;
+    const int64_t nt = std::max<int64_t>((n + RTILE - 1) / RTILE, 1);
+    return (size_t)(256 * nt + 256) * sizeof(uint32_t) + 256;
 }
 
-static ot_status radix_passes(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, uint32_t* hist,
-                              uint32_t* offs, cudaStream_t s, const uint32_t* d_n = nullptr,
-                              uint64_t** result = nullptr) {
-    uint32_t* stmp = offs + 256 * ((n + RTILE - 1) / RTILE);
+ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
+                            cudaStream_t s, const uint32_t* d_n, uint64_t** result) {
+    if (result) *result = d_keys;
+    if (n <= 1 || bit1 <= bit0) return OT_OK;
     const int nt = (int)((n + RTILE - 1) / RTILE);
+    uint32_t* hist = static_cast<uint32_t*>(ws);
+    uint32_t* totals = hist + 256 * (int64_t)nt;
     uint64_t* src = d_keys;
     uint64_t* dst = d_tmp;
-    for (int sh = bit0; sh < bit1; sh += 8) {
-        const int nb = std::min(8, bit1 - sh);
+    for (int sh = bit0, passes = (bit1 - bit0 + 7) / 8; passes > 0; --passes) {
+        const int nb = (bit1 - sh + passes - 1) / passes;
         const uint32_t mask = (1u << nb) - 1u;
         k_radix_hist<<<nt, RT, 0, s>>>(src, n, sh, mask, hist, nt, d_n);
-        count_launch();
-        ot_status st = scan_u32_ws(hist, offs, (int64_t)256 * nt, nullptr, stmp, s);
-        if (st != OT_OK) return st;
-        k_radix_scatter<<<nt, RT, 0, s>>>(src, dst, n, sh, mask, offs, nt, d_n);
-        count_launch();
+        k_radix_rows<<<256, ROW_T, 0, s>>>(hist, nt, totals);
+        k_radix_scatter<<<nt, RT, 0, s>>>(src, dst, n, sh, mask, hist, nt, totals, d_n);
+        count_launch(3);
         std::swap(src, dst);
+        sh += nb;
     }
     if (result)
         *result = src;  // the caller takes the sorted keys where the last pass left them
@@ -234,16 +309,6 @@ static ot_status radix_passes(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int 
     return OT_OK;
 }
 
-ot_status radix_sort_u64_dn(uint64_t* d_keys, uint64_t* d_tmp, int64_t n_max, const uint32_t* d_n, int bit0,
-                            int bit1, void* ws, uint64_t** result, cudaStream_t s) {
-    *result = d_keys;
-    if (n_max <= 1 || bit1 <= bit0) return OT_OK;
-    const int64_t nt = (n_max + RTILE - 1) / RTILE;
-    uint32_t* hist = static_cast<uint32_t*>(ws);
-    uint32_t* offs = hist + 256 * nt;
-    return radix_passes(d_keys, d_tmp, n_max, bit0, bit1, hist, offs, s, d_n, result);
-}
-
 ot_status radix_sort_u64(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, cudaStream_t s) {
     if (n <= 1 || bit1 <= bit0) return OT_OK;
     void* ws = nullptr;
@@ -251,15 +316,6 @@ ot_status radix_sort_u64(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0,
     ot_status st = radix_sort_u64_ws(d_keys, d_tmp, n, bit0, bit1, ws, s);
     cudaFreeAsync(ws, s);
     return st;
-}
-
-ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
-                            cudaStream_t s) {
-    if (n <= 1 || bit1 <= bit0) return OT_OK;
-    const int64_t nt = (n + RTILE - 1) / RTILE;
-    uint32_t* hist = static_cast<uint32_t*>(ws);
-    uint32_t* offs = hist + 256 * nt;
-    return radix_passes(d_keys, d_tmp, n, bit0, bit1, hist, offs, s);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -322,75 +378,6 @@ ot_status unique_u64(uint64_t* d_keys, int64_t n, int64_t* h_count, cudaStream_t
     OT_CUDA(cudaFreeAsync(pos, s));
     OT_CUDA(cudaFreeAsync(tmp, s));
     *h_count = m;
-    return OT_OK;
-}
-
-} // namespace ot
-
-// ------------------------------------------------------------------------------------------
-// Allocation-free variants: every temporary lives in caller-provided scratch.
-// ------------------------------------------------------------------------------------------
-namespace ot {
-
-int64_t scan_noalloc_elems(int64_t n) {
-    int64_t total = 0;
-    int64_t m = n;
-    while (m > SCAN_TILE) {
-        const int64_t nt = (m + SCAN_TILE - 1) / SCAN_TILE;
-        total += nt;
-        m = nt;
-    }
-    return total + 1;
-}
-
-// Exclusive scan with the tile totals of every level in tmp (scan_noalloc_elems(n) uint32).
-ot_status scan_u32_noalloc(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* tmp, cudaStream_t s) {
-    if (n <= 0) return OT_OK;
-    const int64_t nt = (n + SCAN_TILE - 1) / SCAN_TILE;
-    if (nt == 1) {
-        k_scan_tiles<<<1, SCAN_T, 0, s>>>(d_in, d_out, n, nullptr);
-        count_launch();
-    } else {
-        uint32_t* tiles = tmp;
-        k_scan_tiles<<<(unsigned)nt, SCAN_T, 0, s>>>(d_in, d_out, n, tiles);
-        count_launch();
-        ot_status st = scan_u32_noalloc(tiles, tiles, nt, tmp + nt, s);
-        if (st != OT_OK) return st;
-        k_scan_add<<<(unsigned)nt, 256, 0, s>>>(d_out, n, tiles);
-        count_launch();
-    }
-    OT_CUDA(cudaGetLastError());
-    return OT_OK;
-}
-
-size_t radix_noalloc_bytes(int64_t n) {
-    int64_t nt = (n + RTILE - 1) / RTILE;
-    if (nt < 1) nt = 1;
-    return (size_t)(2 * 256 * nt + scan_noalloc_elems(256 * nt)) * sizeof(uint32_t) + 256;
-}
-
-ot_status radix_sort_u64_noalloc(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
-                                 cudaStream_t s) {
-    if (n <= 1 || bit1 <= bit0) return OT_OK;
-    const int nt = (int)((n + RTILE - 1) / RTILE);
-    uint32_t* hist = static_cast<uint32_t*>(ws);
-    uint32_t* offs = hist + 256 * (int64_t)nt;
-    uint32_t* stmp = offs + 256 * (int64_t)nt;
-    uint64_t* src = d_keys;
-    uint64_t* dst = d_tmp;
-    for (int sh = bit0; sh < bit1; sh += 8) {
-        const int nb = std::min(8, bit1 - sh);
-        const uint32_t mask = (1u << nb) - 1u;
-        k_radix_hist<<<nt, RT, 0, s>>>(src, n, sh, mask, hist, nt, nullptr);
-        count_launch();
-        ot_status st = scan_u32_noalloc(hist, offs, (int64_t)256 * nt, stmp, s);
-        if (st != OT_OK) return st;
-        k_radix_scatter<<<nt, RT, 0, s>>>(src, dst, n, sh, mask, offs, nt, nullptr);
-        count_launch();
-        std::swap(src, dst);
-    }
-    if (src != d_keys) OT_CUDA(cudaMemcpyAsync(d_keys, src, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s));
-    OT_CUDA(cudaGetLastError());
     return OT_OK;
 }
 

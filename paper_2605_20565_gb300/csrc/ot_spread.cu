@@ -471,7 +471,7 @@ ot_status spread_sorted(const ot_octree* t, const double* x, const double* y, co
     // so a0 >> 3 is distinct for distinct blocks and keeps their order: sorting on it skips 3 bits
     const int bits = leaf_bits(t->n + 8);
     uint64_t* sorted = pairs;
-    if ((st = radix_sort_u64_dn(pairs, tmp, np, d_np, 35, 32 + bits, rws, &sorted, s)) != OT_OK) return st;
+    if ((st = radix_sort_u64_ws(pairs, tmp, np, 35, 32 + bits, rws, s, d_np, &sorted)) != OT_OK) return st;
     auto kr = k_spread_reduce_rec<T, K>;
     kr<<<grid_for(kr, 256, 0, (np + RC - 1) / RC), 256, 0, s>>>(sorted, d_np, recs, f);  // warps split the pairs
     count_launch();
@@ -528,7 +528,7 @@ namespace ot {
 
 size_t spread_noalloc_bytes(int kernel, int64_t n) {
     const int64_t np = n * stencil_cells(kernel);
-    return (size_t)np * 16 + radix_noalloc_bytes(np) + 256;
+    return (size_t)np * 16 + radix_ws_bytes(np) + 256;
 }
 
 namespace {
@@ -547,7 +547,7 @@ ot_status sorted_noalloc(const ot_octree* t, const double* x, const double* y, c
     ke<<<grid_for(ke, 256, smem, n), 256, smem, s>>>(v, x, y, z, n, pairs);
     count_launch();
     OT_CUDA(cudaGetLastError());
-    if ((st = radix_sort_u64_noalloc(pairs, tmp, np, 32, 32 + leaf_bits(t->n), rws, s)) != OT_OK) return st;
+    if ((st = radix_sort_u64_ws(pairs, tmp, np, 32, 32 + leaf_bits(t->n), rws, s)) != OT_OK) return st;
     auto kr = k_spread_reduce<float, K>;
     kr<<<grid_for(kr, 256, 0, (np + RC - 1) / RC), 256, 0, s>>>(pairs, np, t->lmax, x, y, z, F, dV, n, f);
     count_launch();
