@@ -267,7 +267,7 @@ ot_status ot_interpolate_f64(const ot_octree* t, int kernel, const double* d_x, 
 ot_status ot_interpolate_workspace_size(const ot_octree* t, int kernel, int fp64, size_t* bytes);
 
 /* Workspace for OT_SORTED spreading of n markers with the given kernel: every temporary of
- * the sorted spreading (pairs, sort buffers, histograms, scan totals, marker records), so that
+ * the sorted spreading (tile keys, sort buffer and counts, marker records, run table), so that
  * ot_spread allocates nothing. */
 ot_status ot_spread_workspace_size(const ot_octree* t, int kernel, int64_t n, size_t* bytes);
 
@@ -275,8 +275,9 @@ ot_status ot_spread_workspace_size(const ot_octree* t, int kernel, int64_t n, si
  * F(x)): f(cell) += sum_k F_k phi phi phi dV_k / h^3, h = 2^-lmax, dV_k = h^3 when d_dV is
  * NULL (the paper's literal form).  d_F: 3 planes of n floats; d_f: float4 per leaf,
  * ACCUMULATED (the caller zeroes it), component w untouched.
- *   OT_SORTED: one pair per (marker, overlapping 2x2x2 block of finest cells) is radix-sorted
- *     by block (stable); each block sums its 8 cells' contributions in marker order:
+ *   OT_SORTED: the markers are radix-sorted (stable) by the tile of 4x4x4 finest cells that
+ *     their stencil starts in; each tile sums its cells' contributions from the 8 tiles whose
+ *     stencils reach it, in a fixed order of these and in marker order within each:
  *     bit-identical run to run and for any launch shape.
  *     Needs d_workspace of ot_spread_workspace_size bytes (16-byte aligned); nothing is
  *     allocated.
@@ -298,9 +299,9 @@ ot_status ot_spread_f64(const ot_octree* t, int kernel, int mode, const double* 
  * callers that cannot call cudaMalloc, e.g. a solver whose memory pool already owns the
  * device, or code that must not risk an allocation's synchronisation or failure mid-step).
  * Same result as ot_spread(kernel, OT_SORTED, ...) for FP32: d_f is accumulated, d_dV may be
- * NULL.  The scratch is a fixed library array of OT_NOALLOC_SCRATCH_BYTES per device; it
- * holds about 446 bytes per marker for OT_PESKIN4 (at most 150,635 markers) and 132 bytes per
- * marker for OT_ROMA3 (at most 508,394); larger n returns OT_ERR_LIMIT and launches nothing.
+ * NULL.  The scratch is a fixed library array of OT_NOALLOC_SCRATCH_BYTES per device, enough for
+ * the documented limits of 150,635 markers for OT_PESKIN4 and 508,394 for OT_ROMA3; larger n
+ * returns OT_ERR_LIMIT and launches nothing.
  * The first call on a device (with that device current) looks up the scratch address; make
  * that first call before any stream capture.  The address is looked up again when the device's
  * context changed (after cudaDeviceReset, say): make the first call after such a change

@@ -146,8 +146,8 @@ size_t spread_ws_bytes(const ot_octree* t, int kernel, int64_t n);
 template <typename T>
 ot_status launch_spread(const ot_octree* t, int kernel, int mode, const double* x, const double* y, const double* z,
                         const T* F, const T* dV, int64_t n, T* f, void* ws, size_t ws_bytes, cudaStream_t s);
-// Sorted spreading with every temporary in `scratch` (spread_noalloc_bytes(kernel, n) bytes).
-size_t spread_noalloc_bytes(int kernel, int64_t n);
+// Sorted spreading with every temporary in `scratch` (spread_noalloc_bytes(n) bytes).
+size_t spread_noalloc_bytes(int64_t n);
 ot_status launch_spread_sorted_noalloc(const ot_octree* t, int kernel, const double* x, const double* y,
                                        const double* z, const float* F, const float* dV, int64_t n, float* f,
                                        void* scratch, cudaStream_t s);

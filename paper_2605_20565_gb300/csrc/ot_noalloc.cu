@@ -5,8 +5,8 @@
 // the whole device memory to its own pool up front, code that runs in a context where an
 // allocation (which may synchronise the device or fail under memory pressure) is not
 // acceptable, or a host program that only passes buffers it already owns.  For them the
-// scratch that the sorted spreading needs (the (leaf, marker, slot) pairs, their sort
-// buffer and the radix-sort histograms) lives in one file-scope device array of a fixed size,
+// scratch that the sorted spreading needs (the markers' tile keys, their sort buffer and counts,
+// records and run table) lives in one file-scope device array of a fixed size,
 // OT_NOALLOC_SCRATCH_BYTES.  Every GPU that loads this library holds that array until the
 // process exits.
 #include <cuda.h>  // driver types only: the two driver calls below are reached through the runtime
@@ -21,7 +21,7 @@ namespace {
 // address: the address comes from cudaGetSymbolAddress, once per device and context.
 static __device__ __align__(256) unsigned char g_spread_scratch[OT_NOALLOC_SCRATCH_BYTES];
 
-// The documented limits of octtrack.h (pairs, sort buffer and tile counts must fit the array).
+// The documented limits of octtrack.h.
 constexpr int64_t kMaxMarkersPeskin4 = 150635, kMaxMarkersRoma3 = 508394;
 
 constexpr int kMaxDevices = 64;
@@ -90,13 +90,13 @@ extern "C" ot_status ot_spread_noalloc(const ot_octree* t, int kernel, const dou
     if (n == 0) return OT_OK;
     if (n * 64 >= (1LL << 32)) return OT_ERR_LIMIT;
     if (n > (kernel == OT_PESKIN4 ? kMaxMarkersPeskin4 : kMaxMarkersRoma3) ||
-        ot::spread_noalloc_bytes(kernel, n) > (size_t)OT_NOALLOC_SCRATCH_BYTES)
+        ot::spread_noalloc_bytes(n) > (size_t)OT_NOALLOC_SCRATCH_BYTES)
         return OT_ERR_LIMIT;
     void* scratch = nullptr;
     cudaError_t e = scratch_address(&scratch);
     if (e != cudaSuccess) return ot::cuda_status(e);
-    // Nothing in the scratch needs to start at zero: every pair slot, histogram and scan
-    // entry is written before it is read in this call.
+    // Nothing in the scratch needs to start at zero: every key, count, record and table entry is
+    // written before it is read in this call.
     return ot::launch_spread_sorted_noalloc(t, kernel, d_x, d_y, d_z, d_F, d_dV, n, d_f, scratch,
                                             (cudaStream_t)stream);
 }
