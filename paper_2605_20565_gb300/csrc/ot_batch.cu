@@ -25,11 +25,11 @@ struct ot_batch {
     unsigned* d_counter = nullptr;
     float* d_pyr = nullptr;    // pyramid of cell means, recomputed at every replay
     int kernels = 1;           // kernels in one replay of the graph
-    // value records of the hot leaves (trilinear launch with the level-mate table): per
-    // level-map cell its entry, per hot leaf its index, per (hot leaf, octant) the 8 level-mate
-    // values, rewritten from the field at every replay
-    uint2* d_ent = nullptr;
-    int* d_hot_leaf = nullptr;
+    // value records of the hot leaves' grid nodes (trilinear launch with the level-mate table): the
+    // cells' entries, the list of the nodes, and per node the 8 values around it, rewritten from
+    // the field at every replay
+    void* d_cells = nullptr;
+    uint2* d_nodes = nullptr;
     float* d_rec = nullptr;
     int64_t n_rec = 0;
 };
@@ -123,46 +123,99 @@ __global__ void __launch_bounds__(256, MINB) k_batch(TreeView t, BatchArgs a, co
 
 
 // ------------------------------------------------------------------------------------------
-// Value records of the hot leaves.  A level-map cell that lies inside one leaf of level at most
-// the hot level (a level whose leaves receive several points per launch) gets the entry
-// (leaf, level << 27 | hot ordinal); every other cell (leaf, ~0).  For every hot leaf and octant
-// of its cell, the record holds the 8 level-mate values of its level-mate row (24 floats, corner
-// order), copied from the field and the cell means at every replay.  A point in such a cell then
-// reads one cell entry and one 96-byte record (three 32-byte loads) instead of the row and 8
-// scattered values; the values and the sum are the same, so the results are bit-identical.
+// Value records of the hot leaves.  A leaf is hot when its level is at most the hot level (a level
+// whose leaves receive several points per launch) and so at most the map level.  The 8
+// level-mates of a point in a leaf of level l are the 8 level-l cells around one node of the
+// level-l grid, the corner of the leaf in the point's octant, and the value a cell takes (its own,
+// the coarser leaf's that covers it, its mean when refined) does not depend on which of the 8 is
+// the host; neither does a cell past a face, which takes the value of the one before it.  So the
+// record -- 24 floats by position, copied from a level-mate row at every replay -- is kept per node
+// at the node's place in the level's (2^l + 1)^3 grid: the hot leaves of 50M uniform points on
+// the many-bubble tree (154k leaves) have 0.2M nodes, 19 MB that stay in L2, where a record per
+// (leaf, octant) took 118 MB that did not.  A point reads its cell's entry (leaf and level), computes
+// the node from its coordinates and reads the 96-byte record (three 32-byte loads); values and
+// sums are those of the level-mate row, so the results are bit-identical.
+// What bounds the launch on random points is the traffic from L2 to the SMs (79% of its sector rate
+// on 64 bubbles; DRAM 45%), so the records' smaller set gains where neighbouring points share
+// lines: 20M particles in Morton order 315 -> 307 us, refreshing the records 78 -> 35 us; 50M in
+// random order 1217 -> 1157 us, the refresh 40 -> 18 us.  Looking cells up first in a coarser
+// table that stays in L1 gained 3% there and lost 5% on the others; loading the next row's
+// positions ahead lost 2 to 10%.
 // ------------------------------------------------------------------------------------------
-constexpr uint32_t REC_NONE = 0xFFFFFFFFu;
+// Packed entry of a cell: level << 28 | leaf, all ones where no hot leaf covers the cell.  Trees of
+// 2^28 leaves or more keep leaf and level in two words.
+template <bool WIDE> struct Cell;
+template <> struct Cell<false> {
+    using type = uint32_t;
+    static __host__ __device__ uint32_t none() { return 0xFFFFFFFFu; }
+    static __device__ uint32_t make(uint32_t leaf, int lv) { return ((uint32_t)lv << 28) | leaf; }
+    static __device__ bool hot(uint32_t e) { return e != 0xFFFFFFFFu; }
+    static __device__ int level(uint32_t e) { return (int)(e >> 28); }
+    static __device__ int leaf(uint32_t e) { return (int)(e & 0xFFFFFFFu); }
+};
+template <> struct Cell<true> {
+    using type = uint2;
+    static __device__ uint2 none() { return make_uint2(0u, 0xFFFFFFFFu); }
+    static __device__ uint2 make(uint32_t leaf, int lv) { return make_uint2(leaf, (uint32_t)lv); }
+    static __device__ bool hot(uint2 e) { return e.y != 0xFFFFFFFFu; }
+    static __device__ int level(uint2 e) { return (int)e.y; }
+    static __device__ int leaf(uint2 e) { return (int)e.x; }
+};
 constexpr int REC_FLOATS = 24;
+constexpr int MAX_HOT = 8;  // map levels are at most 8
 
-__global__ void k_hot_flags(const uint8_t* __restrict__ level, int64_t n, int hot_l, uint32_t* __restrict__ flag) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = level[i] <= hot_l ? 1u : 0u;
+// First node of every level's grid, from the tree's coarsest level on.
+struct NodeGrid {
+    uint32_t off[MAX_HOT + 2];
+};
+NodeGrid node_grid(int lmin, int hot_l) {
+    NodeGrid g{};
+    for (int l = lmin; l <= hot_l; ++l) {
+        const uint32_t s = (1u << l) + 1u;
+        g.off[l + 1] = g.off[l] + s * s * s;
+    }
+    return g;
 }
 
-__global__ void k_hot_list(const uint32_t* __restrict__ flag, const uint32_t* __restrict__ ord, int64_t n,
-                           int* __restrict__ hot_leaf) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) hot_leaf[ord[i]] = (int)i;
-}
-
-__global__ void k_cell_entries(TreeView t, const uint32_t* __restrict__ ord, int hot_l, uint2* __restrict__ ent) {
+// Entries of the level-map cells.
+template <bool WIDE>
+__global__ void k_cells(TreeView t, int hot_l, typename Cell<WIDE>::type* __restrict__ cells) {
+    using C = Cell<WIDE>;
     const int64_t ncell = (int64_t)1 << (3 * t.lmap_level);
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
-        const int a = (int)t.lmap[c];
-        const int e = c + 1 < ncell ? (int)t.lmap[c + 1] : t.n;
-        const int lv = t.level[a];
-        const bool hot = e - a <= 1 && lv <= hot_l;
-        ent[c] = make_uint2((uint32_t)a, hot ? ((uint32_t)lv << 27) | ord[a] : REC_NONE);
+        const uint4 d = t.desc[c];
+        const int lv = (int)((d.z >> 16) & 0xFFu);
+        cells[c] = (d.z & DESC_COVERED) && lv <= hot_l ? C::make(d.w, lv) : C::none();
     }
 }
 
-// One record per (hot leaf, octant), rewritten from the field and the cell means.
-__global__ void __launch_bounds__(256) k_hot_records(TreeView t, const int* __restrict__ hot_leaf, int64_t n_rec,
+// The nodes of the hot leaves, each once (seen: one bit per node): the leaf whose row gives the
+// record, and node | octant << 28 (at most 2^25 nodes).  nodes null: counts them only.
+__global__ void k_hot_nodes(TreeView t, int hot_l, NodeGrid g, uint32_t* __restrict__ seen,
+                            uint2* __restrict__ nodes, uint32_t* __restrict__ count) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < t.n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int l = t.level[i];
+        if (l > hot_l) continue;
+        uint32_t c[3];
+        demorton3(t.key[i] >> (3 * (MAXLEVEL - l)), c[0], c[1], c[2]);
+        const uint32_t s = (1u << l) + 1u;
+        for (uint32_t o = 0; o < 8; ++o) {
+            const uint32_t node = g.off[l] + (c[0] + (o & 1)) + s * ((c[1] + ((o >> 1) & 1)) + s * (c[2] + (o >> 2)));
+            const uint32_t bit = 1u << (node & 31);
+            if (atomicOr(seen + (node >> 5), bit) & bit) continue;
+            const uint32_t at = atomicAdd(count, 1u);
+            if (nodes) nodes[at] = make_uint2((uint32_t)i, node | (o << 28));
+        }
+    }
+}
+
+// One record per listed node, rewritten from the field and the cell means.
+__global__ void __launch_bounds__(256) k_hot_records(TreeView t, const uint2* __restrict__ nodes, int64_t n_rec,
                                                      const float* __restrict__ field, const float* __restrict__ pyr,
                                                      float* __restrict__ rec) {
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rec; r += (int64_t)gridDim.x * blockDim.x) {
-        const int h = hot_leaf[r >> 3];
-        const uint4* row = t.mates + 2 * (8 * (long long)h + (r & 7));
+        const uint2 nd = nodes[r];
+        const uint4* row = t.mates + 2 * (8 * (long long)nd.x + (nd.y >> 28));
         const uint4 r0 = __ldg(row), r1 = __ldg(row + 1);
         const uint32_t sl[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
         float v[REC_FLOATS];
@@ -172,18 +225,13 @@ __global__ void __launch_bounds__(256) k_hot_records(TreeView t, const int* __re
             const float4 f = Vec4<float>::load((sv >> 31) ? pyr : field, (long long)(sv & 0x7FFFFFFFu));
             v[3 * corner] = f.x, v[3 * corner + 1] = f.y, v[3 * corner + 2] = f.z;
         }
-        float4* dst = reinterpret_cast<float4*>(rec + REC_FLOATS * r);
+        float4* dst = reinterpret_cast<float4*>(rec + REC_FLOATS * (size_t)(nd.y & 0xFFFFFFFu));
 #pragma unroll
         for (int k = 0; k < REC_FLOATS / 4; ++k) dst[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
     }
 }
 
-// L2 policies: keep lines resident ahead of others (evict-last), or the default priority.
-__device__ __forceinline__ uint64_t policy_keep() {
-    uint64_t pol;
-    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
+// The default L2 priority, as the hint that a 32-byte load takes.
 __device__ __forceinline__ uint64_t policy_normal() {
     uint64_t pol;
     asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
@@ -197,22 +245,16 @@ __device__ __forceinline__ void ld_nc_v8(const float* p, float* r, uint64_t pol)
         : "l"(p), "l"(pol));
 }
 
-__device__ __forceinline__ uint2 ld_nc_u2(const uint2* p, uint64_t pol) {
-    uint2 e;
-    asm("ld.global.nc.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;" : "=r"(e.x), "=r"(e.y) : "l"(p), "l"(pol));
-    return e;
-}
-
-// The trilinear launch with value records.  Per 32-point row: quantise, read the level-map
-// cell's entry; a point in a hot cell takes its octant's record and is done; the others (cold:
+// The trilinear launch with value records.  Per 32-point row: quantise, read the level of the
+// level-map cell; a point in a hot cell takes its node's record and is done; the others (cold:
 // deeper leaves, uncovered cells) are queued per warp and, whenever 32 are queued (and at the
 // end), interpolated together by the level-mate-table routine with every lane busy.
-template <bool LEARNED>
+template <bool LEARNED, bool WIDE>
 __global__ void __launch_bounds__(256, TRI_MINB) k_tri_rec(TreeView t, BatchArgs a, const float* __restrict__ field,
                                                           const float* __restrict__ pyr,
                                                           unsigned* __restrict__ counter,
-                                                          const uint2* __restrict__ ent,
-                                                          const float* __restrict__ rec) {
+                                                          const typename Cell<WIDE>::type* __restrict__ cells,
+                                                          const float* __restrict__ rec, NodeGrid grid) {
     // per warp of the block: its host task list and its queue of cold points (dynamic shared
     // memory sized by the block's warps: what the block does not use is left to the L1 cache)
     extern __shared__ __align__(16) unsigned char tri_smem[];
@@ -223,6 +265,8 @@ __global__ void __launch_bounds__(256, TRI_MINB) k_tri_rec(TreeView t, BatchArgs
     // is spread[cx] | spread[cy] << 1 | spread[cz] << 2 (map levels are at most 8)
     __shared__ uint32_t s_spread[256];
     for (int v = threadIdx.x; v < 256; v += blockDim.x) s_spread[v] = (uint32_t)part1by2((uint32_t)v);
+    __shared__ uint32_t s_off[MAX_HOT + 2];
+    if (threadIdx.x < MAX_HOT + 2) s_off[threadIdx.x] = grid.off[threadIdx.x];
     const int wid = threadIdx.x >> 5;
     HostQueue& wq = s_queue[wid];
     long long* cq = s_cold[wid];
@@ -231,11 +275,10 @@ __global__ void __launch_bounds__(256, TRI_MINB) k_tri_rec(TreeView t, BatchArgs
     const unsigned lt = (1u << lane) - 1u;
     const int cell_shift = MAXLEVEL - t.lmap_level;  // of the 21-bit coordinates
     const int64_t tile_pts = 32 * (int64_t)a.tile;
-    // the cell entries (16 MB at map level 7) are read by every point: evict-last in L2; the
-    // records (about 100 MB) at the default priority (evict-last on them as well measured 3%
-    // slower on the many-bubble step, evict-first 15% slower); the positions and results
-    // stream through once: evict-first (.cs), so they push out neither
-    const uint64_t keep = policy_keep(), normal = policy_normal();
+    // the positions and results stream through once: evict-first (.cs), so that they push out
+    // neither the cells' entries nor the records
+    const uint64_t normal = policy_normal();
+    using C = Cell<WIDE>;
     int qn = 0;  // queued cold points (warp-uniform)
     // the first cnt queued points, one per lane (warp-wide)
     auto drain = [&](int cnt) {
@@ -270,31 +313,34 @@ __global__ void __launch_bounds__(256, TRI_MINB) k_tri_rec(TreeView t, BatchArgs
                          z = active ? __ldcs(gr.z + i) : 0.0;
             uint64_t X[3];
             const bool ok = active && fixpoint3(x, y, z, X);
-            uint2 e = make_uint2(0u, REC_NONE);
-            if (ok) {
-                const uint32_t c = s_spread[(uint32_t)(X[0] >> 32) >> cell_shift] |
+            typename C::type e = C::none();
+            if (ok)
+                e = __ldg(cells + (s_spread[(uint32_t)(X[0] >> 32) >> cell_shift] |
                                    (s_spread[(uint32_t)(X[1] >> 32) >> cell_shift] << 1) |
-                                   (s_spread[(uint32_t)(X[2] >> 32) >> cell_shift] << 2);
-                e = ld_nc_u2(ent + c, keep);
-            }
-            const bool hot = e.y != REC_NONE;
+                                   (s_spread[(uint32_t)(X[2] >> 32) >> cell_shift] << 2)));
+            const bool hot = C::hot(e);
             if (hot) {
-                float at[3];
-                const int oc = tri_octant<float>(X, (int)(e.y >> 27), at);
-                const float* rp = rec + (8 * (size_t)(e.y & 0x7FFFFFFu) + oc) * REC_FLOATS;
+                const int l = C::level(e);
+                const uint32_t s = (1u << l) + 1u;
+                uint32_t nd[3];  // the node: the cell index rounded up in the upper half
+#pragma unroll
+                for (int d = 0; d < 3; ++d) nd[d] = ((uint32_t)(X[d] >> (52 - l)) + 1u) >> 1;
+                const float* rp = rec + REC_FLOATS * (size_t)(s_off[l] + nd[0] + s * (nd[1] + s * nd[2]));
+                float f[3][2];
+                tri_octant<float>(X, l, f);
                 float vv[REC_FLOATS];
                 ld_nc_v8(rp, vv, normal);
                 ld_nc_v8(rp + 8, vv + 8, normal);
                 ld_nc_v8(rp + 16, vv + 16, normal);
                 float v[8][3];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) v[c][0] = vv[3 * c], v[c][1] = vv[3 * c + 1], v[c][2] = vv[3 * c + 2];
+                for (int k = 0; k < 8; ++k) v[k][0] = vv[3 * k], v[k][1] = vv[3 * k + 1], v[k][2] = vv[3 * k + 2];
                 float o[3];
-                tri_sum<float>(at, v, o);
+                tri_sum<float>(f, v, o);
                 __stcs(gr.u + i, o[0]);
                 __stcs(gr.u + gr.n + i, o[1]);
                 __stcs(gr.u + 2 * gr.n + i, o[2]);
-                if (gr.host) __stcs(gr.host + i, (int)e.x);
+                if (gr.host) __stcs(gr.host + i, C::leaf(e));
             } else if (active && !ok) {  // outside the cube: no host, no value
                 atomicOr(t.err, (unsigned)OT_DEV_OUTSIDE);
                 const float nan = qnan<float>();
@@ -350,51 +396,50 @@ unsigned grid_b(int64_t n) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 8));
 }
 
-// Cell entries, hot-leaf list and record buffer of a batch (synchronises the legacy stream;
-// batch creation is not stream-ordered work).  Leaves b->n_rec = 0 when no leaf is hot or the
-// ordinals would not fit the entry's 27 bits.
-ot_status build_hot_records(const ot_octree* t, int hot_l, ot_batch* b) {
-    const int64_t n = t->n;
-    uint32_t *flag = nullptr, *ord = nullptr, *tot = nullptr;
-    auto cleanup = [&]() {
-        if (flag) cudaFree(flag);
-        if (ord) cudaFree(ord);
-        if (tot) cudaFree(tot);
+bool wide_cells(const ot_octree* t) { return t->n >= (int64_t)1 << 28; }
+
+// Cells' entries, node list and record buffer of a batch (synchronises the legacy stream; batch
+// creation is not stream-ordered work).  Leaves b->n_rec = 0, without an error, when no leaf is hot
+// or the records' grids (up to 1.9 GB at hot level 8) find no memory: the rows serve then.
+ot_status build_hot_records(const ot_octree* t, int hot_l, const NodeGrid& grid, ot_batch* b) {
+    const size_t n_node = grid.off[hot_l + 1], seen_bytes = ((n_node + 31) / 32) * 4;
+    uint32_t* seen = nullptr;  // the bits, then the count
+    auto done = [&](cudaError_t e) {
+        if (seen) cudaFree(seen);
+        return e == cudaSuccess ? OT_OK : cuda_status(e);
     };
     cudaStream_t s = nullptr;
     cudaError_t e;
-    if ((e = cudaMalloc(&flag, sizeof(uint32_t) * n)) != cudaSuccess || (e = cudaMalloc(&ord, sizeof(uint32_t) * n)) != cudaSuccess ||
-        (e = cudaMalloc(&tot, sizeof(uint32_t))) != cudaSuccess) {
-        cleanup();
-        return cuda_status(e);
-    }
-    k_hot_flags<<<grid_b(n), 256, 0, s>>>(t->d_level, n, hot_l, flag);
-    count_launch();
-    ot_status st = scan_u32(flag, ord, n, tot, s);
-    uint32_t n_hot = 0;
-    if (st == OT_OK && (e = cudaMemcpy(&n_hot, tot, sizeof(uint32_t), cudaMemcpyDeviceToHost)) != cudaSuccess)
-        st = cuda_status(e);
-    if (st != OT_OK || n_hot == 0 || n_hot >= (1u << 27)) {
-        cleanup();
-        return st;
-    }
-    const int64_t ncell = (int64_t)1 << (3 * t->lmap_level);
-    if ((e = cudaMalloc(&b->d_hot_leaf, sizeof(int) * (size_t)n_hot)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_ent, sizeof(uint2) * (size_t)ncell)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_rec, sizeof(float) * REC_FLOATS * 8 * (size_t)n_hot)) != cudaSuccess) {
-        cleanup();
-        return cuda_status(e);
-    }
     TreeView v = tree_view(t);
-    k_hot_list<<<grid_b(n), 256, 0, s>>>(flag, ord, n, b->d_hot_leaf);
-    k_cell_entries<<<grid_b(ncell), 256, 0, s>>>(v, ord, hot_l, b->d_ent);
-    count_launch(2);
+    uint32_t count = 0;
+    if ((e = cudaMalloc(&seen, seen_bytes + 4)) != cudaSuccess) return done(e);
+    uint32_t* d_count = seen + seen_bytes / 4;
+    for (int pass = 0; pass < 2; ++pass) {  // count, then list
+        if ((e = cudaMemsetAsync(seen, 0, seen_bytes + 4, s)) != cudaSuccess) return done(e);
+        k_hot_nodes<<<grid_b(t->n), 256, 0, s>>>(v, hot_l, grid, seen, b->d_nodes, d_count);
+        count_launch();
+        if (pass == 1) break;
+        if ((e = cudaMemcpy(&count, d_count, sizeof(count), cudaMemcpyDeviceToHost)) != cudaSuccess) return done(e);
+        if (count == 0) return done(cudaSuccess);
+        if (cudaMalloc(&b->d_rec, sizeof(float) * REC_FLOATS * n_node) != cudaSuccess) {
+            cudaGetLastError();
+            b->d_rec = nullptr;
+            return done(cudaSuccess);
+        }
+        if ((e = cudaMalloc(&b->d_nodes, sizeof(uint2) * (size_t)count)) != cudaSuccess) return done(e);
+    }
+    const bool wide = wide_cells(t);
+    const int64_t ncell = (int64_t)1 << (3 * t->lmap_level);
+    if ((e = cudaMalloc(&b->d_cells, (size_t)ncell * (wide ? 8 : 4))) != cudaSuccess) return done(e);
+    if (wide)
+        k_cells<true><<<grid_b(ncell), 256, 0, s>>>(v, hot_l, static_cast<uint2*>(b->d_cells));
+    else
+        k_cells<false><<<grid_b(ncell), 256, 0, s>>>(v, hot_l, static_cast<uint32_t*>(b->d_cells));
+    count_launch();
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cleanup();
-    if (e != cudaSuccess) return cuda_status(e);
-    b->n_rec = 8 * (int64_t)n_hot;
-    return OT_OK;
+    if (e == cudaSuccess) b->n_rec = count;
+    return done(e);
 }
 
 } // namespace ot
@@ -498,10 +543,11 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
         void* fn;
         BatchArgs args;
         unsigned grid;
-        bool records;  // k_tri_rec: two more arguments
+        bool records;  // k_tri_rec: three more arguments
         size_t dsmem;  // dynamic shared memory per block
     };
     std::vector<Launch> launches;
+    NodeGrid grid{};
     auto add_launch = [&](void* fn, const BatchArgs& args, int cap, size_t dsmem = 0) -> cudaError_t {
         int per_sm = 0;
         cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, dsmem);
@@ -551,15 +597,18 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
             while (hot_l < MAXLEVEL && (n_tri >> (3 * (hot_l + 1))) >= 4) ++hot_l;
             hot_l = std::min(hot_l, t->lmap_level);
             if (tri_records > 0) hot_l = std::min(hot_l, tri_records);
-            if (tri_records >= 0 && t->d_lmap) {
-                ot_status st = build_hot_records(t, hot_l, b);
+            if (tri_records >= 0 && t->d_lmap && hot_l >= t->lmin) {
+                grid = node_grid(t->lmin, hot_l);
+                ot_status st = build_hot_records(t, hot_l, grid, b);
                 if (st != OT_OK) {
                     ot_batch_destroy(b);
                     return st;
                 }
             }
             const bool rec = b->n_rec > 0;
-            void* fn = rec ? (learned ? (void*)k_tri_rec<true> : (void*)k_tri_rec<false>)
+            const bool wide = wide_cells(t);
+            void* fn = rec ? (learned ? (wide ? (void*)k_tri_rec<true, true> : (void*)k_tri_rec<true, false>)
+                                      : (wide ? (void*)k_tri_rec<false, true> : (void*)k_tri_rec<false, false>))
                            : (learned ? (void*)k_batch<true, TRI_MINB, true, K_TRI>
                                       : (void*)k_batch<false, TRI_MINB, true, K_TRI>);
             const size_t dsmem = rec ? (sizeof(HostQueue) + 64 * sizeof(long long)) * (size_t)(block / 32) : 0;
@@ -595,13 +644,13 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
     }
     if (cap_ok && has_tri) cap_ok = launch_pyramid<float>(t, d_field, b->d_pyr, cs) == OT_OK;
     if (cap_ok && b->n_rec > 0) {
-        k_hot_records<<<grid_b(b->n_rec), 256, 0, cs>>>(v, b->d_hot_leaf, b->n_rec, d_field, b->d_pyr, b->d_rec);
+        k_hot_records<<<grid_b(b->n_rec), 256, 0, cs>>>(v, b->d_nodes, b->n_rec, d_field, b->d_pyr, b->d_rec);
         count_launch();
     }
     for (size_t i = 0; cap_ok && i < launches.size(); ++i) {
         unsigned* ctr = b->d_counter + i;
-        void* args[] = {&v, &launches[i].args, (void*)&d_field, (void*)&b->d_pyr, &ctr, (void*)&b->d_ent,
-                        (void*)&b->d_rec};
+        void* args[] = {&v, &launches[i].args, (void*)&d_field, (void*)&b->d_pyr, &ctr, (void*)&b->d_cells,
+                        (void*)&b->d_rec, &grid};
         cap_ok = cudaLaunchKernel(launches[i].fn, dim3(launches[i].grid), dim3(block), args, launches[i].dsmem, cs) ==
                  cudaSuccess;
         count_launch();
@@ -642,8 +691,8 @@ extern "C" ot_status ot_batch_destroy(ot_batch* b) {
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->d_counter) cudaFree(b->d_counter);
     if (b->d_pyr) cudaFree(b->d_pyr);
-    if (b->d_ent) cudaFree(b->d_ent);
-    if (b->d_hot_leaf) cudaFree(b->d_hot_leaf);
+    if (b->d_cells) cudaFree(b->d_cells);
+    if (b->d_nodes) cudaFree(b->d_nodes);
     if (b->d_rec) cudaFree(b->d_rec);
     for (void* p : b->bufs) cudaFree(p);
     delete b;

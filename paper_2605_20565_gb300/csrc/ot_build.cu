@@ -530,37 +530,30 @@ ot_status leaf_centres(const ot_octree* t, double* d_xyz, cudaStream_t s) {
     return OT_OK;
 }
 
-// Descriptor of every level-map cell of level L (see desc_leaf): the refined children and
-// grandchildren of an uncovered cell, valid when no leaf of the cell is deeper than L + 3.
-__global__ void k_desc(const uint64_t* __restrict__ key, const uint8_t* __restrict__ level, int n,
-                       const uint32_t* __restrict__ lmap, int L, int64_t ncell, uint4* __restrict__ desc) {
+// Descriptors of the level-map cells of level L (see desc_resolve): first leaf and, where it covers
+// the cell, its level; then every leaf below a cell that is the first of its child or grandchild
+// adds its bit (a thread per leaf: one per cell would walk up to 8^3 leaves in turn).
+__global__ void k_desc_cells(const uint8_t* __restrict__ level, int n, const uint32_t* __restrict__ lmap, int64_t ncell,
+                             uint4* __restrict__ desc) {
     GRID_STRIDE(c, ncell) {
         const int a = (int)lmap[c];
         const int e = c + 1 < ncell ? (int)lmap[c + 1] : n;
-        uint32_t m1 = 0, valid = 1;
-        uint64_t m2 = 0;
-        if (e - a <= 1) {
-            valid = 0;  // covered: the map answers
-        } else {
-            for (int b = a; b < e; ++b) {
-                const int lb = level[b];
-                if (lb > L + 3) {
-                    valid = 0;
-                    break;
-                }
-                const uint64_t kb = key[b];
-                const int c1 = (int)(kb >> (3 * (MAXLEVEL - L - 1))) & 7;
-                if (lb >= L + 2) m1 |= 1u << c1;
-                if (lb >= L + 3) m2 |= 1ULL << (8 * c1 + ((int)(kb >> (3 * (MAXLEVEL - L - 2))) & 7));
-            }
-        }
-        desc[c] = valid ? make_uint4((uint32_t)m2, (uint32_t)(m2 >> 32), m1 | DESC_VALID, 0u) : make_uint4(0u, 0u, 0u, 0u);
+        // a refined cell holds at least 8 leaves, the first starting at its anchor
+        desc[c] = make_uint4(0u, 0u, e - a <= 1 ? DESC_COVERED | ((uint32_t)level[a] << 16) : 0u, (uint32_t)a);
     }
 }
-
-__global__ void k_lmap_lv(const uint32_t* __restrict__ lmap, const uint8_t* __restrict__ level, int64_t ncell,
-                          uint8_t* __restrict__ out) {
-    GRID_STRIDE(c, ncell) out[c] = level[lmap[c]];
+__global__ void k_desc_leaves(const uint64_t* __restrict__ key, const uint8_t* __restrict__ level, int n, int L,
+                              uint32_t* __restrict__ desc) {
+    GRID_STRIDE(i, (int64_t)n) {
+        const int l = level[i];
+        if (l < L + 2) continue;
+        const uint64_t k = key[i];
+        uint32_t* d = desc + 4 * (size_t)(k >> (3 * (MAXLEVEL - L)));
+        const int c1 = (int)(k >> (3 * (MAXLEVEL - L - 1))) & 7, c2 = (int)(k >> (3 * (MAXLEVEL - L - 2))) & 7;
+        if ((k & (key_span(L + 1) - 1)) == 0) atomicOr(d + 2, 1u << c1);
+        if (l >= L + 3 && (k & (key_span(L + 2) - 1)) == 0) atomicOr(d + (c1 >> 2), 1u << (8 * (c1 & 3) + c2));
+        if (l > L + 3 && (k & (key_span(L + 3) - 1)) == 0) atomicOr(d + 2, DESC_DEEP);
+    }
 }
 
 ot_status finish_tree(ot_octree* t, cudaStream_t s, int map_level) {
@@ -588,19 +581,15 @@ ot_status finish_tree(ot_octree* t, cudaStream_t s, int map_level) {
         count_launch();
     }
     t->lmap_level = L;
-    if (t->d_lmap_lv) cudaFree(t->d_lmap_lv);
-    {
-        const int64_t ncell = (int64_t)1 << (3 * L);
-        OT_CUDA(cudaMalloc(&t->d_lmap_lv, ncell));
-        k_lmap_lv<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_lmap, t->d_level, ncell, t->d_lmap_lv);
-        count_launch();
-    }
     if (t->d_desc) cudaFree(t->d_desc);
     t->d_desc = nullptr;
-    if (L + 1 <= t->lmax && L + 1 < MAXLEVEL) {
-        const int64_t ncell = (int64_t)1 << (3 * L);
-        OT_CUDA(cudaMalloc(&t->d_desc, sizeof(uint4) * ncell));
-        k_desc<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_key, t->d_level, (int)t->n, t->d_lmap, L, ncell, t->d_desc);
+    const int64_t ncell = (int64_t)1 << (3 * L);
+    OT_CUDA(cudaMalloc(&t->d_desc, sizeof(uint4) * ncell));
+    k_desc_cells<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_level, (int)t->n, t->d_lmap, ncell, t->d_desc);
+    count_launch();
+    if (L + 2 <= t->lmax) {
+        k_desc_leaves<<<grid1d(t->n, 256), 256, 0, s>>>(t->d_key, t->d_level, (int)t->n, L,
+                                                       reinterpret_cast<uint32_t*>(t->d_desc));
         count_launch();
     }
     if (!t->d_err) {
@@ -623,7 +612,6 @@ TreeView tree_view(const ot_octree* t) {
     v.lmap = t->d_lmap;
     v.lmap_level = t->lmap_level;
     v.desc = t->d_desc;
-    v.lmap_lv = t->d_lmap_lv;
     v.pyr_level = t->pyr_level;
     v.periodic = t->periodic;
     v.mates = reinterpret_cast<const uint4*>(t->d_mates);

@@ -1,8 +1,8 @@
 // ot_mates.cu -- the level-mate table: the trilinear level-mate rule (Sec. 2.3.2 reading:
 // host cell c of level l, level-mates c + {0, s_d}) resolved once per octree instead of at
 // every query.  For leaf h and octant o of its cell (bit d of o: the upper half on axis d, so
-// s_d = +1), row 8h + o holds the 8 value slots of the level-mates in corner order (bit d of
-// the corner: the neighbour on axis d), 32 bytes:
+// s_d = +1), row 8h + o holds the 8 value slots of the level-mates by position (bit d of the
+// corner: the upper of the two cells on axis d), 32 bytes:
 //   slot < 2^31: a leaf index -- a leaf of level l, or the coarser leaf covering the level-mate;
 //   slot >= 2^31: (slot - 2^31) indexes the array of cell means of a refined level-mate (the
 //   dense pyramid for l <= pyr_level, else the node means of level l by first leaf).
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256, 4) k_mates(TreeView t, uint2* __restrict_
         int sidx = 0, p3 = 1;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const int dd = ((corner >> d) & 1) ? (((o >> d) & 1) ? 1 : -1) : 0;
+            const int dd = ((corner >> d) & 1) + ((o >> d) & 1) - 1;  // the host is the lower cell for octant bit 1
             sidx += (dd + 1) * p3;
             p3 *= 3;
         }
@@ -61,7 +61,6 @@ __global__ void __launch_bounds__(256, 4) k_mates(TreeView t, uint2* __restrict_
     const int sx = lane % 3, sy = 3 + (lane / 3) % 3, sz = 6 + (lane / 9) % 3;
     const bool is_mate = lane < 27 && lane != 13;
     const int Lsh = 3 * (MAXLEVEL - t.lmap_level);
-    const uint32_t nmap = 1u << (3 * t.lmap_level);
     // keys and levels of the warp's leaves, one lane each (then broadcast), loaded one
     // iteration ahead
     uint64_t kl = 0;
@@ -79,7 +78,7 @@ __global__ void __launch_bounds__(256, 4) k_mates(TreeView t, uint2* __restrict_
             ll_next = t.level[nxt];
         }
         // every leaf's level-map lookups issued before any is resolved (one round of loads)
-        int lv[MATES_U], a[MATES_U], e[MATES_U], la[MATES_U];
+        int lv[MATES_U];
         uint64_t q[MATES_U];
         uint4 dsc[MATES_U];
         bool nb[MATES_U];
@@ -102,11 +101,7 @@ __global__ void __launch_bounds__(256, 4) k_mates(TreeView t, uint2* __restrict_
             const uint64_t dz = __shfl_sync(0xffffffffu, dil, sz);
             nb[u] = is_mate && base + u < t.n && !(dx & dy & dz & SAME);
             q[u] = ((dx | dy | dz) & ~SAME) << sh3;  // the level-mate cell's anchor key
-            const uint32_t c = nb[u] ? (uint32_t)(q[u] >> Lsh) : 0u;
-            a[u] = (int)t.lmap[c];
-            e[u] = c + 1 < nmap ? (int)t.lmap[c + 1] : t.n;
-            la[u] = t.lmap_lv[c];
-            dsc[u] = t.desc ? __ldg(t.desc + c) : make_uint4(0u, 0u, 0u, 0u);
+            dsc[u] = __ldg(t.desc + (nb[u] ? (uint32_t)(q[u] >> Lsh) : 0u));
         }
         const int Lp = t.pyr_level;
 #pragma unroll
@@ -114,14 +109,10 @@ __global__ void __launch_bounds__(256, 4) k_mates(TreeView t, uint2* __restrict_
             uint32_t slot = (uint32_t)(base + u);
             if (nb[u]) {
                 const int l = lv[u];
-                int leaf = a[u], lvl = la[u];
-                if (e[u] - a[u] > 1) {
-                    if (dsc[u].z & DESC_VALID) {
-                        leaf = desc_leaf(dsc[u], t.lmap_level, q[u], a[u], lvl);
-                    } else {
-                        leaf = search_range(t.key, a[u], e[u] - a[u], q[u]);
-                        lvl = t.level[leaf];
-                    }
+                int leaf, lvl;
+                if (!desc_resolve(dsc[u], t.lmap_level, q[u], leaf, lvl)) {
+                    leaf = search_range(t.key, leaf, map_end(t, map_cell(t, q[u])) - leaf, q[u]);
+                    lvl = t.level[leaf];
                 }
                 if (lvl <= l) {
                     slot = (uint32_t)leaf;
@@ -173,8 +164,7 @@ __global__ void __launch_bounds__(256) k_pnbr(TreeView t, int64_t nslots, int* _
             }
             if (inside) {
                 const uint64_t anchor = morton3((uint32_t)q[0], (uint32_t)q[1], (uint32_t)q[2]) << (3 * sh);
-                const int f = search_plain(t, anchor);
-                if ((int)t.level[f] == t.lmax && ldg_key(t.key + f) == anchor) v = f;
+                v = find_block<false>(t, anchor);
             }
         }
         out[32 * sl + lane] = v;

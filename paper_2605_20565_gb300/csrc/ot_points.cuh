@@ -46,8 +46,7 @@ __device__ __forceinline__ T stencil_weight_1d(int lmax, uint64_t X, int a) {
 // Parent blocks (2x2x2 cells of level lmax, i.e. cells of level lmax-1) overlapping the
 // delta-kernel stencil whose first cell is i0.  With the parent-block table, the middle block's
 // row gives every block's first child; otherwise one search per block finds it.  A parent
-// whose first child is a leaf of level lmax has all 8 children as consecutive leaves.  A parent in the same grandparent as the last one found is usually 8
-// leaves per child-number step away, which one key comparison proves.  The visitor gets
+// whose first child is a leaf of level lmax has all 8 children as consecutive leaves.  The visitor gets
 // (a0, bx, by, bz, P) with a0 the first child's index, or -1 when the parent is outside the
 // cube (a periodic cube wraps it instead) or not refined to the finest level.
 template <int K, bool LEARNED, typename PVisit>
@@ -76,8 +75,7 @@ __device__ __forceinline__ void visit_parents(const TreeView& t, const int i0[3]
         int am = -1;
         if (inside) {
             const uint64_t anchor = morton3((uint32_t)qm[0] << shp, (uint32_t)qm[1] << shp, (uint32_t)qm[2] << shp);
-            const int a = search<LEARNED>(t, anchor);
-            if (ldg_key(t.key + a) == anchor && t.level[a] == t.lmax) am = a;
+            am = find_block<LEARNED>(t, anchor);
         }
         if (am >= 0) {  // else (the middle block is not refined to the finest level) the walk below
             const int* __restrict__ row = t.pnbr + 32 * (size_t)(am >> 3);
@@ -91,7 +89,6 @@ __device__ __forceinline__ void visit_parents(const TreeView& t, const int i0[3]
             return;
         }
     }
-    int prevP[3] = {-1, -1, -1}, prev_a0 = -1;
     for (int bz = 0; bz < pn[2]; ++bz)
         for (int by = 0; by < pn[1]; ++by)
             for (int bx = 0; bx < pn[0]; ++bx) {
@@ -105,23 +102,9 @@ __device__ __forceinline__ void visit_parents(const TreeView& t, const int i0[3]
                 const bool inside = Q[0] >= 0 && Q[1] >= 0 && Q[2] >= 0 && Q[0] < np_cells && Q[1] < np_cells &&
                                     Q[2] < np_cells;
                 int a0 = -1;
-                if (inside) {
-                    const uint64_t anchor =
-                        morton3((uint32_t)Q[0] << shp, (uint32_t)Q[1] << shp, (uint32_t)Q[2] << shp);
-                    int a = -1;
-                    if (prev_a0 >= 0 && (Q[0] >> 1) == (prevP[0] >> 1) && (Q[1] >> 1) == (prevP[1] >> 1) &&
-                        (Q[2] >> 1) == (prevP[2] >> 1)) {
-                        const int g = prev_a0 + 8 * (((Q[0] & 1) | ((Q[1] & 1) << 1) | ((Q[2] & 1) << 2)) -
-                                                     ((prevP[0] & 1) | ((prevP[1] & 1) << 1) | ((prevP[2] & 1) << 2)));
-                        if (g >= 0 && g < t.n && ldg_key(t.key + g) == anchor) a = g;
-                    }
-                    if (a < 0) a = search<LEARNED>(t, anchor);
-                    if (ldg_key(t.key + a) == anchor && t.level[a] == t.lmax) {
-                        a0 = a;
-                        prevP[0] = Q[0], prevP[1] = Q[1], prevP[2] = Q[2];
-                        prev_a0 = a;
-                    }
-                }
+                if (inside)
+                    a0 = find_block<LEARNED>(
+                        t, morton3((uint32_t)Q[0] << shp, (uint32_t)Q[1] << shp, (uint32_t)Q[2] << shp));
                 pvisit(a0, bx, by, bz, P);
             }
 }

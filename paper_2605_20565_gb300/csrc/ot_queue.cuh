@@ -1,9 +1,10 @@
 // ot_queue.cuh -- warp-cooperative host-cell search over a per-warp task list, and the
 // trilinear interpolation (Sec. 2.3.2, level-mate rule) built on it.
 //
-// A point needs up to 8 searches (its host, then the level-mates that are not siblings of the
-// host) and each search takes 0 to ~12 dependent key probes, so a warp that gives each lane its
-// own searches idles most lanes: every corner costs the longest lane's search.  Here the lanes
+// A point needs up to 8 searches (its host, then its level-mates).  Most are answered by the
+// descriptor of the key's level-map cell, one load.  Those in deeper subtrees, and the learned
+// search, take up to ~12 dependent key probes, so a warp that gave each lane its own would
+// idle most lanes: every corner would cost the longest lane's search.  There the lanes
 // first append every search they need to a task list in shared memory (ballot + popc, no
 // atomics); then each lane takes the next task whenever its current one ends and performs one
 // probe per step.  The warp's step count follows the total number of probes / 32 instead of the
@@ -27,7 +28,6 @@ struct WarpQueueN {
     uint64_t q[CAP];
     int lo[CAP];
     int len[CAP];
-    signed char lv[CAP];  // the answer leaf's level when the search learned it, else -1
 };
 using WarpQueue = WarpQueueN<QCAP>;
 using HostQueue = WarpQueueN<32>;
@@ -44,17 +44,21 @@ __device__ __forceinline__ void stage_root(const TreeView& t, RootModel& s_root)
     __syncthreads();
 }
 
-// Level-map lookup of key q: the leaf holding its cell's anchor (a) and the next cell's (e).
-// The cell is covered by one leaf -- leaf a, the answer -- exactly when e - a <= 1 (a refined
-// cell holds at least 8 leaves, its first one starting at its anchor).  Returns true with the
-// answer in a when covered, else false with the cell's leaf range [a, e) to search.
-// lv: the level of leaf a (from the per-cell level table, in the same round trip).
+// Level-map lookup of key q by its cell's descriptor: true with the leaf (a) and its level (lv) when
+// the cell is covered by one leaf or, for the plain search, its subtree is at most 3 levels
+// deep; else false with the cell's leaf range [a, e) to search.
+template <bool LEARNED>
 __device__ __forceinline__ bool map_lookup(const TreeView& t, uint64_t q, int& a, int& e, int& lv) {
-    const uint32_t cell = (uint32_t)(q >> (3 * (MAXLEVEL - t.lmap_level)));
-    a = (int)t.lmap[cell];
-    e = cell < (1u << (3 * t.lmap_level)) - 1u ? (int)t.lmap[cell + 1] : t.n;
-    lv = t.lmap_lv[cell];
-    return e - a <= 1;
+    const uint32_t cell = map_cell(t, q);
+    const uint4 d = __ldg(t.desc + cell);
+    if (LEARNED ? (d.z & DESC_COVERED) != 0 : !(d.z & DESC_DEEP) || (d.z & DESC_COVERED)) {
+        desc_resolve(d, t.lmap_level, q, a, lv);
+        return true;
+    }
+    a = (int)d.w;
+    e = map_end(t, cell);
+    lv = -1;
+    return false;
 }
 
 // Appends a task for every lane with need set (warp-wide call); returns the lane's task index
@@ -75,31 +79,26 @@ __device__ __forceinline__ int push_task(Q& w, int& n, bool need, uint64_t q, in
 // Runs the warp's ntask tasks (warp-wide call).  Each step, a lane without a task takes the
 // next one, and every lane with a task advances it by one step of at most one memory round
 // trip:
-//   plain:   the cell's subtree descriptor, which answers directly when the subtree is at most
-//            3 levels deep; else halving probes over the cell's leaves;
+//   plain:   halving probes over the cell's leaves;
 //   learned: route (root model from shared memory, then the middle model's load), leaf model
 //            load and window (its prediction widened by the stored error bounds, clamped to
 //            the cell), halving probes over the window, and the check key[a] <= q < key[a+1];
 //            a window that missed is replaced by the whole cell (a counted fallback).
-// A finished task's answer (the last index in its range whose key is <= q) replaces its lo;
-// its level goes to lv when the descriptor gave it (-1 otherwise).
+// A finished task's answer (the last index in its range whose key is <= q) replaces its lo.
 // (Routing all tasks side by side before the loop was measured slower: it adds a round trip
 // and registers.)
-enum { ST_ROUTE = 0, ST_MODEL = 1, ST_PROBE = 2, ST_CHECK = 3, ST_DONE = 4, ST_DESC = 5 };
+enum { ST_ROUTE = 0, ST_MODEL = 1, ST_PROBE = 2, ST_CHECK = 3, ST_DONE = 4 };
 
 template <bool LEARNED, typename Q>
 __device__ __forceinline__ void run_tasks(const TreeView& t, const RootModel& root, Q& w, int ntask,
                                           unsigned lt) {
     __syncwarp();
-    int cur = -1, lo = 0, len = 0, next = 0, st = ST_DONE, clo = 0, clen = 0, j = 0, lvr = -1;
+    int cur = -1, lo = 0, len = 0, next = 0, st = ST_DONE, clo = 0, clen = 0, j = 0;
     bool checked = false;
     uint64_t q = 0;
     for (;;) {
         const bool fin = cur >= 0 && st == ST_DONE;
-        if (fin) {
-            w.lo[cur] = lo;
-            w.lv[cur] = (signed char)lvr;
-        }
+        if (fin) w.lo[cur] = lo;
         const bool need = cur < 0 || fin;
         const unsigned m = __ballot_sync(FULL, need);
         if (need) {
@@ -110,23 +109,14 @@ __device__ __forceinline__ void run_tasks(const TreeView& t, const RootModel& ro
                 q = w.q[idx];
                 lo = clo = w.lo[idx];
                 len = clen = w.len[idx];
-                st = LEARNED ? ST_ROUTE : (t.desc ? ST_DESC : ST_PROBE);
+                st = LEARNED ? ST_ROUTE : ST_PROBE;
                 checked = false;
-                lvr = -1;
             }
         }
         next += __popc(m);
         if (!__any_sync(FULL, cur >= 0)) break;
         if (cur < 0) continue;
-        if (!LEARNED && st == ST_DESC) {
-            const uint4 d = __ldg(t.desc + (q >> (3 * (MAXLEVEL - t.lmap_level))));
-            if (d.z & DESC_VALID) {
-                lo = desc_leaf(d, t.lmap_level, q, lo, lvr);
-                st = ST_DONE;
-            } else {
-                st = ST_PROBE;
-            }
-        } else if (LEARNED && st == ST_ROUTE) {
+        if (LEARNED && st == ST_ROUTE) {
             j = root_route(root, q);
             if (t.mids) j = (int)(((int64_t)leaf_predict(t.mids[j], q, t.n) * t.n_leaf) / t.n);
             st = ST_MODEL;
@@ -174,23 +164,62 @@ __device__ __forceinline__ void run_tasks(const TreeView& t, const RootModel& ro
 
 // Host leaf of the point with fixed-point coordinates X, for the lanes with ok set and no host
 // given (h < 0) (warp-wide call): the level-map lookup, then the warp's task list for the lanes
-// whose cell is not covered.  hl receives the leaf's level when the lookup or the descriptor
-// gave it, else stays -1.
+// that it does not answer.  hl receives the leaf's level when the lookup gave it, else stays -1.
 template <bool LEARNED, typename Q>
 __device__ __forceinline__ void host_queued(const TreeView& t, const RootModel& root, Q& w, bool ok,
                                             const uint64_t X[3], int& h, int& hl) {
     const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
     const uint64_t q = morton3((uint32_t)(X[0] >> 32), (uint32_t)(X[1] >> 32), (uint32_t)(X[2] >> 32));
     int ca = 0, ce = 0, clv = -1;
-    const bool need = ok && h < 0 && !map_lookup(t, q, ca, ce, clv);
+    const bool need = ok && h < 0 && !map_lookup<LEARNED>(t, q, ca, ce, clv);
     if (ok && h < 0 && !need) h = ca, hl = clv;
     if (__any_sync(FULL, need)) {
         int n = 0;
         const int ix = push_task(w, n, need, q, ca, ce - ca, lt);
         run_tasks<LEARNED>(t, root, w, n, lt);
-        if (ix >= 0) h = w.lo[ix], hl = w.lv[ix];
+        if (ix >= 0) h = w.lo[ix], hl = -1;
         __syncwarp();
     }
+}
+
+// Octant of the point with fixed-point coordinates X in its host leaf of level l (bit d: the
+// upper half on axis d, where the host is the lower of the two level-mates) and per axis the
+// weights of the lower and the upper level-mate (Sec. 2.3.2), 1 - |t_d| for the host's and
+// |t_d| for the neighbour's, t_d the offset from the host's centre in cell units.
+template <typename T>
+__device__ __forceinline__ int tri_octant(const uint64_t X[3], int l, T f[3][2]) {
+    int o = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const bool up = fix_upper_half(X[d], l);
+        o |= (up ? 1 : 0) << d;
+        const T td = fix_offset<T>(X[d], l);
+        const T at = td < T(0) ? -td : td;
+        f[d][0] = up ? T(1) - at : at;
+        f[d][1] = up ? at : T(1) - at;
+    }
+    return o;
+}
+
+// The trilinear sum over the 8 level-mate values v by position (bit d of the corner: the upper
+// cell on axis d), accumulated in that order, whichever of the 8 is the host: points around one
+// grid node share its 8 values in one order.  Every form of the trilinear interpolation sums so,
+// so their results are bit-identical.
+template <typename T>
+__device__ __forceinline__ void tri_sum(const T f[3][2], const T v[8][3], T out[3]) {
+    // corner weight (f_0 f_1) f_2: the four x-y products once
+    const T wxy[4] = {f[0][0] * f[1][0], f[0][1] * f[1][0], f[0][0] * f[1][1], f[0][1] * f[1][1]};
+    T acc0 = T(0), acc1 = T(0), acc2 = T(0);
+#pragma unroll
+    for (int corner = 0; corner < 8; ++corner) {
+        const T wc = wxy[corner & 3] * f[2][corner >> 2];
+        acc0 += wc * v[corner][0];
+        acc1 += wc * v[corner][1];
+        acc2 += wc * v[corner][2];
+    }
+    out[0] = acc0;
+    out[1] = acc1;
+    out[2] = acc2;
 }
 
 // Trilinear interpolation at one point per lane (warp-wide call; Sec. 2.3.2 with the
@@ -220,113 +249,84 @@ __device__ __forceinline__ int trilinear_queued(const TreeView& t, const RootMod
 
     const int l = hl >= 0 ? hl : (int)t.level[h];
     const int ncell = 1 << l;
-    int c[3], sg[3];
-    T at[3];
+    int c[3];
+    T f[3][2];
+    const int oct = tri_octant<T>(X, l, f);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        c[d] = (int)fix_cell(X[d], l);
-        sg[d] = fix_upper_half(X[d], l) ? 1 : -1;
-        const T td = fix_offset<T>(X[d], l);
-        at[d] = td < T(0) ? -td : td;
-    }
+    for (int d = 0; d < 3; ++d) c[d] = (int)fix_cell(X[d], l);
     const int sh = MAXLEVEL - l;
     // The level-mates are resolved in stages, each issuing its loads for all 8 corners at once
     // (independent loads in flight together instead of one dependent chain per corner).
-    // Stage 1: anchors, weights, and the sibling guess h + (difference of child numbers) for
-    // level-mates in the host's parent cell.
+    // Stage 1: anchors and weights.
     uint64_t anc[8];
     T wt[8];
-    int a[8], gi[8];
-    unsigned self_m = 1u, sib_m = 0u;
-    // per axis the level-mate index (the host's, or the neighbour's clamped into the cube) and
-    // its Morton bits: each corner's anchor is the OR of three of these six
-    int nb[3];
+    int a[8];
+    unsigned self_m = 0u;
+    // per axis the lower and the upper level-mate index (the host's, and the neighbour's clamped
+    // into the cube) and their Morton bits: each corner's anchor is the OR of three of these six
+    int ix[3][2];
     uint64_t dil[3][2];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        nb[d] = c[d] + sg[d];
-        if (nb[d] < 0 || nb[d] >= ncell) nb[d] = t.periodic ? (nb[d] + ncell) & (ncell - 1) : c[d];
-        dil[d][0] = (part1by2((uint32_t)c[d]) << d) << (3 * sh);
-        dil[d][1] = (part1by2((uint32_t)nb[d]) << d) << (3 * sh);
+        const bool up = (oct >> d) & 1;  // the neighbour is the upper one
+        int nb = c[d] + (up ? 1 : -1);
+        if (nb < 0 || nb >= ncell) nb = t.periodic ? (nb + ncell) & (ncell - 1) : c[d];
+        ix[d][0] = up ? c[d] : nb;
+        ix[d][1] = up ? nb : c[d];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) dil[d][k] = (part1by2((uint32_t)ix[d][k]) << d) << (3 * sh);
     }
 #pragma unroll
     for (int corner = 0; corner < 8; ++corner) {
-        int m[3];
         T wc = T(1);
-        bool self = true, sib = true;
+        bool self = true;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const int off = (corner >> d) & 1;
-            const int v = off ? nb[d] : c[d];
-            m[d] = v;
+            const int v = ix[d][(corner >> d) & 1];
             self = self && (v == c[d]);
-            sib = sib && ((v >> 1) == (c[d] >> 1));
-            wc *= off ? at[d] : T(1) - at[d];
+            wc *= f[d][(corner >> d) & 1];
         }
         wt[corner] = wc;
         anc[corner] = dil[0][corner & 1] | dil[1][(corner >> 1) & 1] | dil[2][(corner >> 2) & 1];
         a[corner] = h;
-        gi[corner] = min(max(h + ((m[0] & 1) | ((m[1] & 1) << 1) | ((m[2] & 1) << 2)) -
-                                 ((c[0] & 1) | ((c[1] & 1) << 1) | ((c[2] & 1) << 2)),
-                             0),
-                         t.n - 1);
         if (self) self_m |= 1u << corner;
-        if (sib && !self) sib_m |= 1u << corner;
     }
-    if (!ok) self_m = 0xffu, sib_m = 0u;
-    // Stage 2: the guessed siblings' keys (a match proves the guess: keys are unique) and, in
-    // the same round of loads, the level-map lookups of the other level-mates (a covered cell
-    // settles its level-mate).  Stage 3: a failed guess's lookup.  Stage 4: the rest become
-    // tasks of the warp's list.
-    unsigned pend_m = ~self_m & 0xffu;
+    if (!ok) self_m = 0xffu;
+    // Stage 2: the level-map lookups of the other corners, each one descriptor load and most with the
+    // answer and its level; stage 3: the rest become tasks of the warp's list.
+    int lvl[8];
+    unsigned pend_m = 0u;
     int ca[8], ce[8];
-    {
-        uint64_t gk[8];
-        int unused_lv;
 #pragma unroll
-        for (int corner = 1; corner < 8; ++corner) {
-            ca[corner] = 0;
-            ce[corner] = 0;
-            gk[corner] = 0;
-            if ((sib_m >> corner) & 1u) {
-                gk[corner] = ldg_key(t.key + gi[corner]);
-            } else if ((pend_m >> corner) & 1u) {
-                if (map_lookup(t, anc[corner], ca[corner], ce[corner], unused_lv)) {
-                    a[corner] = ca[corner];
-                    pend_m &= ~(1u << corner);
-                }
-            }
-        }
-#pragma unroll
-        for (int corner = 1; corner < 8; ++corner) {
-            if (!((sib_m >> corner) & 1u)) continue;
-            if (gk[corner] == anc[corner] || map_lookup(t, anc[corner], ca[corner], ce[corner], unused_lv)) {
-                a[corner] = gk[corner] == anc[corner] ? gi[corner] : ca[corner];
-                pend_m &= ~(1u << corner);
-            }
-        }
+    for (int corner = 0; corner < 8; ++corner) {
+        ca[corner] = ce[corner] = 0;
+        lvl[corner] = l;
+        if ((self_m >> corner) & 1u) continue;
+        if (map_lookup<false>(t, anc[corner], ca[corner], ce[corner], lvl[corner]))
+            a[corner] = ca[corner];
+        else
+            pend_m |= 1u << corner;
     }
     if (__any_sync(FULL, pend_m != 0u)) {
         int n = 0;
         int tix[8];
 #pragma unroll
-        for (int corner = 1; corner < 8; ++corner)
+        for (int corner = 0; corner < 8; ++corner)
             tix[corner] = push_task(w, n, (pend_m >> corner) & 1u, anc[corner], ca[corner], ce[corner] - ca[corner], lt);
         run_tasks<LEARNED>(t, root, w, n, lt);
 #pragma unroll
-        for (int corner = 1; corner < 8; ++corner)
-            if (tix[corner] >= 0) a[corner] = w.lo[tix[corner]];
+        for (int corner = 0; corner < 8; ++corner)
+            if (tix[corner] >= 0) {
+                a[corner] = w.lo[tix[corner]];
+                lvl[corner] = (int)t.level[a[corner]];
+            }
         __syncwarp();
     }
     if (!ok) {
         out[0] = out[1] = out[2] = qnan<T>();
         return -1;
     }
-    // Stage 6: the levels of the level-mates' leaves (carrying them along from the lookups was
-    // measured slower: registers); stage 7: the values.
-    int lvl[8];
-#pragma unroll
-    for (int corner = 0; corner < 8; ++corner) lvl[corner] = ((self_m >> corner) & 1u) ? l : (int)t.level[a[corner]];
+    // Stage 4: the values.
     // a refined level-mate: the pyramid cell (l <= pyramid level) or the node mean of level l
     // indexed by its first leaf
     const bool in_pyr = l <= t.pyr_level;
@@ -337,8 +337,8 @@ __device__ __forceinline__ int trilinear_queued(const TreeView& t, const RootMod
     for (int corner = 0; corner < 8; ++corner) {
         const bool refined = lvl[corner] > l;
         const long long ri = in_pyr ? (long long)(anc[corner] >> (3 * sh)) : (long long)a[corner];
-        const auto f = V::load(refined ? rbase : field, refined ? ri : (long long)a[corner]);
-        v[corner][0] = f.x, v[corner][1] = f.y, v[corner][2] = f.z;
+        const auto fv = V::load(refined ? rbase : field, refined ? ri : (long long)a[corner]);
+        v[corner][0] = fv.x, v[corner][1] = fv.y, v[corner][2] = fv.z;
     }
     T acc0 = T(0), acc1 = T(0), acc2 = T(0);
 #pragma unroll
@@ -351,42 +351,6 @@ __device__ __forceinline__ int trilinear_queued(const TreeView& t, const RootMod
     out[1] = acc1;
     out[2] = acc2;
     return h;
-}
-
-// Octant of the point with fixed-point coordinates X in its host leaf of level l (bit d: the
-// upper half on axis d) and the distances |t_d| of the point from the leaf's centre in cell
-// units (Sec. 2.3.2 trilinear weights).
-template <typename T>
-__device__ __forceinline__ int tri_octant(const uint64_t X[3], int l, T at[3]) {
-    int o = 0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        o |= (fix_upper_half(X[d], l) ? 1 : 0) << d;
-        const T td = fix_offset<T>(X[d], l);
-        at[d] = td < T(0) ? -td : td;
-    }
-    return o;
-}
-
-// The trilinear sum over the 8 level-mate values v (corner order: bit d of the corner set for
-// the neighbour on axis d), weights prod (1 - |t_d|) or |t_d|, accumulated in corner order.
-// Every form of the trilinear interpolation ends here, so their results are bit-identical.
-template <typename T>
-__device__ __forceinline__ void tri_sum(const T at[3], const T v[8][3], T out[3]) {
-    // corner weight (f_0 f_1) f_2 with f_d = |t_d| or 1 - |t_d|: the four x-y products once
-    const T b0 = T(1) - at[0], b1 = T(1) - at[1], b2 = T(1) - at[2];
-    const T wxy[4] = {b0 * b1, at[0] * b1, b0 * at[1], at[0] * at[1]};
-    T acc0 = T(0), acc1 = T(0), acc2 = T(0);
-#pragma unroll
-    for (int corner = 0; corner < 8; ++corner) {
-        const T wc = wxy[corner & 3] * ((corner & 4) ? at[2] : b2);
-        acc0 += wc * v[corner][0];
-        acc1 += wc * v[corner][1];
-        acc2 += wc * v[corner][2];
-    }
-    out[0] = acc0;
-    out[1] = acc1;
-    out[2] = acc2;
 }
 
 // The same interpolation with the level-mates read from the octree's level-mate table (built
@@ -409,8 +373,8 @@ __device__ __forceinline__ int trilinear_mates(const TreeView& t, const RootMode
         return -1;
     }
     const int l = hl >= 0 ? hl : (int)t.level[h];
-    T at[3];
-    const int o = tri_octant<T>(X, l, at);
+    T w8[3][2];
+    const int o = tri_octant<T>(X, l, w8);
     const uint4* row = t.mates + 2 * (8 * (long long)h + o);
     const uint4 r0 = __ldg(row), r1 = __ldg(row + 1);
     const uint32_t sl[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
@@ -421,7 +385,7 @@ __device__ __forceinline__ int trilinear_mates(const TreeView& t, const RootMode
         const auto f = V::load((sv >> 31) ? pyr : field, (long long)(sv & 0x7FFFFFFFu));
         v[corner][0] = f.x, v[corner][1] = f.y, v[corner][2] = f.z;
     }
-    tri_sum<T>(at, v, out);
+    tri_sum<T>(w8, v, out);
     return h;
 }
 

@@ -483,14 +483,9 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
             const uint32_t total = __shfl_sync(FULLM, incl, 7);
             const uint32_t first = st - (incl - (en - st));  // record of list place p: first + p
             // the tile's 8 blocks of 8 finest leaves: first leaf, -1 when not refined to the finest
-            int a0 = -1;
-            {
-                const uint64_t anchor = morton3((uint32_t)(2 * tc[0] + (s & 1)) << shb,
-                                                (uint32_t)(2 * tc[1] + ((s >> 1) & 1)) << shb,
-                                                (uint32_t)(2 * tc[2] + (s >> 2)) << shb);
-                const int a = search_plain(t, anchor);
-                if (ldg_key(t.key + a) == anchor && (int)t.level[a] == t.lmax) a0 = a;
-            }
+            const int a0 = find_block<false>(t, morton3((uint32_t)(2 * tc[0] + (s & 1)) << shb,
+                                                        (uint32_t)(2 * tc[1] + ((s >> 1) & 1)) << shb,
+                                                        (uint32_t)(2 * tc[2] + (s >> 2)) << shb));
             const unsigned valid = __ballot_sync(FULLM, a0 >= 0) & 0xffu;
             const int mine0 = __shfl_sync(FULLM, a0, (cx >> 1) | ((cy >> 1) << 1) | (zh << 2));
             const int leaf = mine0 + ((cx & 1) | ((cy & 1) << 1));  // and leaf + 4 above it
