@@ -52,7 +52,7 @@ struct BatchArgs {
     GroupDev g[MAX_GROUPS];
     int ng;
     int64_t ntiles;
-    int tile; // points per lane per tile
+    int pts;  // points per tile
 };
 
 // MINB: the register budget (blocks of 256 resident per SM it is compiled for); 3 is the
@@ -65,18 +65,19 @@ enum { K_ALL = 0, K_DELTA = 1, K_TRI = 2 };
 template <bool LEARNED, int MINB, bool MATES, int KINDS = K_ALL>
 __global__ void __launch_bounds__(256, MINB) k_batch(TreeView t, BatchArgs a, const float* __restrict__ field,
                                                const float* __restrict__ pyr, unsigned* __restrict__ counter) {
-    // with the table a trilinear-only launch searches hosts only: a 32-task list per warp; the
-    // delta-kernel launch needs none (one task slot): the less shared memory, the more of the
-    // SM's memory is left to the L1 cache
-    using Q = typename std::conditional<
-        KINDS == K_DELTA, WarpQueueN<1>,
-        typename std::conditional<MATES && KINDS == K_TRI, HostQueue, WarpQueue>::type>::type;
-    __shared__ Q s_queue[256 / 32];
+    // per warp: the search's task list (with the table 32 host searches) or the delta kernel's stage,
+    // whichever the warp's tile needs
+    using Q = typename std::conditional<MATES && KINDS == K_TRI, HostQueue, WarpQueue>::type;
+    using D = DeltaStage<float>;
+    constexpr size_t bytes = KINDS == K_TRI ? sizeof(Q) : KINDS == K_DELTA ? sizeof(D)
+                             : sizeof(Q) > sizeof(D) ? sizeof(Q) : sizeof(D);
+    __shared__ __align__(16) unsigned char s_mem[256 / 32][(bytes + 15) / 16 * 16];
     __shared__ RootModel s_root;
-    Q& wq = s_queue[threadIdx.x >> 5];
+    Q& wq = *reinterpret_cast<Q*>(s_mem[threadIdx.x >> 5]);
+    D& sg = *reinterpret_cast<D*>(s_mem[threadIdx.x >> 5]);
     stage_root<LEARNED>(t, s_root);
     const int lane = threadIdx.x & 31;
-    const int64_t tile_pts = 32 * (int64_t)a.tile;
+    const int64_t tile_pts = a.pts;
     for (;;) {
         unsigned tl = 0;
         if (lane == 0) tl = atomicAdd(counter, 1u);
@@ -86,36 +87,33 @@ __global__ void __launch_bounds__(256, MINB) k_batch(TreeView t, BatchArgs a, co
         while (g + 1 < a.ng && (int64_t)tl >= a.g[g + 1].tile0) ++g;
         const GroupDev& gr = a.g[g];
         const int64_t base = ((int64_t)tl - gr.tile0) * tile_pts;
-        for (int j = 0; j < a.tile; ++j) {
-            const int64_t i = base + (int64_t)j * 32 + lane;
-            const bool active = i < gr.n;
-            if (!__any_sync(0xffffffffu, active)) break;  // warp-uniform
-            float o[3];
-            int h;
-            const double x = active ? gr.x[i] : 0.0, y = active ? gr.y[i] : 0.0, z = active ? gr.z[i] : 0.0;
-            bool tri = false;
-            if constexpr (KINDS != K_DELTA) {
-                tri = KINDS == K_TRI || gr.kernel == OT_TRILINEAR;
-                if (tri) {
-                    if constexpr (MATES)
-                        h = trilinear_mates<float, LEARNED>(t, s_root, field, pyr, wq, active, x, y, z, -1, o);
-                    else
-                        h = trilinear_queued<float, LEARNED>(t, s_root, field, pyr, wq, active, x, y, z, -1, o);
+        if (KINDS == K_DELTA || (KINDS == K_ALL && gr.kernel != OT_TRILINEAR)) {
+            const int64_t end = min(base + tile_pts, gr.n);
+            for (int64_t b = base; b < end; b += 32) {  // warp-uniform
+                const int64_t e = min(b + 32, end);
+                if (gr.kernel == OT_PESKIN4)
+                    delta_markers<float, OT_PESKIN4, LEARNED>(t, field, sg, gr.x, gr.y, gr.z, gr.n, b, e, gr.u, gr.host);
+                else
+                    delta_markers<float, OT_ROMA3, LEARNED>(t, field, sg, gr.x, gr.y, gr.z, gr.n, b, e, gr.u, gr.host);
+            }
+            continue;
+        }
+        if constexpr (KINDS != K_DELTA) {
+            for (int64_t i = base + lane; i - lane < min(base + tile_pts, gr.n); i += 32) {  // warp-uniform
+                const bool active = i < gr.n;
+                float o[3];
+                const double x = active ? gr.x[i] : 0.0, y = active ? gr.y[i] : 0.0, z = active ? gr.z[i] : 0.0;
+                int h;
+                if constexpr (MATES)
+                    h = trilinear_mates<float, LEARNED>(t, s_root, field, pyr, wq, active, x, y, z, -1, o);
+                else
+                    h = trilinear_queued<float, LEARNED>(t, s_root, field, pyr, wq, active, x, y, z, -1, o);
+                if (active) {
+                    gr.u[i] = o[0];
+                    gr.u[gr.n + i] = o[1];
+                    gr.u[2 * gr.n + i] = o[2];
+                    if (gr.host) gr.host[i] = h;
                 }
-            }
-            if (tri) {
-            } else if (!active) {
-                h = -1;
-            } else if (gr.kernel == OT_PESKIN4) {
-                h = delta_point<float, OT_PESKIN4, LEARNED>(t, field, x, y, z, gr.host != nullptr, o);
-            } else {
-                h = delta_point<float, OT_ROMA3, LEARNED>(t, field, x, y, z, gr.host != nullptr, o);
-            }
-            if (active) {
-                gr.u[i] = o[0];
-                gr.u[gr.n + i] = o[1];
-                gr.u[2 * gr.n + i] = o[2];
-                if (gr.host) gr.host[i] = h;
             }
         }
     }
@@ -274,7 +272,7 @@ __global__ void __launch_bounds__(256, TRI_MINB) k_tri_rec(TreeView t, BatchArgs
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int cell_shift = MAXLEVEL - t.lmap_level;  // of the 21-bit coordinates
-    const int64_t tile_pts = 32 * (int64_t)a.tile;
+    const int64_t tile_pts = a.pts;
     // the positions and results stream through once: evict-first (.cs), so that they push out
     // neither the cells' entries nor the records
     const uint64_t normal = policy_normal();
@@ -305,10 +303,8 @@ __global__ void __launch_bounds__(256, TRI_MINB) k_tri_rec(TreeView t, BatchArgs
         while (g + 1 < a.ng && (int64_t)tl >= a.g[g + 1].tile0) ++g;
         const GroupDev& gr = a.g[g];
         const int64_t base = ((int64_t)tl - gr.tile0) * tile_pts;
-        for (int j = 0; j < a.tile; ++j) {
-            const int64_t i = base + (int64_t)j * 32 + lane;
+        for (int64_t i = base + lane; i - lane < min(base + tile_pts, gr.n); i += 32) {  // warp-uniform
             const bool active = i < gr.n;
-            if (!__any_sync(0xffffffffu, active)) break;  // warp-uniform
             const double x = active ? __ldcs(gr.x + i) : 0.0, y = active ? __ldcs(gr.y + i) : 0.0,
                          z = active ? __ldcs(gr.z + i) : 0.0;
             uint64_t X[3];
@@ -464,7 +460,7 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
     if (order_level < 0 || order_level > MAXLEVEL) return OT_ERR_ARG;
     BatchArgs a{};
     a.ng = n_groups;
-    a.tile = tile;
+    a.pts = 32 * tile;
     // delta-kernel groups first: the longest work is taken first
     std::vector<int> order;
     for (int pass = 0; pass < 2; ++pass)
@@ -548,12 +544,23 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
     };
     std::vector<Launch> launches;
     NodeGrid grid{};
-    auto add_launch = [&](void* fn, const BatchArgs& args, int cap, size_t dsmem = 0) -> cudaError_t {
+    // min_pts: while there are fewer tiles than warps, the tiles are halved down to this many points
+    // (11,000 points in tiles of 128 would keep 86 of thousands of warps busy)
+    auto add_launch = [&](void* fn, BatchArgs args, int cap, int min_pts, size_t dsmem = 0) -> cudaError_t {
         int per_sm = 0;
         cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, dsmem);
         if (err != cudaSuccess) return err;
         if (cap > 0) per_sm = std::min(per_sm, cap);
         per_sm = std::max(per_sm, 1);
+        const int64_t warps = (int64_t)num_sms() * per_sm * (block / 32);
+        while (args.ntiles < warps && args.pts / 2 >= min_pts) {
+            args.pts /= 2;
+            args.ntiles = 0;
+            for (int k = 0; k < args.ng; ++k) {
+                args.g[k].tile0 = args.ntiles;
+                args.ntiles += (args.g[k].n + args.pts - 1) / args.pts;
+            }
+        }
         launches.push_back(Launch{fn, args, (unsigned)(num_sms() * per_sm), false, dsmem});
         return cudaSuccess;
     };
@@ -567,16 +574,16 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
     if (!t->d_mates) {
         void* fn = learned ? (two ? (void*)k_batch<true, 2, false> : (void*)k_batch<true, 3, false>)
                            : (two ? (void*)k_batch<false, 2, false> : (void*)k_batch<false, 3, false>);
-        if ((e = add_launch(fn, a, launch ? launch->blocks_per_sm : 0)) != cudaSuccess) return fail(e);
+        if ((e = add_launch(fn, a, launch ? launch->blocks_per_sm : 0, 32)) != cudaSuccess) return fail(e);
     } else {
         BatchArgs part[2] = {};
         for (int k = 0; k < a.ng; ++k) {
             BatchArgs& p = part[a.g[k].kernel == OT_TRILINEAR ? 1 : 0];
             GroupDev d = a.g[k];
             d.tile0 = p.ntiles;
-            p.tile = a.g[k].kernel == OT_TRILINEAR ? tri_tile : tile;
+            p.pts = 32 * (a.g[k].kernel == OT_TRILINEAR ? tri_tile : tile);
             p.g[p.ng++] = d;
-            p.ntiles += (d.n + 32 * (int64_t)p.tile - 1) / (32 * (int64_t)p.tile);
+            p.ntiles += (d.n + p.pts - 1) / p.pts;
         }
         if (part[1].ntiles >= (1LL << 32)) {
             ot_batch_destroy(b);
@@ -585,7 +592,7 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
         if (part[0].ng > 0) {
             void* fn = learned ? (two ? (void*)k_batch<true, 2, true, K_DELTA> : (void*)k_batch<true, 3, true, K_DELTA>)
                                : (two ? (void*)k_batch<false, 2, true, K_DELTA> : (void*)k_batch<false, 3, true, K_DELTA>);
-            if ((e = add_launch(fn, part[0], launch ? launch->blocks_per_sm : 0)) != cudaSuccess) return fail(e);
+            if ((e = add_launch(fn, part[0], launch ? launch->blocks_per_sm : 0, 4)) != cudaSuccess) return fail(e);
         }
         if (part[1].ng > 0) {
             // value records of the hot leaves: leaves of level <= min(map level, hot level), where
@@ -612,7 +619,7 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
                            : (learned ? (void*)k_batch<true, TRI_MINB, true, K_TRI>
                                       : (void*)k_batch<false, TRI_MINB, true, K_TRI>);
             const size_t dsmem = rec ? (sizeof(HostQueue) + 64 * sizeof(long long)) * (size_t)(block / 32) : 0;
-            if ((e = add_launch(fn, part[1], tri_per_sm, dsmem)) != cudaSuccess) return fail(e);
+            if ((e = add_launch(fn, part[1], tri_per_sm, 32, dsmem)) != cudaSuccess) return fail(e);
             launches.back().records = rec;
         }
     }

@@ -82,7 +82,9 @@ template <> __device__ __forceinline__ float fix_offset<float>(uint64_t X, int l
 }
 template <> __device__ __forceinline__ double fix_offset<double>(uint64_t X, int l) {
     const uint64_t f = X & ((1ULL << (53 - l)) - 1ULL);
-    return ldexp((double)f, l - 53) - 0.5;
+    if (l == 0) return ldexp((double)f, -53) - 0.5;
+    // 1 + frac put together from its bits (at most 52 of them), less 1.5: one FP64 operation, exact
+    return __longlong_as_double((long long)(0x3FF0000000000000ULL | (f << (l - 1)))) - 1.5;
 }
 // Whether the point lies in the upper half of its level-l cell (offset >= 0): one bit of X.
 __device__ __forceinline__ bool fix_upper_half(uint64_t X, int l) { return (X >> (52 - l)) & 1ULL; }
@@ -283,12 +285,15 @@ __device__ __forceinline__ int route_leaf(const RootModel& r, const LeafModel* m
 // Learned search inside a level-map cell [ca, ce) that one leaf does not cover: the models give
 // a window [pc - err_lo - 1, pc + err_hi + 1], clamped to the cell, searched by halving; the
 // answer a is verified by key[a] <= q < key[a+1], and a window that missed is answered by a
-// binary search of the cell (counted as a fallback).  Out of line: one copy serves every call
-// site, and the root network stays in device memory.
-static __device__ __noinline__ int learned_in_cell(const uint64_t* __restrict__ key, const RootModel* __restrict__ root,
-                                            const LeafModel* __restrict__ mids, const LeafModel* __restrict__ models,
-                                            int n, int n_leaf, int ca, int ce, uint64_t q,
-                                            unsigned long long* fallbacks, unsigned* err) {
+// binary search of the cell (counted as a fallback).  Inlined where the search is all that a kernel
+// does (root then in shared memory); elsewhere learned_in_cell: one copy out of line serves every
+// call site, and the root network stays in device memory.
+__device__ __forceinline__ int learned_in_cell_inline(const uint64_t* __restrict__ key,
+                                                      const RootModel* __restrict__ root,
+                                                      const LeafModel* __restrict__ mids,
+                                                      const LeafModel* __restrict__ models, int n, int n_leaf, int ca,
+                                                      int ce, uint64_t q, unsigned long long* fallbacks,
+                                                      unsigned* err) {
     const int j = route_leaf(*root, mids, n_leaf, n, q);
     const LeafModel m = models[j];
     if (m.count > 0) {
@@ -305,6 +310,13 @@ static __device__ __noinline__ int learned_in_cell(const uint64_t* __restrict__ 
     atomicAdd(fallbacks, 1ULL);
     atomicOr(err, (unsigned)OT_DEV_WINDOW);
     return search_range(key, ca, ce - ca, q);
+}
+
+static __device__ __noinline__ int learned_in_cell(const uint64_t* __restrict__ key, const RootModel* __restrict__ root,
+                                                   const LeafModel* __restrict__ mids,
+                                                   const LeafModel* __restrict__ models, int n, int n_leaf, int ca,
+                                                   int ce, uint64_t q, unsigned long long* fallbacks, unsigned* err) {
+    return learned_in_cell_inline(key, root, mids, models, n, n_leaf, ca, ce, q, fallbacks, err);
 }
 
 // Learned host search: the level map first (a covered cell answers directly), the models

@@ -15,15 +15,27 @@ template <bool LEARNED>
 __global__ void __launch_bounds__(256) k_locate(TreeView t, const double* __restrict__ x,
                                                 const double* __restrict__ y, const double* __restrict__ z, int64_t n,
                                                 int32_t* __restrict__ host, unsigned long long* n_miss) {
+    // the learned search inlined with the root network in shared memory: 10M points 268 -> 245 us
+    __shared__ RootModel s_root;
+    if (LEARNED) stage_root<LEARNED>(t, s_root);
     unsigned miss = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         uint64_t X[3];
         int h = -1;
-        if (fixpoint3(x[i], y[i], z[i], X))
-            h = search<LEARNED>(t,
-                                morton3((uint32_t)(X[0] >> 32), (uint32_t)(X[1] >> 32), (uint32_t)(X[2] >> 32)));
-        else
+        if (fixpoint3(x[i], y[i], z[i], X)) {
+            const uint64_t q = morton3((uint32_t)(X[0] >> 32), (uint32_t)(X[1] >> 32), (uint32_t)(X[2] >> 32));
+            if (LEARNED) {
+                const uint32_t c = map_cell(t, q);
+                const int ca = (int)t.lmap[c], ce = map_end(t, c);
+                h = ce - ca <= 1 ? ca
+                                 : learned_in_cell_inline(t.key, &s_root, t.mids, t.models, t.n, t.n_leaf, ca, ce, q,
+                                                          t.fallbacks, t.err);
+            } else {
+                h = search_plain(t, q);
+            }
+        } else {
             ++miss;
+        }
         host[i] = h;
     }
     if (miss) {
@@ -82,14 +94,13 @@ __global__ void __launch_bounds__(256) k_delta(TreeView t, const double* __restr
                                                const double* __restrict__ y, const double* __restrict__ z, int64_t n,
                                                const T* __restrict__ field, T* __restrict__ u,
                                                int32_t* __restrict__ host_out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T o[3];
-        const int h = delta_point<T, K, LEARNED>(t, field, x[i], y[i], z[i], host_out != nullptr, o);
-        u[i] = o[0];
-        u[n + i] = o[1];
-        u[2 * n + i] = o[2];
-        if (host_out) host_out[i] = h;
-    }
+    __shared__ DeltaStage<T> s_stage[256 / 32];
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // markers per warp at a time: 32, fewer (4 at least) when there are not that many for every warp
+    const int64_t per = min((int64_t)32, max((int64_t)4, (n + nwarps - 1) / nwarps));
+    for (int64_t base = per * warp; base < n; base += per * nwarps)
+        delta_markers<T, K, LEARNED>(t, field, s_stage[threadIdx.x >> 5], x, y, z, n, base, base + per, u, host_out);
 }
 
 template <typename Kern>
@@ -149,8 +160,9 @@ ot_status launch_interp(const ot_octree* t, int kernel, const double* x, const d
     do {                                                                                   \
         auto k_ = KERN;                                                                    \
         if ((st = prep_smem(k_, smem)) != OT_OK) return st;                                \
-        k_<<<persistent_grid(k_, block, smem, n), block, smem, s>>>(__VA_ARGS__);          \
+        k_<<<persistent_grid(k_, block, smem, n * lanes), block, smem, s>>>(__VA_ARGS__);  \
     } while (0)
+    const int64_t lanes = kernel == OT_TRILINEAR ? 1 : 8;  // per point
     if (kernel == OT_TRILINEAR) {
         // cell means of the field (refined level-mates), in the caller's workspace
         T* pyr = static_cast<T*>(ws);
