@@ -145,6 +145,11 @@ size_t spread_ws_bytes(const ot_octree* t, int kernel, int64_t n);
 template <typename T>
 ot_status launch_spread(const ot_octree* t, int kernel, int mode, const double* x, const double* y, const double* z,
                         const T* F, const T* dV, int64_t n, T* f, void* ws, size_t ws_bytes, cudaStream_t s);
+// Multi-direct forcing by tiles (lmax >= 2, n > 0); slip2 (nullable): n_iter + 1 squared slips, zeroed
+// by the caller; f zeroed by the caller; ws of spread_ws_bytes.
+ot_status launch_mdf_tiles(const ot_octree* t, int kernel, const double* x, const double* y, const double* z,
+                           const float* U, const float* dV, int64_t n, float rho, float dt, int n_iter, float* u,
+                           float* f, double* slip2, void* ws, cudaStream_t s);
 // Sorted spreading with every temporary in `scratch` (spread_noalloc_bytes(n) bytes).
 size_t spread_noalloc_bytes(int64_t n);
 ot_status launch_spread_sorted_noalloc(const ot_octree* t, int kernel, const double* x, const double* y,

@@ -230,7 +230,7 @@ __device__ __forceinline__ uint32_t bits_of(float v) { return __float_as_uint(v)
 __device__ __forceinline__ uint32_t bits_of(double v) { return (uint32_t)__double_as_longlong(v); }
 constexpr uint32_t OFF_NONE = 0x404040u;  // a marker that reaches no tile
 
-// Records in home-tile order, and the runs: a warp takes 32 consecutive markers, finds the first of
+// Records in home-tile order (F null: the forces come later), and the runs: a warp takes 32 consecutive markers, finds the first of
 // each run, its end (for the last one of the warp a 32-ary search over the markers that follow)
 // and enters it in the table and the list of runs (whose order does not matter; one atomic
 // per block's 256 markers).
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(REC_T) k_tile_records(TileOrder o, const T* __
                 if (out) atomicOr(err, (unsigned)OT_DEV_STENCIL);
                 const T vol = marker_volume(dV, k, o.lmax);
 #pragma unroll
-                for (int d = 0; d < 3; ++d) r.F[d] = F[d * n + k] * vol;
+                for (int d = 0; d < 3; ++d) r.F[d] = F ? F[d * n + k] * vol : T(0);
             } else {
                 atomicOr(err, (unsigned)OT_DEV_OUTSIDE);
 #pragma unroll
@@ -402,6 +402,23 @@ __device__ __forceinline__ void add_leaf(double* f, int leaf, const Acc3<double>
     p[0] += a.x, p[1] += a.y, p[2] += a.z;
 }
 
+// Where a tile's sums go: added to f and, scaled, to u when there is one (multi-direct forcing's
+// velocity correction).
+template <typename T> struct TileOut {
+    T* f;
+    T* u;
+    T scale;
+    __device__ __forceinline__ void add(int leaf, const Acc3<T>& a) const {
+        add_leaf(f, leaf, a);
+        if constexpr (sizeof(T) == 4) {  // (the forcing is FP32)
+            if (!u) return;
+            Acc3<T> b;
+            b.x = scale * a.x, b.y = scale * a.y, b.z = scale * a.z;
+            add_leaf(u, leaf, b);
+        }
+    }
+};
+
 // A run of home tile H stands for the tiles H + {0,1}^3; each tile is taken by the first of its 8
 // home tiles (in the order of their offsets) that has markers.  Its markers are listed run after run
 // and summed in segments of SEG list places, each from zero and the segments in order, so that
@@ -417,7 +434,7 @@ template <typename T, int K>
 __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o, RunTable rt,
                                                         const uint32_t* __restrict__ runs,
                                                         const uint32_t* __restrict__ n_runs,
-                                                        const MarkerRec<T>* __restrict__ recs, T* __restrict__ f) {
+                                                        const MarkerRec<T>* __restrict__ recs, TileOut<T> out) {
     constexpr int W = Stencil<K>::W, NW = TILE_T / 32;
     constexpr unsigned FULLM = 0xffffffffu;
     __shared__ TileStage<T> s_stage[NW];
@@ -490,8 +507,8 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
             const int mine0 = __shfl_sync(FULLM, a0, (cx >> 1) | ((cy >> 1) << 1) | (zh << 2));
             const int leaf = mine0 + ((cx & 1) | ((cy & 1) << 1));  // and leaf + 4 above it
             if (mine0 >= 0) {
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(f + 4 * (size_t)leaf));
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(f + 4 * (size_t)(leaf + 4)));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(out.f + 4 * (size_t)leaf));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(out.f + 4 * (size_t)(leaf + 4)));
             }
             // adds up to 32 list places from base to acc
             auto add32 = [&](uint32_t base, Acc3<T>(&acc)[2]) {
@@ -597,8 +614,8 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
                 if (warp != 0) continue;  // every warp has the sums; one writes them
             }
             if (mine0 >= 0) {
-                if (!sum[0].zero()) add_leaf(f, leaf, sum[0]);
-                if (!sum[1].zero()) add_leaf(f, leaf + 4, sum[1]);
+                if (!sum[0].zero()) out.add(leaf, sum[0]);
+                if (!sum[1].zero()) out.add(leaf + 4, sum[1]);
             }
         }
     }
@@ -678,16 +695,18 @@ size_t sorted_ws_bytes(int64_t n, size_t rec) {
            align_up((size_t)table_size(n) * 8) + align_up((size_t)n * 4) + 256 + 256;
 }
 
+// What a sorted spreading keeps in its workspace.
+template <typename T> struct TilePlan {
+    TileOrder o;
+    MarkerRec<T>* recs;
+    RunTable rt;
+    uint32_t *runs, *n_runs;
+};
+
+// Sorts the markers by home tile and writes records (forces from F when given) and runs.
 template <typename T, int K>
-ot_status spread_sorted(const ot_octree* t, const double* x, const double* y, const double* z, const T* F,
-                        const T* dV, int64_t n, T* f, void* ws, cudaStream_t s) {
-    TreeView v = tree_view(t);
-    if (t->lmax < 2) {
-        k_spread_unit<T, K><<<1, 8, 0, s>>>(v, x, y, z, F, dV, n, f);
-        count_launch();
-        OT_CUDA(cudaGetLastError());
-        return OT_OK;
-    }
+ot_status plan_tiles(const ot_octree* t, const double* x, const double* y, const double* z, const T* F, const T* dV,
+                     int64_t n, void* ws, cudaStream_t s, TilePlan<T>& pl) {
     // from a 256-byte boundary (records are read in 16-byte pieces)
     char* p = reinterpret_cast<char*>(((uintptr_t)ws + 255) & ~(uintptr_t)255);
     auto take = [&p](size_t bytes) {
@@ -698,17 +717,19 @@ ot_status spread_sorted(const ot_octree* t, const double* x, const double* y, co
     uint64_t* pairs = reinterpret_cast<uint64_t*>(take((size_t)n * 8));
     uint64_t* tmp = reinterpret_cast<uint64_t*>(take((size_t)n * 8));
     void* rws = take(radix_ws_bytes(n));
-    MarkerRec<T>* recs = reinterpret_cast<MarkerRec<T>*>(take((size_t)n * sizeof(MarkerRec<T>)));
-    RunTable rt{reinterpret_cast<unsigned long long*>(take((size_t)table_size(n) * 8)), (uint32_t)(table_size(n) - 1)};
-    uint32_t* runs = reinterpret_cast<uint32_t*>(take((size_t)n * 4));
-    uint32_t* n_runs = reinterpret_cast<uint32_t*>(take(4));
+    pl.recs = reinterpret_cast<MarkerRec<T>*>(take((size_t)n * sizeof(MarkerRec<T>)));
+    pl.rt = RunTable{reinterpret_cast<unsigned long long*>(take((size_t)table_size(n) * 8)),
+                     (uint32_t)(table_size(n) - 1)};
+    pl.runs = reinterpret_cast<uint32_t*>(take((size_t)n * 4));
+    pl.n_runs = reinterpret_cast<uint32_t*>(take(4));
     const int bits = 3 * (t->lmax - 2), ib = index_bits(n), room = 64 - ib;
-    TileOrder o{pairs, x, y, z, n, ib, bits <= room, t->lmax, t->periodic};
+    TileOrder& o = pl.o;
+    o = TileOrder{pairs, x, y, z, n, ib, bits <= room, t->lmax, t->periodic};
     ot_status st;
     if (n <= SMALL_SORT && o.whole) {
         auto k = k_tile_sort_small<K>;
         OT_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM));
-        k<<<1, SMALL_T, SMALL_SMEM, s>>>(o, bits, pairs, rt, n_runs);
+        k<<<1, SMALL_T, SMALL_SMEM, s>>>(o, bits, pairs, pl.rt, pl.n_runs);
         count_launch();
     } else {
         uint64_t* cur = nullptr;  // the markers' order so far (null: as given)
@@ -716,7 +737,7 @@ ot_status spread_sorted(const ot_octree* t, const double* x, const double* y, co
             const int nb = std::min(bits - sh, room);
             uint64_t* a = cur ? cur : pairs;
             auto k = k_tile_keys<K>;
-            k<<<grid_for(k, 256, 0, n), 256, 0, s>>>(o, cur, sh, nb, a, rt, n_runs);
+            k<<<grid_for(k, 256, 0, n), 256, 0, s>>>(o, cur, sh, nb, a, pl.rt, pl.n_runs);
             count_launch();
             if ((st = radix_sort_u64_ws(a, a == pairs ? tmp : pairs, n, ib, ib + nb, rws, s, nullptr, &cur)) != OT_OK)
                 return st;
@@ -724,12 +745,168 @@ ot_status spread_sorted(const ot_octree* t, const double* x, const double* y, co
         o.pairs = cur;
     }
     auto kr = k_tile_records<T, K>;
-    kr<<<grid_for(kr, REC_T, 0, n), REC_T, 0, s>>>(o, F, dV, recs, rt, runs, n_runs, v.err);
-    auto kt = k_tile_reduce<T, K>;
-    kt<<<grid_for(kt, TILE_T, 0, (int64_t)n * 8 * TILE_T), TILE_T, 0, s>>>(v, o, rt, runs, n_runs, recs, f);
-    count_launch(2);
+    kr<<<grid_for(kr, REC_T, 0, n), REC_T, 0, s>>>(o, F, dV, pl.recs, pl.rt, pl.runs, pl.n_runs, t->d_err);
+    count_launch();
     OT_CUDA(cudaGetLastError());
     return OT_OK;
+}
+
+template <typename T, int K>
+ot_status reduce_tiles(const TreeView& v, const TilePlan<T>& pl, TileOut<T> out, cudaStream_t s) {
+    auto kt = k_tile_reduce<T, K>;
+    kt<<<grid_for(kt, TILE_T, 0, pl.o.n * 8 * TILE_T), TILE_T, 0, s>>>(v, pl.o, pl.rt, pl.runs, pl.n_runs, pl.recs,
+                                                                     out);
+    count_launch();
+    OT_CUDA(cudaGetLastError());
+    return OT_OK;
+}
+
+template <typename T, int K>
+ot_status spread_sorted(const ot_octree* t, const double* x, const double* y, const double* z, const T* F,
+                        const T* dV, int64_t n, T* f, void* ws, cudaStream_t s) {
+    TreeView v = tree_view(t);
+    if (t->lmax < 2) {
+        k_spread_unit<T, K><<<1, 8, 0, s>>>(v, x, y, z, F, dV, n, f);
+        count_launch();
+        OT_CUDA(cudaGetLastError());
+        return OT_OK;
+    }
+    TilePlan<T> pl;
+    const ot_status st = plan_tiles<T, K>(t, x, y, z, F, dV, n, ws, s, pl);
+    return st == OT_OK ? reduce_tiles<T, K>(v, pl, TileOut<T>{f, nullptr, T(0)}, s) : st;
+}
+
+// Marker forces of a round of multi-direct forcing, in home-tile order: the velocity interpolated at
+// each marker, F = (U - u) / dt times the volume factor into its record, and the squared slip
+// summed into *slip2 (nullable; FP64, one atomic per block).  forces 0: the slip only.
+// A warp takes `per` consecutive markers (at most 32).  The records hold the weights, and the
+// markers of a run share the 4x4x4 blocks of finest leaves from their home tile on, looked up
+// once per run; then 8 lanes per marker sum its stencil as delta_sum does.
+template <int K>
+__global__ void __launch_bounds__(REC_T) k_tile_forces(TreeView t, TileOrder o, MarkerRec<float>* __restrict__ recs,
+                                                       const float* __restrict__ field, const float* __restrict__ U,
+                                                       const float* __restrict__ dV, float inv_dt, int per, int forces,
+                                                       double* __restrict__ slip2) {
+    constexpr int W = Stencil<K>::W;
+    constexpr unsigned FULLM = 0xffffffffu;
+    __shared__ int s_blk[REC_T / 32][64];
+    __shared__ double s_part[REC_T / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ch = lane & 7;
+    int* blk = s_blk[warp];
+    const int64_t n = o.n, nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int nb = 1 << (o.lmax - 1);  // blocks per axis
+    const int shb = MAXLEVEL - (o.lmax - 1);
+    double slip = 0.0;
+    bool missing = false;
+    for (int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * per; base < n; base += nwarps * per) {
+        const int cnt = (int)min((int64_t)per, n - base);
+        const uint64_t tile = lane < cnt ? tile_at<K>(o, base + lane) : ~0ULL;
+        for (int s0 = 0; s0 < cnt;) {  // the warp's markers of one tile: s0 .. s1 - 1
+            const uint64_t here = __shfl_sync(FULLM, tile, s0);
+            const unsigned rest = ~__ballot_sync(FULLM, tile == here) & (FULLM << s0);
+            const int s1 = rest ? min(__ffs(rest) - 1, cnt) : cnt;
+            uint32_t h[3];
+            demorton3(here, h[0], h[1], h[2]);
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int k = lane + 32 * r, b[3] = {k & 3, (k >> 2) & 3, k >> 4};
+                bool inside = true;
+                uint64_t q = 0;
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    int v = 2 * (int)h[d] + b[d];
+                    if (o.periodic) v &= nb - 1;
+                    inside = inside && v < nb;
+                    q |= part1by2((uint32_t)v << shb) << d;
+                }
+                blk[k] = inside ? find_block<false>(t, q) : -1;
+            }
+            __syncwarp();
+            for (int m = s0 + (lane >> 3); __any_sync(FULLM, m < s1); m += 4) {
+                float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;
+                uint32_t off = OFF_NONE;
+                if (m < s1) off = bits_of(recs[base + m].off);
+                const bool ok = off != OFF_NONE;
+                if (ok) {
+                    const MarkerRec<float>& rc = recs[base + m];
+                    float w[3][2];
+                    int b0[3];
+                    bool two[3];
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        const int rel = (int)((off >> (8 * d)) & 0xffu) - 8, par = rel & 1, cd = (ch >> d) & 1;
+                        const int a = cd ^ par;
+                        b0[d] = (rel >> 1) + (par & ~cd);
+                        two[d] = W == 4 || a == 0;
+                        w[d][0] = rc.w[d][a];
+                        w[d][1] = rc.w[d][a + 2];
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
+                        if ((ex && !two[0]) || (ey && !two[1]) || (ez && !two[2])) continue;
+                        const int bx = b0[0] + ex, by = b0[1] + ey, bz = b0[2] + ez;
+                        // (a stencil that starts outside the cube: blocks before the tile's)
+                        const int first = (bx | by | bz) >= 0 ? blk[bx + 4 * by + 16 * bz] : -1;
+                        missing = missing || first < 0;
+                        if (first < 0) continue;
+                        const float4 f = Vec4<float>::load(field, first + ch);
+                        const float wt = w[0][ex] * w[1][ey] * w[2][ez];
+                        u0 += wt * f.x;
+                        u1 += wt * f.y;
+                        u2 += wt * f.z;
+                    }
+                }
+#pragma unroll
+                for (int k = 1; k < 8; k <<= 1) {
+                    u0 += __shfl_xor_sync(FULLM, u0, k);
+                    u1 += __shfl_xor_sync(FULLM, u1, k);
+                    u2 += __shfl_xor_sync(FULLM, u2, k);
+                }
+                if (m < s1 && ch < 3) {
+                    const int64_t k = (int64_t)(o.pairs[base + m] & ((1ULL << o.ib) - 1));
+                    const float uk = ok ? (ch == 0 ? u0 : ch == 1 ? u1 : u2) : qnan<float>();
+                    const float e = U[ch * n + k] - uk;
+                    if (forces && ok) recs[base + m].F[ch] = e * inv_dt * marker_volume(dV, k, o.lmax);
+                    slip += (double)e * (double)e;
+                }
+            }
+            s0 = s1;
+        }
+    }
+    if (missing) atomicOr(t.err, (unsigned)OT_DEV_STENCIL);
+    if (!slip2) return;
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) slip += __shfl_xor_sync(FULLM, slip, k);
+    if (lane == 0) s_part[warp] = slip;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double b = 0.0;
+        for (int w = 0; w < REC_T / 32; ++w) b += s_part[w];
+        atomicAdd(slip2, b);
+    }
+}
+
+template <int K>
+ot_status mdf_tiles(const ot_octree* t, const double* x, const double* y, const double* z, const float* U,
+                    const float* dV, int64_t n, float rho, float dt, int n_iter, float* u, float* f, double* slip2,
+                    void* ws, cudaStream_t s) {
+    TreeView v = tree_view(t);
+    TilePlan<float> pl;
+    ot_status st = plan_tiles<float, K>(t, x, y, z, nullptr, dV, n, ws, s, pl);
+    auto k = k_tile_forces<K>;
+    const unsigned grid = grid_for(k, REC_T, 0, n * 8);
+    const int64_t warps = (int64_t)grid * (REC_T / 32);
+    const int per = (int)std::min<int64_t>(32, std::max<int64_t>(4, (n + warps - 1) / warps));
+    for (int it = 0; st == OT_OK && it <= n_iter; ++it) {
+        if (it == n_iter && !slip2) break;  // the last interpolation is for the slip alone
+        k<<<grid, REC_T, 0, s>>>(v, pl.o, pl.recs, u, U, dV, 1.0f / dt, per, it < n_iter, slip2 ? slip2 + it : nullptr);
+        count_launch();
+        if (it < n_iter) st = reduce_tiles<float, K>(v, pl, TileOut<float>{f, u, dt / rho}, s);
+    }
+    OT_CUDA(cudaGetLastError());
+    return st;
 }
 
 } // namespace
@@ -765,6 +942,16 @@ template ot_status launch_spread<float>(const ot_octree*, int, int, const double
                                         const float*, const float*, int64_t, float*, void*, size_t, cudaStream_t);
 template ot_status launch_spread<double>(const ot_octree*, int, int, const double*, const double*, const double*,
                                          const double*, const double*, int64_t, double*, void*, size_t, cudaStream_t);
+
+// Rounds of multi-direct forcing on trees of two levels or more (see ot_mdf.cu): the markers are
+// sorted and their records written once, a round is two launches.  ws: spread_ws_bytes.
+ot_status launch_mdf_tiles(const ot_octree* t, int kernel, const double* x, const double* y, const double* z,
+                           const float* U, const float* dV, int64_t n, float rho, float dt, int n_iter, float* u,
+                           float* f, double* slip2, void* ws, cudaStream_t s) {
+    if (kernel == OT_PESKIN4)
+        return mdf_tiles<OT_PESKIN4>(t, x, y, z, U, dV, n, rho, dt, n_iter, u, f, slip2, ws, s);
+    return mdf_tiles<OT_ROMA3>(t, x, y, z, U, dV, n, rho, dt, n_iter, u, f, slip2, ws, s);
+}
 
 // The same spreading with caller scratch of spread_noalloc_bytes(n) bytes (FP32 records).
 size_t spread_noalloc_bytes(int64_t n) { return sorted_ws_bytes(n, sizeof(MarkerRec<float>)); }
