@@ -126,43 +126,34 @@ __global__ void k_close_dense(const uint8_t* __restrict__ need, int64_t ncell, u
             for (int k = 0; k < 8; ++k) child_need[8 * c + k] = 1;
 }
 
-// The refined children of a refined cell of level l whose first leaf is a (anchor key[a]): each
-// child's first leaf is the leaf holding its anchor, searched within the cell's leaves from a.
-__device__ __forceinline__ void mark_refined_children(const uint64_t* __restrict__ key,
-                                                      const uint8_t* __restrict__ level, int n, int l, int a,
-                                                      int e, uint8_t* __restrict__ child_need) {
-    const uint64_t anchor = key[a] & ~(key_span(l) - 1);
+// The refined children of the refined cell of level l with the given anchor key, flagged by their
+// first leaves (a search per child).
+__device__ __forceinline__ void mark_refined_children(const TreeView& t, uint64_t anchor, int l,
+                                                      uint8_t* __restrict__ child_need) {
+#pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const uint64_t ca = anchor + (uint64_t)k * key_span(l + 1);
-        const int f = search_range(key, a, e - a, ca);
-        if ((int)level[f] > l + 1) child_need[f] = 1;
+        int lv;
+        const int f = search_plain(t, anchor + (uint64_t)k * key_span(l + 1), lv);
+        if (lv > l + 1) child_need[f] = 1;
     }
 }
 
 // needed base cells (level Lc) that are refined -> their refined children (node level 0)
-__global__ void k_close_base(const uint8_t* __restrict__ need, const uint32_t* __restrict__ pmap,
-                             const uint64_t* __restrict__ key, const uint8_t* __restrict__ level, int n, int Lc,
-                             uint8_t* __restrict__ child_need) {
+__global__ void k_close_base(TreeView t, const uint8_t* __restrict__ need, int Lc, uint8_t* __restrict__ child_need) {
     const int64_t ncell = (int64_t)1 << (3 * Lc);
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
         if (!need[c]) continue;
-        const int a = (int)pmap[c];
-        const int e = c + 1 < ncell ? (int)pmap[c + 1] : n;
-        if (e - a > 1) mark_refined_children(key, level, n, Lc, a, e, child_need);
+        const uint64_t anchor = (uint64_t)c * key_span(Lc);
+        int lv;
+        search_plain(t, anchor, lv);
+        if (lv > Lc) mark_refined_children(t, anchor, Lc, child_need);
     }
 }
 
 // needed refined cells of level l (by first leaf) -> their refined children (level l + 1)
-__global__ void k_close_node(const uint8_t* __restrict__ need, const uint64_t* __restrict__ key,
-                             const uint8_t* __restrict__ level, int n, int l, uint8_t* __restrict__ child_need) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n; a += (int64_t)gridDim.x * blockDim.x) {
-        if (!need[a]) continue;
-        // the cell's leaves end where the next cell of level l begins (at most 8^(lmax - l) leaves;
-        // the search range is capped at the leaf count)
-        const uint64_t next = (key[a] & ~(key_span(l) - 1)) + key_span(l);
-        const int e = next == 0 ? n : search_range(key, (int)a, n - (int)a, next - 1) + 1;
-        mark_refined_children(key, level, n, l, (int)a, e, child_need);
-    }
+__global__ void k_close_node(TreeView t, const uint8_t* __restrict__ need, int l, uint8_t* __restrict__ child_need) {
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < t.n; a += (int64_t)gridDim.x * blockDim.x)
+        if (need[a]) mark_refined_children(t, t.key[a] & ~(key_span(l) - 1), l, child_need);
 }
 
 // The leaves that start a refined cell of level l: level > l and key aligned to level l.
@@ -248,6 +239,7 @@ ot_status close_need_flags(ot_octree* t, uint8_t* need, cudaStream_t s) {
     const int Lc = t->pyr_level;
     const int nl = node_levels(t);
     const int n = (int)t->n;
+    const TreeView v = tree_view(t);
     for (int l = 0; l < Lc; ++l) {
         const int64_t nc = (int64_t)1 << (3 * l);
         k_close_dense<<<grid_n(nc, 256), 256, 0, s>>>(need + pyramid_offset(l), nc, need + pyramid_offset(l + 1));
@@ -256,12 +248,11 @@ ot_status close_need_flags(ot_octree* t, uint8_t* need, cudaStream_t s) {
     uint8_t* node_need = need + pyramid_offset(Lc + 1);
     if (nl > 0) {
         const int64_t nc = (int64_t)1 << (3 * Lc);
-        k_close_base<<<grid_n(nc, 256), 256, 0, s>>>(need + pyramid_offset(Lc), t->d_pmap, t->d_key, t->d_level, n, Lc,
-                                                     node_need);
+        k_close_base<<<grid_n(nc, 256), 256, 0, s>>>(v, need + pyramid_offset(Lc), Lc, node_need);
         count_launch();
     }
     for (int k = 0; k + 1 < nl; ++k) {
-        k_close_node<<<grid_n(n, 256), 256, 0, s>>>(node_need + (int64_t)k * n, t->d_key, t->d_level, n, Lc + 1 + k,
+        k_close_node<<<grid_n(n, 256), 256, 0, s>>>(v, node_need + (int64_t)k * n, Lc + 1 + k,
                                                      node_need + (int64_t)(k + 1) * n);
         count_launch();
     }
