@@ -186,6 +186,7 @@ ot_status ot_octree_build(const ot_sphere* h_spheres, int n, const ot_build_para
     ot_octree* t = new (std::nothrow) ot_octree();
     if (!t) return OT_ERR_OOM;
     cudaGetDevice(&t->device);
+    pool_octree(t->device, 1);
     cudaStream_t s = (cudaStream_t)stream;
     ot_status st = build_tree(h_spheres, n, p, s, t);
     if (st == OT_OK) st = finish_tree(t, s);
@@ -209,8 +210,9 @@ ot_status ot_octree_from_leaves(const uint64_t* d_keys, const uint8_t* d_levels,
     ot_octree* t = new (std::nothrow) ot_octree();
     if (!t) return OT_ERR_OOM;
     cudaGetDevice(&t->device);
-    cudaError_t e = cudaMalloc(&t->d_key, sizeof(uint64_t) * n);
-    if (e == cudaSuccess) e = cudaMalloc(&t->d_level, n);
+    pool_octree(t->device, 1);
+    cudaError_t e = pool_malloc((void**)&t->d_key, sizeof(uint64_t) * n, s);
+    if (e == cudaSuccess) e = pool_malloc((void**)&t->d_level, n, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(t->d_key, d_keys, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(t->d_level, d_levels, n, cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) {
@@ -285,6 +287,8 @@ ot_status ot_octree_centres(const ot_octree* t, double* d_xyz, void* stream) {
 
 ot_status ot_octree_destroy(ot_octree* t) {
     if (!t) return OT_OK;
+    // pool memory is handed out again without a wait: the work that reads it has to be done
+    cudaDeviceSynchronize();
     if (t->d_key) cudaFree(t->d_key);
     if (t->d_level) cudaFree(t->d_level);
     if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);
@@ -297,6 +301,7 @@ ot_status ot_octree_destroy(ot_octree* t) {
     if (t->d_mids) cudaFree(t->d_mids);
     if (t->d_root) cudaFree(t->d_root);
     if (t->d_err) cudaFree(t->d_err);
+    pool_octree(t->device, -1);
     delete t;
     return OT_OK;
 }

@@ -209,7 +209,7 @@ template <typename T>
 ot_status dalloc(T** p, int64_t n, cudaStream_t s) {
     *p = nullptr;
     if (n <= 0) return OT_OK;
-    OT_CUDA(cudaMallocAsync((void**)p, sizeof(T) * (size_t)n, s));
+    OT_CUDA(pool_malloc((void**)p, sizeof(T) * (size_t)n, s));
     return OT_OK;
 }
 
@@ -233,7 +233,7 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
     Guard g{s, {}};
     ot_sphere* d_sph = nullptr;
     if (nsph > 0) {
-        OT_CUDA(cudaMallocAsync(&d_sph, sizeof(ot_sphere) * nsph, s));
+        OT_CUDA(pool_malloc((void**)&d_sph, sizeof(ot_sphere) * nsph, s));
         g.keep(d_sph);
         OT_CUDA(cudaMemcpyAsync(d_sph, h_spheres, sizeof(ot_sphere) * nsph, cudaMemcpyHostToDevice, s));
     }
@@ -265,9 +265,9 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
             off[b + 1] = off[b] + (int)bins[b].size();
             idx.insert(idx.end(), bins[b].begin(), bins[b].end());
         }
-        OT_CUDA(cudaMallocAsync(&d_bin_off, sizeof(int) * off.size(), s));
+        OT_CUDA(pool_malloc((void**)&d_bin_off, sizeof(int) * off.size(), s));
         g.keep(d_bin_off);
-        OT_CUDA(cudaMallocAsync(&d_bin_sph, sizeof(int) * std::max<size_t>(idx.size(), 1), s));
+        OT_CUDA(pool_malloc((void**)&d_bin_sph, sizeof(int) * std::max<size_t>(idx.size(), 1), s));
         g.keep(d_bin_sph);
         OT_CUDA(cudaMemcpyAsync(d_bin_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, s));
         if (!idx.empty())
@@ -391,8 +391,8 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
         nleaf = M[lmin];
     }
     if (nleaf <= 0 || nleaf > OT_MAX_LEAVES) return OT_ERR_LIMIT;
-    OT_CUDA(cudaMalloc(&t->d_key, sizeof(uint64_t) * nleaf));
-    OT_CUDA(cudaMalloc(&t->d_level, nleaf));
+    OT_CUDA(pool_malloc((void**)&t->d_key, sizeof(uint64_t) * nleaf, s));
+    OT_CUDA(pool_malloc((void**)&t->d_level, nleaf, s));
     for (int l = lmin; l <= lmax; ++l) {
         if (M[l] == 0) continue;
         const uint32_t* o = off[l];
@@ -468,8 +468,8 @@ ot_status validate_leaves(const uint64_t* d_key, const uint8_t* d_level, int64_t
                           int* lmax) {
     unsigned* bad = nullptr;
     int* lr = nullptr;
-    OT_CUDA(cudaMallocAsync(&bad, 2 * sizeof(unsigned), s));
-    OT_CUDA(cudaMallocAsync(&lr, 2 * sizeof(int), s));
+    OT_CUDA(pool_malloc((void**)&bad, 2 * sizeof(unsigned), s));
+    OT_CUDA(pool_malloc((void**)&lr, 2 * sizeof(int), s));
     int init[2] = {1 << 20, -1};
     OT_CUDA(cudaMemsetAsync(bad, 0, 2 * sizeof(unsigned), s));
     OT_CUDA(cudaMemcpyAsync(lr, init, sizeof(init), cudaMemcpyHostToDevice, s));
@@ -563,20 +563,22 @@ ot_status finish_tree(ot_octree* t, cudaStream_t s, int map_level) {
     const int Lp = std::min(t->lmax, 7);
     if (!t->d_pmap) {
         const int64_t np = (int64_t)1 << (3 * Lp);
-        OT_CUDA(cudaMalloc(&t->d_pmap, sizeof(uint32_t) * np));
+        OT_CUDA(pool_malloc((void**)&t->d_pmap, sizeof(uint32_t) * np, s));
         k_lmap<<<grid1d(np, 256), 256, 0, s>>>(t->d_key, (int)t->n, Lp, np, t->d_pmap);
         count_launch();
         t->pyr_level = Lp;
         ot_status st = build_node_lists(t, s);
         if (st != OT_OK) return st;
     }
+    // (a change of the map level: work on other streams may still read the old map)
+    if (t->d_lmap || t->d_desc) OT_CUDA(cudaDeviceSynchronize());
     if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);
     t->d_lmap = nullptr;
     if (L == Lp) {
         t->d_lmap = t->d_pmap;
     } else {
         const int64_t ncell = (int64_t)1 << (3 * L);
-        OT_CUDA(cudaMalloc(&t->d_lmap, sizeof(uint32_t) * ncell));
+        OT_CUDA(pool_malloc((void**)&t->d_lmap, sizeof(uint32_t) * ncell, s));
         k_lmap<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_key, (int)t->n, L, ncell, t->d_lmap);
         count_launch();
     }
@@ -584,7 +586,7 @@ ot_status finish_tree(ot_octree* t, cudaStream_t s, int map_level) {
     if (t->d_desc) cudaFree(t->d_desc);
     t->d_desc = nullptr;
     const int64_t ncell = (int64_t)1 << (3 * L);
-    OT_CUDA(cudaMalloc(&t->d_desc, sizeof(uint4) * ncell));
+    OT_CUDA(pool_malloc((void**)&t->d_desc, sizeof(uint4) * ncell, s));
     k_desc_cells<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_level, (int)t->n, t->d_lmap, ncell, t->d_desc);
     count_launch();
     if (L + 2 <= t->lmax) {
@@ -593,7 +595,7 @@ ot_status finish_tree(ot_octree* t, cudaStream_t s, int map_level) {
         count_launch();
     }
     if (!t->d_err) {
-        OT_CUDA(cudaMalloc(&t->d_err, 64));
+        OT_CUDA(pool_malloc((void**)&t->d_err, 64, s));
         OT_CUDA(cudaMemsetAsync(t->d_err, 0, 64, s));
         t->d_fallbacks = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(t->d_err) + 8);
     }

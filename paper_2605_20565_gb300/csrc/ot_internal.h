@@ -65,6 +65,12 @@ ot_status cuda_status(cudaError_t e);
     } while (0)
 
 int num_sms();
+int blocks_per_sm(const void* fn, int block, size_t smem);
+
+// Stream-ordered device memory from the library's pool (ot_pool.cu); freed with cudaFreeAsync, or
+// with cudaFree once no work uses it.  pool_octree: an octree was made on (1) or left (-1) dev.
+cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s);
+void pool_octree(int dev, int change);
 
 TreeView tree_view(const ot_octree* t);
 
@@ -133,6 +139,7 @@ template <typename T> ot_status launch_pyramid(const ot_octree* t, const T* fiel
 ot_status build_mates(ot_octree* t, cudaStream_t s);
 size_t mates_bytes(const ot_octree* t);
 bool mates_fit(const ot_octree* t);
+void drop_need_flags(ot_octree* t);
 
 // Morton order of points (ot_order.cu) ----------------------------------------------------------
 size_t order_ws_bytes(int64_t n);

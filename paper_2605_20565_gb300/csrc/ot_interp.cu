@@ -105,9 +105,7 @@ __global__ void __launch_bounds__(256) k_delta(TreeView t, const double* __restr
 
 template <typename Kern>
 unsigned persistent_grid(Kern k, int block, size_t smem, int64_t n) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
-    per_sm = std::max(per_sm, 1);
+    const int per_sm = blocks_per_sm((const void*)k, block, smem);
     int64_t need = (n + block - 1) / block;
     int64_t g = std::min<int64_t>((int64_t)num_sms() * per_sm, need);
     return (unsigned)std::max<int64_t>(g, 1);

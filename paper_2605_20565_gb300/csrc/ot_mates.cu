@@ -191,21 +191,27 @@ bool mates_fit(const ot_octree* t) {
     return means < ((int64_t)1 << 31) && t->n < ((int64_t)1 << 31);
 }
 
+// Frees the flags (pool memory, whose release does not wait for work that may still read it).
+void drop_need_flags(ot_octree* t) {
+    if (!t->d_need_flags) return;
+    cudaDeviceSynchronize();
+    cudaFree(t->d_need_flags);
+    t->d_need_flags = nullptr;
+}
+
 // Fills the octree's table (t->d_mates, mates_bytes(t) bytes) on stream s.
 ot_status build_mates(ot_octree* t, cudaStream_t s) {
     if (!t->d_mates) return OT_ERR_ARG;
     if (!mates_fit(t)) return OT_ERR_LIMIT;
     TreeView v = tree_view(t);
-    int per_sm = 0;
-    OT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mates, MATES_T, 0));
-    const int64_t grid = std::min<int64_t>((t->n + MATES_T - 1) / MATES_T, (int64_t)num_sms() * std::max(per_sm, 1));
+    const int64_t grid = std::min<int64_t>((t->n + MATES_T - 1) / MATES_T,
+                                           (int64_t)num_sms() * blocks_per_sm((const void*)k_mates, MATES_T, 0));
     // flags of the cell means the table reads (kept by the octree: later pyramids compute
     // those only)
     const size_t nbytes = std::max<size_t>(need_flag_bytes(t), 1);
-    if (t->d_need_flags) cudaFree(t->d_need_flags);
-    t->d_need_flags = nullptr;
+    drop_need_flags(t);
     uint8_t* need = nullptr;
-    OT_CUDA(cudaMalloc(&need, nbytes));
+    OT_CUDA(pool_malloc((void**)&need, nbytes, s));
     OT_CUDA(cudaMemsetAsync(need, 0, nbytes, s));
     int* pn = pnbr_slots(t) ? reinterpret_cast<int*>(reinterpret_cast<char*>(t->d_mates) + (size_t)256 * t->n) : nullptr;
     k_mates<<<(unsigned)std::max<int64_t>(grid, 1), MATES_T, 0, s>>>(v, reinterpret_cast<uint4*>(t->d_mates), pn, need);
@@ -213,7 +219,7 @@ ot_status build_mates(ot_octree* t, cudaStream_t s) {
     OT_CUDA(cudaGetLastError());
     const ot_status st = close_need_flags(t, need, s);
     if (st != OT_OK) {
-        cudaFree(need);
+        cudaFreeAsync(need, s);
         return st;
     }
     t->d_need_flags = need;
@@ -229,8 +235,7 @@ namespace {
 
 // Drops the octree's table (freed when the library owns it).
 void drop_mates(ot_octree* t) {
-    if (t->d_need_flags) cudaFree(t->d_need_flags);  // without the table every mean is computed again
-    t->d_need_flags = nullptr;
+    drop_need_flags(t);  // without the table every mean is computed again
     if (t->d_mates && t->mates_owned) cudaFree(t->d_mates);
     t->d_mates = nullptr;
     t->mates_owned = false;

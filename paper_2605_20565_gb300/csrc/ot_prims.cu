@@ -13,13 +13,6 @@ ot_status cuda_status(cudaError_t e) {
     return OT_ERR_CUDA;
 }
 
-int num_sms() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
-}
-
 // ------------------------------------------------------------------------------------------
 // Exclusive scan (uint32): block-local scans, scan of block totals (recursive), add-back.
 // ------------------------------------------------------------------------------------------
@@ -132,7 +125,7 @@ ot_status scan_u32_ws(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t
 
 ot_status scan_u32(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* d_total, cudaStream_t s) {
     void* ws = nullptr;
-    OT_CUDA(cudaMallocAsync(&ws, scan_ws_bytes(n), s));
+    OT_CUDA(pool_malloc((void**)&ws, scan_ws_bytes(n), s));
     ot_status st = scan_u32_ws(d_in, d_out, n, d_total, ws, s);
     cudaFreeAsync(ws, s);
     return st;
@@ -312,7 +305,7 @@ ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bi
 ot_status radix_sort_u64(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, cudaStream_t s) {
     if (n <= 1 || bit1 <= bit0) return OT_OK;
     void* ws = nullptr;
-    OT_CUDA(cudaMallocAsync(&ws, radix_ws_bytes(n), s));
+    OT_CUDA(pool_malloc((void**)&ws, radix_ws_bytes(n), s));
     ot_status st = radix_sort_u64_ws(d_keys, d_tmp, n, bit0, bit1, ws, s);
     cudaFreeAsync(ws, s);
     return st;
@@ -340,7 +333,7 @@ ot_status compact_u64(const uint64_t* d_in, const uint32_t* d_flag, uint32_t* d_
         return OT_OK;
     }
     uint32_t* tot = nullptr;
-    OT_CUDA(cudaMallocAsync(&tot, sizeof(uint32_t), s));
+    OT_CUDA(pool_malloc((void**)&tot, sizeof(uint32_t), s));
     ot_status st = scan_u32(d_flag, d_scan, n, tot, s);
     if (st != OT_OK) return st;
     k_compact<<<grid_for(n, 256), 256, 0, s>>>(d_in, d_flag, d_scan, n, d_out);
@@ -365,9 +358,9 @@ ot_status unique_u64(uint64_t* d_keys, int64_t n, int64_t* h_count, cudaStream_t
     }
     uint32_t *flag = nullptr, *pos = nullptr;
     uint64_t* tmp = nullptr;
-    OT_CUDA(cudaMallocAsync(&flag, sizeof(uint32_t) * n, s));
-    OT_CUDA(cudaMallocAsync(&pos, sizeof(uint32_t) * n, s));
-    OT_CUDA(cudaMallocAsync(&tmp, sizeof(uint64_t) * n, s));
+    OT_CUDA(pool_malloc((void**)&flag, sizeof(uint32_t) * n, s));
+    OT_CUDA(pool_malloc((void**)&pos, sizeof(uint32_t) * n, s));
+    OT_CUDA(pool_malloc((void**)&tmp, sizeof(uint64_t) * n, s));
     k_head_flags<<<grid_for(n, 256), 256, 0, s>>>(d_keys, n, flag);
     count_launch();
     int64_t m = 0;

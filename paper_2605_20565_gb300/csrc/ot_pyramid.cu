@@ -191,9 +191,9 @@ ot_status build_node_lists(ot_octree* t, cudaStream_t s) {
     t->d_nodes = nullptr;
     if (nl == 0 || t->n == 0) return OT_OK;
     uint32_t *flag = nullptr, *pos = nullptr, *tot = nullptr;
-    OT_CUDA(cudaMallocAsync(&flag, sizeof(uint32_t) * t->n, s));
-    OT_CUDA(cudaMallocAsync(&pos, sizeof(uint32_t) * t->n, s));
-    OT_CUDA(cudaMallocAsync(&tot, sizeof(uint32_t), s));
+    OT_CUDA(pool_malloc((void**)&flag, sizeof(uint32_t) * t->n, s));
+    OT_CUDA(pool_malloc((void**)&pos, sizeof(uint32_t) * t->n, s));
+    OT_CUDA(pool_malloc((void**)&tot, sizeof(uint32_t), s));
     std::vector<int64_t> cnt(nl);
     for (int k = 0; k < nl; ++k) {  // counts first, then one allocation
         k_flag_nodes<<<grid_n(t->n, 256), 256, 0, s>>>(t->d_key, t->d_level, (int)t->n, t->pyr_level + 1 + k, flag);
@@ -211,7 +211,7 @@ ot_status build_node_lists(ot_octree* t, cudaStream_t s) {
         t->node_cnt[k] = cnt[k];
         total += cnt[k];
     }
-    OT_CUDA(cudaMalloc(&t->d_nodes, sizeof(int) * std::max<int64_t>(total, 1)));
+    OT_CUDA(pool_malloc((void**)&t->d_nodes, sizeof(int) * std::max<int64_t>(total, 1), s));
     for (int k = 0; k < nl; ++k) {
         k_flag_nodes<<<grid_n(t->n, 256), 256, 0, s>>>(t->d_key, t->d_level, (int)t->n, t->pyr_level + 1 + k, flag);
         ot_status st = scan_u32(flag, pos, t->n, nullptr, s);

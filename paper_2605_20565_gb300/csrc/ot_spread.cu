@@ -668,9 +668,7 @@ __global__ void k_spread_unit(TreeView t, const double* __restrict__ x, const do
 
 template <typename Kern>
 unsigned grid_for(Kern k, int block, size_t smem, int64_t n) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
-    per_sm = std::max(per_sm, 1);
+    const int per_sm = blocks_per_sm((const void*)k, block, smem);
     int64_t need = (n + block - 1) / block;
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * per_sm, need));
 }
