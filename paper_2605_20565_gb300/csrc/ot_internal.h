@@ -90,12 +90,14 @@ ot_status radix_sort_u64(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0,
 size_t radix_ws_bytes(int64_t n);
 ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
                             cudaStream_t s, const uint32_t* d_n = nullptr, uint64_t** result = nullptr);
+// Exclusive scan of a short row in place by one block; its total to *d_total.
+ot_status scan_row(uint32_t* d_row, int n, uint32_t* d_total, cudaStream_t s);
 // Compaction: out[j] = in[i] for the i with flag[i] != 0, in order; *h_count on the host
-// (synchronises).  d_scan: n uint32 scratch.
-ot_status compact_u64(const uint64_t* d_in, const uint32_t* d_flag, uint32_t* d_scan, int64_t n, uint64_t* d_out,
-                      int64_t* h_count, cudaStream_t s);
-// Sorted input -> unique values in place; *h_count on the host (synchronises).
-ot_status unique_u64(uint64_t* d_keys, int64_t n, int64_t* h_count, cudaStream_t s);
+// (synchronises).
+ot_status compact_u64(const uint64_t* d_in, const uint32_t* d_flag, int64_t n, uint64_t* d_out, int64_t* h_count,
+                      cudaStream_t s);
+// Sorted input -> its unique values in d_out; *h_count on the host (synchronises).
+ot_status unique_u64(const uint64_t* d_keys, int64_t n, uint64_t* d_out, int64_t* h_count, cudaStream_t s);
 
 // builder (ot_build.cu) ------------------------------------------------------------------------
 ot_status build_tree(const ot_sphere* h_spheres, int n, const ot_build_params* p, cudaStream_t s, ot_octree* t);

@@ -3,6 +3,7 @@
 #include <algorithm>
 
 #include "ot_internal.h"
+#include "ot_select.cuh"
 
 namespace ot {
 
@@ -314,64 +315,61 @@ ot_status radix_sort_u64(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0,
 // ------------------------------------------------------------------------------------------
 // Compaction and unique.
 // ------------------------------------------------------------------------------------------
-__global__ void k_compact(const uint64_t* __restrict__ in, const uint32_t* __restrict__ flag,
-                          const uint32_t* __restrict__ pos, int64_t n, uint64_t* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) out[pos[i]] = in[i];
-}
+namespace {
+struct Flagged {
+    const uint32_t* flag;
+    __device__ bool operator()(int64_t i) const { return __ldg(flag + i) != 0; }
+};
+struct FirstOfEqual {
+    const uint64_t* k;
+    __device__ bool operator()(int64_t i) const { return i == 0 || k[i] != k[i - 1]; }
+};
+struct CopyTo {
+    const uint64_t* in;
+    uint64_t* out;
+    __device__ void operator()(int64_t i, uint32_t at) const { out[at] = in[i]; }
+};
 
-static unsigned grid_for(int64_t n, int block) {
-    int64_t g = (n + block - 1) / block;
-    int64_t cap = (int64_t)num_sms() * 32;
-    return (unsigned)std::max<int64_t>(1, std::min(g, cap));
-}
-
-ot_status compact_u64(const uint64_t* d_in, const uint32_t* d_flag, uint32_t* d_scan, int64_t n, uint64_t* d_out,
-                      int64_t* h_count, cudaStream_t s) {
-    if (n <= 0) {
-        *h_count = 0;
-        return OT_OK;
-    }
-    uint32_t* tot = nullptr;
-    OT_CUDA(pool_malloc((void**)&tot, sizeof(uint32_t), s));
-    ot_status st = scan_u32(d_flag, d_scan, n, tot, s);
-    if (st != OT_OK) return st;
-    k_compact<<<grid_for(n, 256), 256, 0, s>>>(d_in, d_flag, d_scan, n, d_out);
-    count_launch();
+template <typename Pred>
+ot_status select_u64(Pred pred, const uint64_t* d_in, int64_t n, uint64_t* d_out, int64_t* h_count, cudaStream_t s) {
+    uint32_t* cnt = nullptr;
+    const int64_t nt = select_tiles(n);
+    OT_CUDA(pool_malloc((void**)&cnt, sizeof(uint32_t) * (size_t)(nt + 1), s));
+    ot_status st = select_count(pred, n, cnt, cnt + nt, s);
+    if (st == OT_OK) st = select_emit(pred, CopyTo{d_in, d_out}, n, cnt, s);
     uint32_t h = 0;
-    OT_CUDA(cudaMemcpyAsync(&h, tot, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    OT_CUDA(cudaFreeAsync(tot, s));
+    cudaError_t e = cudaMemcpyAsync(&h, cnt + nt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    cudaFreeAsync(cnt, s);
+    if (st != OT_OK) return st;
+    OT_CUDA(e);
     OT_CUDA(cudaStreamSynchronize(s));
     *h_count = h;
     return OT_OK;
 }
+} // namespace
 
-__global__ void k_head_flags(const uint64_t* __restrict__ k, int64_t n, uint32_t* __restrict__ flag) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = (i == 0 || k[i] != k[i - 1]) ? 1u : 0u;
+ot_status scan_row(uint32_t* d_row, int n, uint32_t* d_total, cudaStream_t s) {
+    k_radix_rows<<<1, ROW_T, 0, s>>>(d_row, n, d_total);
+    count_launch();
+    OT_CUDA(cudaGetLastError());
+    return OT_OK;
 }
 
-ot_status unique_u64(uint64_t* d_keys, int64_t n, int64_t* h_count, cudaStream_t s) {
-    if (n <= 1) {
-        *h_count = n;
+ot_status compact_u64(const uint64_t* d_in, const uint32_t* d_flag, int64_t n, uint64_t* d_out, int64_t* h_count,
+                      cudaStream_t s) {
+    if (n <= 0) {
+        *h_count = 0;
         return OT_OK;
     }
-    uint32_t *flag = nullptr, *pos = nullptr;
-    uint64_t* tmp = nullptr;
-    OT_CUDA(pool_malloc((void**)&flag, sizeof(uint32_t) * n, s));
-    OT_CUDA(pool_malloc((void**)&pos, sizeof(uint32_t) * n, s));
-    OT_CUDA(pool_malloc((void**)&tmp, sizeof(uint64_t) * n, s));
-    k_head_flags<<<grid_for(n, 256), 256, 0, s>>>(d_keys, n, flag);
-    count_launch();
-    int64_t m = 0;
-    ot_status st = compact_u64(d_keys, flag, pos, n, tmp, &m, s);
-    if (st != OT_OK) return st;
-    OT_CUDA(cudaMemcpyAsync(d_keys, tmp, sizeof(uint64_t) * m, cudaMemcpyDeviceToDevice, s));
-    OT_CUDA(cudaFreeAsync(flag, s));
-    OT_CUDA(cudaFreeAsync(pos, s));
-    OT_CUDA(cudaFreeAsync(tmp, s));
-    *h_count = m;
-    return OT_OK;
+    return select_u64(Flagged{d_flag}, d_in, n, d_out, h_count, s);
+}
+
+ot_status unique_u64(const uint64_t* d_keys, int64_t n, uint64_t* d_out, int64_t* h_count, cudaStream_t s) {
+    if (n <= 0) {
+        *h_count = 0;
+        return OT_OK;
+    }
+    return select_u64(FirstOfEqual{d_keys}, d_keys, n, d_out, h_count, s);
 }
 
 } // namespace ot

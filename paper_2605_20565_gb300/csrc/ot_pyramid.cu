@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "ot_internal.h"
+#include "ot_select.cuh"
 
 namespace ot {
 
@@ -157,18 +158,18 @@ __global__ void k_close_node(TreeView t, const uint8_t* __restrict__ need, int l
 }
 
 // The leaves that start a refined cell of level l: level > l and key aligned to level l.
-__global__ void k_flag_nodes(const uint64_t* __restrict__ key, const uint8_t* __restrict__ level, int n, int l,
-                             uint32_t* __restrict__ flag) {
-    const uint64_t mask = key_span(l) - 1;
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n; a += (int64_t)gridDim.x * blockDim.x)
-        flag[a] = ((int)level[a] > l && (key[a] & mask) == 0) ? 1u : 0u;
-}
-
-__global__ void k_scatter_nodes(const uint32_t* __restrict__ flag, const uint32_t* __restrict__ pos, int n,
-                                int* __restrict__ out) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n; a += (int64_t)gridDim.x * blockDim.x)
-        if (flag[a]) out[pos[a]] = (int)a;
-}
+struct StartsCell {
+    const uint64_t* key;
+    const uint8_t* level;
+    int l;
+    __device__ bool operator()(int64_t i) const {
+        return (int)__ldg(level + i) > l && (ldg_key(key + i) & (key_span(l) - 1)) == 0;
+    }
+};
+struct ListLeaf {
+    int* out;
+    __device__ void operator()(int64_t i, uint32_t at) const { out[at] = (int)i; }
+};
 
 unsigned grid_n(int64_t n, int b) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + b - 1) / b, (int64_t)num_sms() * 16));
@@ -190,39 +191,31 @@ ot_status build_node_lists(ot_octree* t, cudaStream_t s) {
     if (t->d_nodes) cudaFree(t->d_nodes);
     t->d_nodes = nullptr;
     if (nl == 0 || t->n == 0) return OT_OK;
-    uint32_t *flag = nullptr, *pos = nullptr, *tot = nullptr;
-    OT_CUDA(pool_malloc((void**)&flag, sizeof(uint32_t) * t->n, s));
-    OT_CUDA(pool_malloc((void**)&pos, sizeof(uint32_t) * t->n, s));
-    OT_CUDA(pool_malloc((void**)&tot, sizeof(uint32_t), s));
-    std::vector<int64_t> cnt(nl);
-    for (int k = 0; k < nl; ++k) {  // counts first, then one allocation
-        k_flag_nodes<<<grid_n(t->n, 256), 256, 0, s>>>(t->d_key, t->d_level, (int)t->n, t->pyr_level + 1 + k, flag);
-        count_launch();
-        ot_status st = scan_u32(flag, pos, t->n, tot, s);
-        if (st != OT_OK) return st;
-        uint32_t h = 0;
-        OT_CUDA(cudaMemcpyAsync(&h, tot, sizeof(h), cudaMemcpyDeviceToHost, s));
+    // counts of all levels first, then one allocation
+    const int64_t nt = select_tiles(t->n);
+    uint32_t* cnt = nullptr;
+    OT_CUDA(pool_malloc((void**)&cnt, sizeof(uint32_t) * (size_t)(nl * (nt + 1)), s));
+    uint32_t* tot = cnt + nl * nt;
+    ot_status st = OT_OK;
+    for (int k = 0; k < nl && st == OT_OK; ++k)
+        st = select_count(StartsCell{t->d_key, t->d_level, t->pyr_level + 1 + k}, t->n, cnt + k * nt, tot + k, s);
+    std::vector<uint32_t> h(nl);
+    if (st == OT_OK) {
+        OT_CUDA(cudaMemcpyAsync(h.data(), tot, sizeof(uint32_t) * nl, cudaMemcpyDeviceToHost, s));
         OT_CUDA(cudaStreamSynchronize(s));
-        cnt[k] = h;
+        int64_t total = 0;
+        for (int k = 0; k < nl; ++k) {
+            t->node_off[k] = total;
+            t->node_cnt[k] = h[k];
+            total += h[k];
+        }
+        OT_CUDA(pool_malloc((void**)&t->d_nodes, sizeof(int) * std::max<int64_t>(total, 1), s));
     }
-    int64_t total = 0;
-    for (int k = 0; k < nl; ++k) {
-        t->node_off[k] = total;
-        t->node_cnt[k] = cnt[k];
-        total += cnt[k];
-    }
-    OT_CUDA(pool_malloc((void**)&t->d_nodes, sizeof(int) * std::max<int64_t>(total, 1), s));
-    for (int k = 0; k < nl; ++k) {
-        k_flag_nodes<<<grid_n(t->n, 256), 256, 0, s>>>(t->d_key, t->d_level, (int)t->n, t->pyr_level + 1 + k, flag);
-        ot_status st = scan_u32(flag, pos, t->n, nullptr, s);
-        if (st != OT_OK) return st;
-        k_scatter_nodes<<<grid_n(t->n, 256), 256, 0, s>>>(flag, pos, (int)t->n, t->d_nodes + t->node_off[k]);
-        count_launch(2);
-    }
-    cudaFreeAsync(flag, s);
-    cudaFreeAsync(pos, s);
-    cudaFreeAsync(tot, s);
-    OT_CUDA(cudaGetLastError());
+    for (int k = 0; k < nl && st == OT_OK; ++k)
+        st = select_emit(StartsCell{t->d_key, t->d_level, t->pyr_level + 1 + k}, ListLeaf{t->d_nodes + t->node_off[k]},
+                         t->n, cnt + k * nt, s);
+    cudaFreeAsync(cnt, s);
+    if (st != OT_OK) return st;
     OT_CUDA(cudaStreamSynchronize(s));
     return OT_OK;
 }
