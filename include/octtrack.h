@@ -241,7 +241,8 @@ ot_status ot_locate(const ot_octree* t, const double* d_x, const double* d_y, co
  *     The refined means are rebuilt by each call from the field, in the caller's workspace:
  *     a dense pyramid of cell means over levels 0 .. L = min(lmax, 7) (16 * (8^(L+1) - 1) / 7
  *     bytes in FP32, 38 MB at L = 7) and, for levels L+1 .. lmax-1, one array of N means per
- *     level indexed by the refined cell's first leaf (16 N bytes per level in FP32).
+ *     level indexed by the refined cell's first leaf (16 N bytes per level in FP32); then a
+ *     flag byte per mean (calls with few points compute only the means they read).
  *   OT_PESKIN4 / OT_ROMA3 (Sec. 2.2, Eq. ibm_interpolate): u(X) = sum over the 4^3 / 3^3
  *     finest-level cells around X of phi(rx) phi(ry) phi(rz) u(cell); Peskin's 4-point or
  *     the paper's 3-point function.  Cells outside the cube or not finest-level leaves are
@@ -262,7 +263,7 @@ ot_status ot_interpolate_f64(const ot_octree* t, int kernel, const double* d_x, 
                              size_t ws_bytes, void* stream);
 
 /* *bytes = the workspace of ot_interpolate (fp64 = 0) or ot_interpolate_f64 (fp64 = 1) with
- * the given kernel on this octree: the cell means for OT_TRILINEAR, 0 for the delta kernels.
+ * the given kernel on this octree: the cell means and flags for OT_TRILINEAR, 0 for the delta kernels.
  * It does not depend on the point count. */
 ot_status ot_interpolate_workspace_size(const ot_octree* t, int kernel, int fp64, size_t* bytes);
 

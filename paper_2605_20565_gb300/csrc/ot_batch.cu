@@ -649,7 +649,7 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
                                                           o.user.z, o.xs, o.ys, o.zs);
         count_launch();
     }
-    if (cap_ok && has_tri) cap_ok = launch_pyramid<float>(t, d_field, b->d_pyr, cs) == OT_OK;
+    if (cap_ok && has_tri) cap_ok = launch_pyramid<float>(t, d_field, b->d_pyr, t->d_need_flags, cs) == OT_OK;
     if (cap_ok && b->n_rec > 0) {
         k_hot_records<<<grid_b(b->n_rec), 256, 0, cs>>>(v, b->d_nodes, b->n_rec, d_field, b->d_pyr, b->d_rec);
         count_launch();

@@ -116,7 +116,7 @@ ot_status mlp_grad(const float* d_params, const float* d_x, const float* d_t, in
 ot_status launch_locate(const ot_octree* t, const double* x, const double* y, const double* z, int64_t n, int search,
                         int32_t* host, unsigned long long* n_miss, cudaStream_t s);
 // Trilinear interpolation needs interp_ws_bytes(t, OT_TRILINEAR, sizeof(T)) bytes of workspace
-// (the cell means of the field, 16-byte aligned); the delta kernels need none.
+// (the cell means of the field and their flags, 16-byte aligned); the delta kernels need none.
 template <typename T>
 ot_status launch_interp(const ot_octree* t, int kernel, const double* x, const double* y, const double* z, int64_t n,
                         const int32_t* host_in, int search, const T* field, T* u, int32_t* host_out, void* ws,
@@ -133,9 +133,11 @@ ot_status build_node_lists(ot_octree* t, cudaStream_t s);
 // Flags of the means the level-mate table reads (need_flag_bytes(t) bytes, one per entry of
 // the means array, set by the table builder), closed under "a mean needs its children's".
 size_t need_flag_bytes(const ot_octree* t);
-ot_status close_need_flags(ot_octree* t, uint8_t* need, cudaStream_t s);
+ot_status close_need_flags(const ot_octree* t, uint8_t* need, cudaStream_t s);
 size_t pyramid_bytes(const ot_octree* t, size_t elem);  // elem: sizeof the field type
-template <typename T> ot_status launch_pyramid(const ot_octree* t, const T* field, T* pyr, cudaStream_t s);
+// need (nullable): flags, closed, of the means to compute.
+template <typename T>
+ot_status launch_pyramid(const ot_octree* t, const T* field, T* pyr, const uint8_t* need, cudaStream_t s);
 
 // level-mate table (ot_mates.cu): fills t->d_mates (mates_bytes(t) bytes) on stream s -----
 ot_status build_mates(ot_octree* t, cudaStream_t s);

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "ot_internal.h"
+#include "ot_points.cuh"
 #include "ot_select.cuh"
 
 namespace ot {
@@ -26,72 +27,80 @@ __device__ __forceinline__ double count_bits(int c, double) { return __longlong_
 __device__ __forceinline__ int bits_count(float v) { return __float_as_int(v); }
 __device__ __forceinline__ int bits_count(double v) { return (int)__double_as_longlong(v); }
 
-// Mean of the 8 children of the refined cell of level l whose first leaf is a, written to p
-// with the cell's leaf count.  child: node means of level l + 1 (null when l + 1 == lmax: every
-// child is a leaf).
+// Mean of the 8 children of the refined cell of level l whose first leaf is a, written to p with the
+// cell's leaf count.  child: node means of level l + 1 (not read when l + 1 == lmax: every child is a
+// leaf, the 8 from a on, loaded together).  Otherwise from child to child by their leaf counts
+// (searching the 8 children side by side measured 10% slower: more to read).
 template <typename T>
-__device__ __forceinline__ void children_mean(const uint8_t* __restrict__ level, int l, const T* __restrict__ field,
+__device__ __forceinline__ void children_mean(const TreeView& t, int l, const T* __restrict__ field,
                                               const T* __restrict__ child, int a, T* __restrict__ p) {
     using V = Vec4<T>;
-    int pos = a;
     T s0 = T(0), s1 = T(0), s2 = T(0);
-    for (int ch = 0; ch < 8; ++ch) {
-        typename V::type f;
-        int step = 1;
-        if ((int)level[pos] == l + 1) {
-            f = V::load(field, pos);
-        } else {
-            f = V::load(child, pos);
-            step = bits_count(f.w);
+    int pos = a;
+    if (l + 1 == t.lmax) {
+#pragma unroll
+        for (int ch = 0; ch < 8; ++ch) {
+            const auto f = V::load(field, a + ch);
+            s0 += f.x;
+            s1 += f.y;
+            s2 += f.z;
         }
-        s0 += f.x;
-        s1 += f.y;
-        s2 += f.z;
-        pos += step;
+        pos += 8;
+    } else {
+        for (int ch = 0; ch < 8; ++ch) {
+            typename V::type f;
+            int step = 1;
+            if ((int)t.level[pos] == l + 1) {
+                f = V::load(field, pos);
+            } else {
+                f = V::load(child, pos);
+                step = bits_count(f.w);
+            }
+            s0 += f.x;
+            s1 += f.y;
+            s2 += f.z;
+            pos += step;
+        }
     }
     p[0] = s0 * T(0.125), p[1] = s1 * T(0.125), p[2] = s2 * T(0.125), p[3] = count_bits(pos - a, T(0));
 }
 
-// Level Lc of the pyramid: cell c holds leaves [pmap[c], pmap[c+1]); one leaf covers it when
-// that range has at most one leaf.
+// Level Lc of the pyramid: the covering leaf's value, or the mean of the 8 children.
 template <typename T>
-__device__ __forceinline__ void base_mean(const uint32_t* __restrict__ pmap, const uint8_t* __restrict__ level, int n,
-                                          int Lc, const T* __restrict__ field, const T* __restrict__ child, int64_t c,
-                                          T* __restrict__ out) {
+__device__ __forceinline__ void base_mean(const TreeView& t, int Lc, const T* __restrict__ field,
+                                          const T* __restrict__ child, int64_t c, T* __restrict__ out) {
     using V = Vec4<T>;
-    const int64_t ncell = (int64_t)1 << (3 * Lc);
-    const int a = (int)pmap[c];
-    const int e = c + 1 < ncell ? (int)pmap[c + 1] : n;
+    const uint64_t anchor = (uint64_t)c * key_span(Lc);
+    int lv;
+    const int a = search_plain(t, anchor, lv);
     T* p = out + 4 * c;
-    if (e - a <= 1) {
+    if (lv <= Lc) {
         const auto f = V::load(field, a);
         p[0] = f.x, p[1] = f.y, p[2] = f.z, p[3] = T(0);
     } else {
-        children_mean<T>(level, Lc, field, child, a, p);
+        children_mean<T>(t, Lc, field, child, a, p);
     }
 }
 
 // need (nullable): only the cells flagged there
 template <typename T>
-__global__ void __launch_bounds__(256) k_pyr_base(const uint32_t* __restrict__ pmap, const uint8_t* __restrict__ level,
-                                                  int n, int Lc, const T* __restrict__ field,
+__global__ void __launch_bounds__(256) k_pyr_base(TreeView t, int Lc, const T* __restrict__ field,
                                                   const T* __restrict__ child, T* __restrict__ out,
                                                   const uint8_t* __restrict__ need) {
     const int64_t ncell = (int64_t)1 << (3 * Lc);
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x)
-        if (!need || need[c]) base_mean<T>(pmap, level, n, Lc, field, child, c, out);
+        if (!need || need[c]) base_mean<T>(t, Lc, field, child, c, out);
 }
 
 // Refined cells of level l listed in nodes[0, cnt): their means, at index first leaf (need,
 // nullable: only the cells flagged there, by first leaf).
 template <typename T>
-__global__ void __launch_bounds__(256) k_node_means(const int* __restrict__ nodes, int64_t cnt,
-                                                    const uint8_t* __restrict__ level, int l,
+__global__ void __launch_bounds__(256) k_node_means(TreeView t, const int* __restrict__ nodes, int64_t cnt, int l,
                                                     const T* __restrict__ field, const T* __restrict__ child,
                                                     T* __restrict__ out, const uint8_t* __restrict__ need) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
         const int a = nodes[i];
-        if (!need || need[a]) children_mean<T>(level, l, field, child, a, out + 4 * (int64_t)a);
+        if (!need || need[a]) children_mean<T>(t, l, field, child, a, out + 4 * (int64_t)a);
     }
 }
 
@@ -115,6 +124,28 @@ __global__ void __launch_bounds__(256) k_pyr_up(const T* __restrict__ fine, T* _
                                                 const uint8_t* __restrict__ need) {
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x)
         if (!need || need[c]) up_mean<T>(fine, coarse, c);
+}
+
+// The levels from TOP_LEVEL (512 cells) up in one block and one launch: they take less than a launch each.
+constexpr int TOP_LEVEL = 3;
+template <typename T>
+__global__ void __launch_bounds__(1024) k_pyr_top(T* pyr, int top, const uint8_t* __restrict__ need) {
+    for (int l = top; l >= 0; --l) {
+        const long long o = pyr_offset(l), fine = pyr_offset(l + 1);
+        for (int c = threadIdx.x; c < 1 << (3 * l); c += blockDim.x) {
+            if (need && !need[o + c]) continue;
+            // (plain loads: the level below was written by this block)
+            const T* f = pyr + 4 * (fine + 8 * (long long)c);
+            T s[3] = {T(0), T(0), T(0)};
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) s[d] += f[4 * k + d];
+            T* p = pyr + 4 * (o + c);
+            p[0] = s[0] * T(0.125), p[1] = s[1] * T(0.125), p[2] = s[2] * T(0.125), p[3] = T(0);
+        }
+        __syncthreads();
+    }
 }
 
 // ---- the cell means the level-mate table reads, closed under "a mean needs its children's" ----
@@ -228,7 +259,7 @@ size_t need_flag_bytes(const ot_octree* t) {
 // means array, dense pyramid then node levels, set by the table builder) under "a mean needs
 // its children's"; the octree keeps them, and every later pyramid computes the flagged means
 // only.
-ot_status close_need_flags(ot_octree* t, uint8_t* need, cudaStream_t s) {
+ot_status close_need_flags(const ot_octree* t, uint8_t* need, cudaStream_t s) {
     const int Lc = t->pyr_level;
     const int nl = node_levels(t);
     const int n = (int)t->n;
@@ -254,39 +285,43 @@ ot_status close_need_flags(ot_octree* t, uint8_t* need, cudaStream_t s) {
 }
 
 template <typename T>
-ot_status launch_pyramid(const ot_octree* t, const T* field, T* pyr, cudaStream_t s) {
+ot_status launch_pyramid(const ot_octree* t, const T* field, T* pyr, const uint8_t* need, cudaStream_t s) {
     const int Lc = t->pyr_level;
     const int nl = node_levels(t);
+    const TreeView v = tree_view(t);
     T* nodes = pyr + 4 * pyramid_offset(Lc + 1);
-    // with the level-mate table, only the means it reads and the ones they are made of
-    const uint8_t* need = t->d_need_flags;
     // node means, deepest level first (each reads the next level's)
     for (int k = nl - 1; k >= 0; --k) {
         T* out = nodes + 4 * (int64_t)k * t->n;
         const T* child = k + 1 < nl ? out + 4 * (int64_t)t->n : nullptr;
         if (t->node_cnt[k] > 0) {
             const uint8_t* nk = need ? need + pyramid_offset(Lc + 1) + (int64_t)k * t->n : nullptr;
-            k_node_means<T><<<grid_n(t->node_cnt[k], 256), 256, 0, s>>>(t->d_nodes + t->node_off[k], t->node_cnt[k],
-                                                                       t->d_level, Lc + 1 + k, field, child, out, nk);
+            k_node_means<T><<<grid_n(t->node_cnt[k], 256), 256, 0, s>>>(v, t->d_nodes + t->node_off[k], t->node_cnt[k],
+                                                                       Lc + 1 + k, field, child, out, nk);
             count_launch();
         }
     }
     const int64_t ncell = (int64_t)1 << (3 * Lc);
-    k_pyr_base<T><<<grid_n(ncell, 256), 256, 0, s>>>(t->d_pmap, t->d_level, (int)t->n, Lc, field,
-                                                    nl > 0 ? nodes : nullptr, pyr + 4 * pyramid_offset(Lc),
+    k_pyr_base<T><<<grid_n(ncell, 256), 256, 0, s>>>(v, Lc, field, nl > 0 ? nodes : nullptr,
+                                                    pyr + 4 * pyramid_offset(Lc),
                                                     need ? need + pyramid_offset(Lc) : nullptr);
     count_launch();
-    for (int l = Lc - 1; l >= 0; --l) {
+    int l = Lc - 1;
+    for (; l > TOP_LEVEL; --l) {
         const int64_t nc = (int64_t)1 << (3 * l);
         k_pyr_up<T><<<grid_n(nc, 256), 256, 0, s>>>(pyr + 4 * pyramid_offset(l + 1), pyr + 4 * pyramid_offset(l), nc,
                                                     need ? need + pyramid_offset(l) : nullptr);
+        count_launch();
+    }
+    if (l >= 0) {
+        k_pyr_top<T><<<1, 1024, 0, s>>>(pyr, l, need);
         count_launch();
     }
     OT_CUDA(cudaGetLastError());
     return OT_OK;
 }
 
-template ot_status launch_pyramid<float>(const ot_octree*, const float*, float*, cudaStream_t);
-template ot_status launch_pyramid<double>(const ot_octree*, const double*, double*, cudaStream_t);
+template ot_status launch_pyramid<float>(const ot_octree*, const float*, float*, const uint8_t*, cudaStream_t);
+template ot_status launch_pyramid<double>(const ot_octree*, const double*, double*, const uint8_t*, cudaStream_t);
 
 } // namespace ot

@@ -222,48 +222,43 @@ __device__ __forceinline__ void tri_sum(const T f[3][2], const T v[8][3], T out[
     out[2] = acc2;
 }
 
-// Trilinear interpolation at one point per lane (warp-wide call; Sec. 2.3.2 with the
-// level-mate rule):
-//   host leaf of level l, cell c; t_d = offset from the cell centre; s_d = +1 if t_d >= 0;
-//   level-mates c + {0, s_d}; weights prod (1 - |t_d|) or |t_d|;
-//   level-mate value: leaf of level l -> its value; inside a coarser leaf -> that leaf's
-//   value; refined -> volume-weighted mean of its leaves, one load: from the dense pyramid of
-//   cell means for l <= the pyramid level, else from the node means of level l (both in pyr);
-//   outside the cube -> the host's index on that axis, or the wrapped index when periodic.
-// Lanes with active == false take part in the warp's steps only.  host_in >= 0 gives the host.
-// Returns the host leaf (-1 when inactive or outside the cube, out = NaN).
-template <typename T, bool LEARNED>
-__device__ __forceinline__ int trilinear_queued(const TreeView& t, const RootModel& root, const T* __restrict__ field,
-                                                const T* __restrict__ pyr, WarpQueue& w, bool active, double x,
-                                                double y, double z, int host_in, T out[3]) {
-    using V = Vec4<T>;
-    const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
-    uint64_t X[3] = {0, 0, 0};
-    const bool ok = active && fixpoint3(x, y, z, X);
-    if (active && !ok) atomicOr(t.err, (unsigned)OT_DEV_OUTSIDE);
+// A point's host leaf and level-mates (Sec. 2.3.2 with the level-mate rule): host leaf of level l, cell
+// c; t_d = offset from the cell centre; s_d = +1 if t_d >= 0; level-mates c + {0, s_d}; outside the
+// cube the host's index on that axis, or the wrapped index when periodic.
+template <typename T>
+struct TriCorners {
+    int h, l;         // host leaf and its level
+    T f[3][2];        // weights per axis, lower and upper cell
+    uint64_t anc[8];  // anchors of the level-mates, by position
+    int a[8], lvl[8]; // the leaf that holds each anchor and its level (above l: the level-mate is refined)
+    // Entry of the cell means (in values of 4) of refined corner k.
+    __device__ __forceinline__ long long mean(const TreeView& t, int k) const {
+        if (l <= t.pyr_level) return pyr_offset(l) + (long long)(anc[k] >> (3 * (MAXLEVEL - l)));
+        return pyr_offset(t.pyr_level + 1) + (long long)(l - t.pyr_level - 1) * t.n + a[k];
+    }
+};
 
+// Resolves the corners of one point per lane (warp-wide call); ok: the lane has a point inside the
+// cube, with fixed-point coordinates X.  host_in >= 0 gives the host.
+template <typename T, bool LEARNED>
+__device__ __forceinline__ void tri_corners(const TreeView& t, const RootModel& root, WarpQueue& w, bool ok,
+                                            const uint64_t X[3], int host_in, TriCorners<T>& c8) {
+    const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
     // host (and its level, when the lookup gives it)
     int h = host_in, hl = -1;
     host_queued<LEARNED>(t, root, w, ok, X, h, hl);
     if (!ok) h = 0, hl = -1;  // keeps the lane's reads in bounds; its result is discarded
-
     const int l = hl >= 0 ? hl : (int)t.level[h];
+    c8.h = h, c8.l = l;
     const int ncell = 1 << l;
     int c[3];
-    T f[3][2];
-    const int oct = tri_octant<T>(X, l, f);
+    const int oct = tri_octant<T>(X, l, c8.f);
 #pragma unroll
     for (int d = 0; d < 3; ++d) c[d] = (int)fix_cell(X[d], l);
     const int sh = MAXLEVEL - l;
-    // The level-mates are resolved in stages, each issuing its loads for all 8 corners at once
-    // (independent loads in flight together instead of one dependent chain per corner).
-    // Stage 1: anchors and weights.
-    uint64_t anc[8];
-    T wt[8];
-    int a[8];
-    unsigned self_m = 0u;
     // per axis the lower and the upper level-mate index (the host's, and the neighbour's clamped
     // into the cube) and their Morton bits: each corner's anchor is the OR of three of these six
+    unsigned self_m = 0u;
     int ix[3][2];
     uint64_t dil[3][2];
 #pragma unroll
@@ -277,80 +272,71 @@ __device__ __forceinline__ int trilinear_queued(const TreeView& t, const RootMod
         for (int k = 0; k < 2; ++k) dil[d][k] = (part1by2((uint32_t)ix[d][k]) << d) << (3 * sh);
     }
 #pragma unroll
-    for (int corner = 0; corner < 8; ++corner) {
-        T wc = T(1);
-        bool self = true;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int v = ix[d][(corner >> d) & 1];
-            self = self && (v == c[d]);
-            wc *= f[d][(corner >> d) & 1];
-        }
-        wt[corner] = wc;
-        anc[corner] = dil[0][corner & 1] | dil[1][(corner >> 1) & 1] | dil[2][(corner >> 2) & 1];
-        a[corner] = h;
-        if (self) self_m |= 1u << corner;
+    for (int k = 0; k < 8; ++k) {
+        c8.anc[k] = dil[0][k & 1] | dil[1][(k >> 1) & 1] | dil[2][k >> 2];
+        if (ix[0][k & 1] == c[0] && ix[1][(k >> 1) & 1] == c[1] && ix[2][k >> 2] == c[2]) self_m |= 1u << k;
     }
     if (!ok) self_m = 0xffu;
-    // Stage 2: the level-map lookups of the other corners, each one descriptor load and most with the
-    // answer and its level; stage 3: the rest become tasks of the warp's list.
-    int lvl[8];
+    // the level-map lookups of the other corners, each one descriptor load and most with the answer and
+    // its level; the rest become tasks of the warp's list
     unsigned pend_m = 0u;
     int ca[8], ce[8];
 #pragma unroll
-    for (int corner = 0; corner < 8; ++corner) {
-        ca[corner] = ce[corner] = 0;
-        lvl[corner] = l;
-        if ((self_m >> corner) & 1u) continue;
-        if (map_lookup<false>(t, anc[corner], ca[corner], ce[corner], lvl[corner]))
-            a[corner] = ca[corner];
+    for (int k = 0; k < 8; ++k) {
+        ca[k] = ce[k] = 0;
+        c8.a[k] = h;
+        c8.lvl[k] = l;
+        if ((self_m >> k) & 1u) continue;
+        if (map_lookup<false>(t, c8.anc[k], ca[k], ce[k], c8.lvl[k]))
+            c8.a[k] = ca[k];
         else
-            pend_m |= 1u << corner;
+            pend_m |= 1u << k;
     }
     if (__any_sync(FULL, pend_m != 0u)) {
         int n = 0;
         int tix[8];
 #pragma unroll
-        for (int corner = 0; corner < 8; ++corner)
-            tix[corner] = push_task(w, n, (pend_m >> corner) & 1u, anc[corner], ca[corner], ce[corner] - ca[corner], lt);
+        for (int k = 0; k < 8; ++k) tix[k] = push_task(w, n, (pend_m >> k) & 1u, c8.anc[k], ca[k], ce[k] - ca[k], lt);
         run_tasks<LEARNED>(t, root, w, n, lt);
 #pragma unroll
-        for (int corner = 0; corner < 8; ++corner)
-            if (tix[corner] >= 0) {
-                a[corner] = w.lo[tix[corner]];
-                lvl[corner] = (int)t.level[a[corner]];
+        for (int k = 0; k < 8; ++k)
+            if (tix[k] >= 0) {
+                c8.a[k] = w.lo[tix[k]];
+                c8.lvl[k] = (int)t.level[c8.a[k]];
             }
         __syncwarp();
     }
+}
+
+// Trilinear interpolation at one point per lane (warp-wide call; Sec. 2.3.2): level-mate value: leaf of
+// level l -> its value; inside a coarser leaf -> that leaf's value; refined -> volume-weighted mean of
+// its leaves, one load: from the dense pyramid of cell means for l <= the pyramid level, else from
+// the node means of level l (both in pyr).
+// Lanes with active == false take part in the warp's steps only.  host_in >= 0 gives the host.
+// Returns the host leaf (-1 when inactive or outside the cube, out = NaN).
+template <typename T, bool LEARNED>
+__device__ __forceinline__ int trilinear_queued(const TreeView& t, const RootModel& root, const T* __restrict__ field,
+                                                const T* __restrict__ pyr, WarpQueue& w, bool active, double x,
+                                                double y, double z, int host_in, T out[3]) {
+    using V = Vec4<T>;
+    uint64_t X[3] = {0, 0, 0};
+    const bool ok = active && fixpoint3(x, y, z, X);
+    if (active && !ok) atomicOr(t.err, (unsigned)OT_DEV_OUTSIDE);
+    TriCorners<T> c8;
+    tri_corners<T, LEARNED>(t, root, w, ok, X, host_in, c8);
     if (!ok) {
         out[0] = out[1] = out[2] = qnan<T>();
         return -1;
     }
-    // Stage 4: the values.
-    // a refined level-mate: the pyramid cell (l <= pyramid level) or the node mean of level l
-    // indexed by its first leaf
-    const bool in_pyr = l <= t.pyr_level;
-    const T* rbase = in_pyr ? pyr + 4 * pyr_offset(l) : pyr + 4 * (pyr_offset(t.pyr_level + 1) +
-                                                               (long long)(l - t.pyr_level - 1) * t.n);
     T v[8][3];
 #pragma unroll
-    for (int corner = 0; corner < 8; ++corner) {
-        const bool refined = lvl[corner] > l;
-        const long long ri = in_pyr ? (long long)(anc[corner] >> (3 * sh)) : (long long)a[corner];
-        const auto fv = V::load(refined ? rbase : field, refined ? ri : (long long)a[corner]);
-        v[corner][0] = fv.x, v[corner][1] = fv.y, v[corner][2] = fv.z;
+    for (int k = 0; k < 8; ++k) {
+        const bool refined = c8.lvl[k] > c8.l;
+        const auto fv = V::load(refined ? pyr : field, refined ? c8.mean(t, k) : (long long)c8.a[k]);
+        v[k][0] = fv.x, v[k][1] = fv.y, v[k][2] = fv.z;
     }
-    T acc0 = T(0), acc1 = T(0), acc2 = T(0);
-#pragma unroll
-    for (int corner = 0; corner < 8; ++corner) {
-        acc0 += wt[corner] * v[corner][0];
-        acc1 += wt[corner] * v[corner][1];
-        acc2 += wt[corner] * v[corner][2];
-    }
-    out[0] = acc0;
-    out[1] = acc1;
-    out[2] = acc2;
-    return h;
+    tri_sum<T>(c8.f, v, out);
+    return c8.h;
 }
 
 // The same interpolation with the level-mates read from the octree's level-mate table (built
