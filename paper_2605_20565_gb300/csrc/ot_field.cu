@@ -9,6 +9,7 @@
 #include <cmath>
 
 #include "ot_internal.h"
+#include "ot_sum.cuh"
 
 namespace ot {
 
@@ -70,22 +71,6 @@ __global__ void __launch_bounds__(256) k_field_fourier(const uint64_t* __restric
 // floats cannot take exactly are added in FP64 at once.  17.3M leaves 197 -> 61 us (the finishing block
 // 32 -> 4 us).
 constexpr int MT = 256;
-
-// Sum of floats without rounding to one: the error of each addition (Knuth's two-sum) is carried to
-// the next float.
-struct Sum3 {
-    float a = 0.0f, b = 0.0f, c = 0.0f;
-    __device__ __forceinline__ static float two_sum(float& s, float v) {
-        const float t = __fadd_rn(s, v), u = __fsub_rn(t, s);
-        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, u)), __fsub_rn(v, u));
-        s = t;
-        return e;
-    }
-    __device__ __forceinline__ void add(float v) { c = __fadd_rn(c, two_sum(b, two_sum(a, v))); }
-    __device__ __forceinline__ double value() const { return ((double)c + (double)b) + (double)a; }
-};
-// v 8^-l is exact in FP32 and far from overflow: v is zero or 2^-60 <= |v| < 2^74.
-__device__ __forceinline__ bool plain(float v) { return v == 0.0f || ((__float_as_uint(v) >> 23) & 0xFFu) - 67u < 134u; }
 
 __global__ void __launch_bounds__(MT) k_field_sum(const uint8_t* __restrict__ level, int64_t n,
                                                   const float4* __restrict__ f, double* __restrict__ part) {

@@ -16,8 +16,8 @@ def env():
     import __graft_entry__
     __graft_entry__.build()
     import paper_2605_20565_gb300 as ot
-    # 3.7M leaves of levels 3 to 10: refined level-mates in the dense pyramid and on two node levels
-    tree = ot.ot_octree_build(np.array([[0.42, 0.55, 0.5, 0.1, 0.0035], [0.8, 0.2, 0.7, 0.02, 0.004]]), 3, 10)
+    # about 6M leaves of levels 3 to 10: refined level-mates in the dense pyramid and on two node levels
+    tree = ot.ot_octree_build(np.array([[0.42, 0.55, 0.5, 0.2, 0.0035], [0.8, 0.2, 0.7, 0.02, 0.004]]), 3, 10)
     assert ot.ot_octree_info(tree)[0] > 3_000_000
     return torch, ot, tree
 
@@ -31,7 +31,7 @@ def test_same_bits_as_all_means(env, n, given, fp64):
     rng = np.random.default_rng(n)
     c = np.array([[0.42], [0.55], [0.5]])
     d = rng.normal(size=(3, n))
-    P = c + d / np.linalg.norm(d, axis=0) * 0.1 * (1.0 + rng.normal(size=n) * 0.1)  # across the shell's steps
+    P = c + d / np.linalg.norm(d, axis=0) * 0.2 * (1.0 + rng.normal(size=n) * 0.1)  # across the shell's steps
     P[:, ::5] = rng.random((3, P[:, ::5].shape[1]))
     P[0, 7::50] = 1.5
     more = rng.random((3, N // 8))
