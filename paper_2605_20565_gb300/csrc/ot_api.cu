@@ -47,11 +47,16 @@ __device__ __forceinline__ double add_displacement(double x, float d) {
     return x + (double)d;
 }
 
+// Whether f_p / tau is a normal number for every f_p (1 to 2^87 for finite arguments): one division per
+// particle then (ONE), else one per component.
+bool one_division(float tau) { return tau >= 0x1p-40f && tau <= 0x1p60f; }
+
 // AB2 step of point-particle velocity and position, FP32 state, FP64 positions: one component.
-__device__ __forceinline__ void advect_one(double& x, float& v, float& ap, float& vp, float rel, float rate, float dt,
-                                           int first, int periodic) {
+template <bool ONE>
+__device__ __forceinline__ void advect_one(double& x, float& v, float& ap, float& vp, float rel, float rate, float tau,
+                                           float dt, int first, int periodic) {
     const float vn = v;
-    const float an = rate * rel;
+    const float an = ONE ? rate * rel : rate * rel / tau;
     const float am = first ? an : ap;
     const float vm = first ? vn : vp;
     v = vn + dt * (1.5f * an - 0.5f * am);
@@ -68,18 +73,20 @@ __device__ __forceinline__ void advect_one(double& x, float& v, float& ap, float
     ap = an;
     vp = vn;
 }
-// f_p / tau of the Schiller-Naumann drag: one division per particle.
+// f_p / tau of the Schiller-Naumann drag (f_p alone without ONE).
+template <bool ONE>
 __device__ __forceinline__ float drag_rate(const float rel[3], float tau, float re_coef) {
     float mag2 = 0.0f;
 #pragma unroll
     for (int d = 0; d < 3; ++d) mag2 += rel[d] * rel[d];
     float fp = 1.0f;
     if (re_coef > 0.0f) fp = 1.0f + 0.15f * powf(re_coef * sqrtf(mag2), 0.687f);
-    return fp / tau;
+    return ONE ? fp / tau : fp;
 }
 
 // Any count and alignment: a thread's two particles, a block apart, loaded before either is advanced
 // (20,000,001 particles 738 -> 466 us).
+template <bool ONE>
 __global__ void __launch_bounds__(256) k_advect(double* __restrict__ x, float* __restrict__ v, float* __restrict__ ap,
                                                 float* __restrict__ vp, const float* __restrict__ u, int64_t n,
                                                 float tau, float re_coef, float dt, int first, int periodic) {
@@ -103,10 +110,10 @@ __global__ void __launch_bounds__(256) k_advect(double* __restrict__ x, float* _
             float rel[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) rel[d] = uu[r][d] - vv[r][d];
-            const float rate = drag_rate(rel, tau, re_coef);
+            const float rate = drag_rate<ONE>(rel, tau, re_coef);
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                advect_one(xx[r][d], vv[r][d], aa[r][d], pp[r][d], rel[d], rate, dt, first, periodic);
+                advect_one<ONE>(xx[r][d], vv[r][d], aa[r][d], pp[r][d], rel[d], rate, tau, dt, first, periodic);
                 x[d * n + i] = xx[r][d], v[d * n + i] = vv[r][d], ap[d * n + i] = aa[r][d], vp[d * n + i] = pp[r][d];
             }
         }
@@ -116,6 +123,7 @@ __global__ void __launch_bounds__(256) k_advect(double* __restrict__ x, float* _
 // The same step for 4 consecutive particles per thread with 16-byte loads and stores (every
 // component plane 16-byte aligned: n % 4 == 0 and aligned bases); identical arithmetic.  With the
 // positions' additions off the FP64 pipe: 200M particles 5.62 -> 4.20 ms (6.29 TB/s of the 26.4 GB).
+template <bool ONE>
 __global__ void __launch_bounds__(256) k_advect4(double* __restrict__ x, float* __restrict__ v,
                                                  float* __restrict__ ap, float* __restrict__ vp,
                                                  const float* __restrict__ u, int64_t n, float tau, float re_coef,
@@ -144,11 +152,11 @@ __global__ void __launch_bounds__(256) k_advect4(double* __restrict__ x, float* 
             float rel[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) rel[d] = uf[d][j] - vf[d][j];
-            const float rate = drag_rate(rel, tau, re_coef);
+            const float rate = drag_rate<ONE>(rel, tau, re_coef);
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 double& xr = j < 2 ? (j == 0 ? xx[d][0].x : xx[d][0].y) : (j == 2 ? xx[d][1].x : xx[d][1].y);
-                advect_one(xr, vf[d][j], af[d][j], pf[d][j], rel[d], rate, dt, first, periodic);
+                advect_one<ONE>(xr, vf[d][j], af[d][j], pf[d][j], rel[d], rate, tau, dt, first, periodic);
             }
         }
 #pragma unroll
@@ -452,12 +460,12 @@ ot_status ot_advect_ab2(double* x, float* v, float* ap, float* vp, const float* 
                          ((uintptr_t)ap & 15) == 0 && ((uintptr_t)vp & 15) == 0 && ((uintptr_t)u & 15) == 0;
     if (aligned) {
         const int64_t g = std::min<int64_t>((n / 4 + 255) / 256, (int64_t)num_sms() * 8);
-        k_advect4<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, v, ap, vp, u, n, tau, re_coef, dt, first,
-                                                                 periodic);
+        auto k = one_division(tau) ? k_advect4<true> : k_advect4<false>;
+        k<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, v, ap, vp, u, n, tau, re_coef, dt, first, periodic);
     } else {
         const int64_t g = std::min<int64_t>((n + 511) / 512, (int64_t)num_sms() * 8);
-        k_advect<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, v, ap, vp, u, n, tau, re_coef, dt, first,
-                                                                periodic);
+        auto k = one_division(tau) ? k_advect<true> : k_advect<false>;
+        k<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, v, ap, vp, u, n, tau, re_coef, dt, first, periodic);
     }
     count_launch();
     OT_CUDA(cudaGetLastError());

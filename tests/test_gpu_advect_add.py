@@ -45,3 +45,23 @@ def test_positions_add_as_fp64(n):
     assert use.mean() > 0.7 or n < 10
     assert np.array_equal(got[use].view(np.int64)[~np.isnan(ref[use])], ref[use].view(np.int64)[~np.isnan(ref[use])])
     assert np.all(np.isnan(got[use][np.isnan(ref[use])]))
+
+
+@pytest.mark.parametrize("n", [400, 401])
+@pytest.mark.parametrize("tau", [1e-39, 2.0 ** -40, 1e-12, 1.0, 2.0 ** 60, 1e19, 1e38])
+def test_relaxation_times(tau, n):
+    """One division per particle where f_p / tau is a normal number, else one per component: rel / tau
+    to two roundings (2^-22), and 0 where rel is 0."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2605_20565_gb300 as ot
+    rng = np.random.default_rng(n)
+    U = (rng.normal(size=(3, n)) * (1e-6 if tau < 1e-20 else 1e6)).astype(np.float32)
+    U[:, ::3] = 0.0
+    x = torch.zeros((3, n), dtype=torch.float64, device="cuda")
+    v = torch.zeros((3, n), device="cuda")
+    ap = torch.zeros_like(v)
+    ot.ot_advect_ab2(x, v, ap, torch.zeros_like(v), torch.as_tensor(U, device="cuda"), tau, 0.0, 0.0, first=True)
+    ref = U.astype(np.float64) / float(np.float32(tau))
+    assert np.all(np.abs(ap.cpu().numpy() - ref) <= np.abs(ref) * 2.0 ** -22)
