@@ -332,7 +332,7 @@ ot_status ot_octree_centres(const ot_octree* t, double* d_xyz, void* stream) {
 ot_status ot_octree_destroy(ot_octree* t) {
     if (!t) return OT_OK;
     // pool memory is handed out again without a wait: the work that reads it has to be done
-    cudaDeviceSynchronize();
+    wait_device(t->device);
     if (t->d_key) cudaFree(t->d_key);
     if (t->d_level) cudaFree(t->d_level);
     if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);

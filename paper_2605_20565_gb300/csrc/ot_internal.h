@@ -71,6 +71,7 @@ int blocks_per_sm(const void* fn, int block, size_t smem);
 // with cudaFree once no work uses it.  pool_octree: an octree was made on (1) or left (-1) dev.
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s);
 void pool_octree(int dev, int change);
+void wait_device(int dev);  // until the device's work is done, whichever device is current
 
 TreeView tree_view(const ot_octree* t);
 

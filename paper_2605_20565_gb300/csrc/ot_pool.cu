@@ -67,6 +67,14 @@ void pool_octree(int dev, int change) {
     if (change < 0 && q.octrees == 0 && q.pool) cudaMemPoolTrimTo(q.pool, 0);
 }
 
+void wait_device(int dev) {
+    int cur = dev;
+    cudaGetDevice(&cur);
+    if (cur != dev) cudaSetDevice(dev);
+    cudaDeviceSynchronize();
+    if (cur != dev) cudaSetDevice(cur);
+}
+
 int num_sms() {
     static std::mutex mu;
     static int sms[MAX_DEVICES] = {};
@@ -95,8 +103,11 @@ int blocks_per_sm(const void* fn, int block, size_t smem) {
     }
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, smem) != cudaSuccess || per_sm < 1) return 1;
-    std::lock_guard<std::mutex> lock(mu);
-    known[key] = per_sm;
+    try {
+        std::lock_guard<std::mutex> lock(mu);
+        known[key] = per_sm;
+    } catch (...) {  // no memory to keep it: asked for again
+    }
     return per_sm;
 }
 
