@@ -119,8 +119,8 @@ ot_status ot_octree_copy_leaves(const ot_octree* t, uint64_t* d_keys, uint8_t* d
 /* Level of the level map that every host search starts from (0 .. 8, capped at lmax): for
  * each cell of that level the map holds the leaf at the cell's anchor, so a point in a cell
  * covered by one leaf is located with one table read, and any other point is searched only
- * among its cell's leaves.  8^level * 4 bytes of device memory.  Octrees are created with
- * min(lmax, 7), or 8 when lmax > 10 (a level-map cell's subtree descriptor resolves leaves up
+ * among its cell's leaves.  8^level * 20 bytes of device memory (the map and the cells' subtree
+ * descriptors).  Octrees are created with min(lmax, 7), or 8 when lmax > 10 (a level-map cell's subtree descriptor resolves leaves up
  * to 3 levels below it).  Synchronises the stream. */
 ot_status ot_octree_set_map_level(ot_octree* t, int level, void* stream);
 /* The current level-map level. */
@@ -348,7 +348,8 @@ ot_status ot_ibm_mdf(const ot_octree* t, int kernel, const double* d_x, const do
  * against the text and omit rho_f); with v = F_k at the surface markers and scale = -1: the
  * IBM force -sum F_k dV_k and torque -sum (X_k - x_b) x F_k dV_k.  The markers of body b are
  * d_start[b] .. d_start[b+1]-1 (device int64, n_bodies + 1 entries); d_xb: n_bodies x 3 body
- * centres; d_lin, d_ang: n_bodies x 3 doubles.  FP64 sums in a fixed order (deterministic).
+ * centres; d_lin, d_ang: n_bodies x 3 doubles.  Sums of FP64's precision or better, in a fixed
+ * order (deterministic).
  * -------------------------------------------------------------------------------------*/
 ot_status ot_body_sums(const double* d_x, const double* d_y, const double* d_z, const float* d_v, const float* d_dV,
                        float w, int64_t n, const int64_t* d_start, int n_bodies, const double* d_xb, double scale,
@@ -392,12 +393,14 @@ typedef struct {
     int tri_records;   /* with the level-mate table: 0 (default): value records for the hot
                           leaves -- the leaves of level <= min(level-map level, hot level),
                           the hot level being the deepest at which the trilinear points, spread
-                          evenly, would give every leaf at least 4 -- holding for each octant
-                          of the leaf's cell its 8 level-mate values (96 bytes), rewritten from
-                          the field at every replay; a point in a level-map cell inside a hot
-                          leaf reads the cell's 8-byte entry and one record instead of the
-                          level-mate row and 8 scattered values; identical results.  Costs
-                          8 bytes per level-map cell and 768 bytes per hot leaf.  k > 0: the
+                          evenly, would give every leaf at least 4 -- holding for each node
+                          of their levels' grids the 8 values around it (96 bytes), rewritten
+                          from the field at every replay; a point in a level-map cell inside
+                          a hot leaf reads the cell's entry and one record instead of the
+                          level-mate row and 8 scattered values; identical results.  Costs 4
+                          bytes per level-map cell (8 in octrees of 2^28 leaves or more) and
+                          96 (2^l + 1)^3 bytes for each hot level l (1.9 GB at hot level 8,
+                          0.25 GB at 7); without that memory the rows serve.  k > 0: the
                           same with the hot level capped at k (a smaller record set); -1: off */
 } ot_launch;
 
