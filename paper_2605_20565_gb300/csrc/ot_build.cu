@@ -114,49 +114,115 @@ __global__ void k_refine(const uint64_t* __restrict__ parent, int64_t ncand, int
     }
 }
 
-__device__ __forceinline__ bool contains_sorted(const uint64_t* __restrict__ a, int64_t n, uint64_t q, int64_t* at) {
-    int64_t lo = 0, hi = n;
+// A sorted set of keys of one level, with the places of its first keys per bucket of leading bits
+// (tab[b] .. tab[b + 1], null: none).  A search is a chain of dependent loads, some 20 in the sets of
+// a large tree; the table leaves some 7: ranks 114 -> 52 us, balance 410 -> 270 us, the tables 61 us
+// (17.3M leaves).
+struct KeySet {
+    const uint64_t* a;
+    int64_t n;
+    const uint32_t* tab;
+    int sh;
+};
+__device__ __forceinline__ int64_t lower_bound(const uint64_t* __restrict__ a, int64_t lo, int64_t hi, uint64_t q) {
     while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
+        const int64_t mid = (lo + hi) >> 1;
         if (a[mid] < q)
             lo = mid + 1;
         else
             hi = mid;
     }
+    return lo;
+}
+__device__ __forceinline__ bool contains_sorted(const KeySet& s, uint64_t q, int64_t* at) {
+    const uint64_t b = q >> s.sh;
+    const int64_t lo = lower_bound(s.a, s.tab ? s.tab[b] : 0, s.tab ? s.tab[b + 1] : s.n, q);
     if (at) *at = lo;
-    return lo < n && a[lo] == q;
+    return lo < s.n && s.a[lo] == q;
+}
+__global__ void k_buckets(const uint64_t* __restrict__ a, int64_t n, int sh, int64_t nb, uint32_t* __restrict__ tab) {
+    GRID_STRIDE(b, nb + 1) tab[b] = (uint32_t)(b < nb ? lower_bound(a, 0, n, (uint64_t)b << sh) : n);
 }
 
 // Balance requirement of refined cells p of level l: the parents (level l-1) of p's neighbour
-// cells and of p itself must be refined.  Missing ones are appended to `miss`.
-__global__ void k_balance_req(const uint64_t* __restrict__ R, int64_t nR, int l, const uint64_t* __restrict__ Rp,
-                              int64_t nRp, int full, uint64_t* __restrict__ miss, uint32_t* __restrict__ nmiss,
-                              int64_t cap) {
-    const int64_t ncell = (int64_t)1 << l;
-    GRID_STRIDE(j, nR) {
+// cells and of p itself must be refined: its own parent and per axis the next one on the side that p
+// lies at.  Missing ones are appended to `miss`, those of a warp once each (siblings miss
+// the same parents) and those of a block with one addition to their count: the additions, one per key,
+// were most of the rest of its time (17.3M leaves 270 -> 170 us).
+constexpr int BAL_T = 256;
+__global__ void __launch_bounds__(BAL_T) k_balance_req(const uint64_t* __restrict__ R, int64_t nR, int l, KeySet Rp, int full,
+                              uint64_t* __restrict__ miss, uint32_t* __restrict__ nmiss, int64_t cap) {
+    constexpr unsigned FULLM = 0xffffffffu;
+    const uint32_t np = 1u << (l - 1);  // parents per axis
+    __shared__ uint32_t s_cnt[BAL_T / 32], s_at;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t j0 = blockIdx.x * (int64_t)BAL_T; j0 < nR; j0 += (int64_t)gridDim.x * BAL_T) {
+        const int64_t j = j0 + threadIdx.x;
+        const bool in = j < nR;
         uint32_t c[3];
-        demorton3(R[j], c[0], c[1], c[2]);
-        // candidate parent coordinates per axis
-        int64_t plo[3], phi[3];
+        demorton3(in ? R[j] : 0ULL, c[0], c[1], c[2]);
+        uint64_t dil[3][2];
+        unsigned there = 0;  // bit d: axis d has the other parent
+#pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const int64_t a = (int64_t)c[d] - 1, b = (int64_t)c[d] + 1;
-            plo[d] = (a < 0 ? 0 : a) >> 1;
-            phi[d] = (b > ncell - 1 ? ncell - 1 : b) >> 1;
+            const uint32_t own = c[d] >> 1, other = (c[d] & 1u) ? own + 1u : own - 1u;  // (0 - 1 is not below np)
+            if (other < np) there |= 1u << d;
+            dil[d][0] = part1by2(own) << d;
+            dil[d][1] = part1by2(other & (np - 1u)) << d;
         }
-        for (int64_t pz = plo[2]; pz <= phi[2]; ++pz)
-            for (int64_t py = plo[1]; py <= phi[1]; ++py)
-                for (int64_t px = plo[0]; px <= phi[0]; ++px) {
-                    if (!full) {
-                        // face balance: p's own parent, or the parent of a face neighbour
-                        int differ = (px != (c[0] >> 1)) + (py != (c[1] >> 1)) + (pz != (c[2] >> 1));
-                        if (differ > 1) continue;
-                    }
-                    uint64_t key = morton3((uint32_t)px, (uint32_t)py, (uint32_t)pz);
-                    if (!contains_sorted(Rp, nRp, key, nullptr)) {
-                        uint32_t at = atomicAdd(nmiss, 1u);
-                        if (at < cap) miss[at] = key;
-                    }
-                }
+        // the 8 searches step by step together: their loads do not wait for one another
+        uint64_t key[8];
+        uint32_t lo[8], len[8], most = 0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            // face balance: p's own parent, or the parent of a face neighbour
+            const bool want = in && !(e & ~there) && (full || !(e & (e - 1)));
+            key[e] = dil[0][e & 1] | dil[1][(e >> 1) & 1] | dil[2][e >> 2];
+            const uint64_t b = key[e] >> Rp.sh;
+            lo[e] = !want || !Rp.tab ? 0u : Rp.tab[b];
+            len[e] = !want ? 0u : (Rp.tab ? Rp.tab[b + 1] : (uint32_t)Rp.n) - lo[e];
+            if (!want) key[e] = ~0ULL;
+            most = max(most, len[e]);
+        }
+        for (; most > 1u; most -= most >> 1) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const uint32_t half = len[e] >> 1;
+                if (half && Rp.a[lo[e] + half] <= key[e]) lo[e] += half;
+                len[e] -= half;
+            }
+        }
+        uint32_t mine = 0;  // bit e: this lane appends key e
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const bool missing = key[e] != ~0ULL && !(len[e] && Rp.a[lo[e]] == key[e]);
+            if (!__any_sync(FULLM, missing)) continue;
+            const unsigned same = __match_any_sync(FULLM, missing ? key[e] : ~0ULL);
+            if (missing && !(same & ((1u << lane) - 1u))) mine |= 1u << e;
+        }
+        uint32_t incl = (uint32_t)__popc(mine);
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const uint32_t v = __shfl_up_sync(FULLM, incl, k);
+            if (lane >= k) incl += v;
+        }
+        if (lane == 31) s_cnt[warp] = incl;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t all = 0;
+            for (int w = 0; w < BAL_T / 32; ++w) all += s_cnt[w];
+            s_at = all ? atomicAdd(nmiss, all) : 0u;
+        }
+        __syncthreads();
+        uint32_t at = s_at + incl - (uint32_t)__popc(mine);
+        for (int w = 0; w < warp; ++w) at += s_cnt[w];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if ((mine >> e) & 1u) {
+                if (at < cap) miss[at] = key[e];
+                ++at;
+            }
+        __syncthreads();  // s_cnt, s_at
     }
 }
 
@@ -164,11 +230,10 @@ __device__ __forceinline__ uint64_t node_key(const uint64_t* __restrict__ Rparen
     return Rparent ? ((Rparent[j >> 3] << 3) | (uint64_t)(j & 7)) : (uint64_t)j;
 }
 
-__global__ void k_rank(const uint64_t* __restrict__ Rparent, int64_t M, const uint64_t* __restrict__ R, int64_t nR,
-                       int32_t* __restrict__ rank) {
+__global__ void k_rank(const uint64_t* __restrict__ Rparent, int64_t M, KeySet R, int32_t* __restrict__ rank) {
     GRID_STRIDE(j, M) {
         int64_t at;
-        rank[j] = contains_sorted(R, nR, node_key(Rparent, j), &at) ? (int32_t)at : -1;
+        rank[j] = contains_sorted(R, node_key(Rparent, j), &at) ? (int32_t)at : -1;
     }
 }
 
@@ -218,6 +283,19 @@ ot_status dalloc(T** p, int64_t n, cudaStream_t s) {
     if (n <= 0) return OT_OK;
     OT_CUDA(pool_malloc((void**)p, sizeof(T) * (size_t)n, s));
     return OT_OK;
+}
+
+// The set of the n sorted keys a of level l.  A bucket per key at most, tab has room for 2^MAX_BUCKET
+// + 1; few keys go without.
+constexpr int MAX_BUCKET = 18;
+KeySet key_set(const uint64_t* a, int64_t n, int l, uint32_t* tab, cudaStream_t s) {
+    int bits = std::min(3 * l, MAX_BUCKET);
+    while (bits > 0 && ((int64_t)1 << bits) > n) --bits;
+    if (bits < 10) return KeySet{a, n, nullptr, 0};
+    const int64_t nb = (int64_t)1 << bits;
+    k_buckets<<<grid1d(nb + 1, 256), 256, 0, s>>>(a, n, 3 * l - bits, nb, tab);
+    count_launch();
+    return KeySet{a, n, tab, 3 * l - bits};
 }
 
 struct Guard {
@@ -307,6 +385,13 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
         R[l] = out;
     }
 
+    uint32_t* tab = nullptr;  // of the set searched next
+    {
+        const ot_status st = dalloc(&tab, ((int64_t)1 << MAX_BUCKET) + 1, s);
+        if (st != OT_OK) return st;
+    }
+    g.keep(tab);
+
     // 2. balance, finest refined level first
     for (int l = lmax - 1; l >= lmin + 1; --l) {
         if (nR[l] == 0) continue;
@@ -319,8 +404,8 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
         if ((st = dalloc(&nmiss, 1, s)) != OT_OK) return st;
         g.keep(nmiss);
         OT_CUDA(cudaMemsetAsync(nmiss, 0, sizeof(uint32_t), s));
-        k_balance_req<<<grid1d(nR[l], 256), 256, 0, s>>>(R[l], nR[l], l, R[l - 1], nR[l - 1], p->balance_full, miss,
-                                                        nmiss, cap);
+        const KeySet parents = key_set(R[l - 1], nR[l - 1], l - 1, tab, s);
+        k_balance_req<<<grid1d(nR[l], BAL_T), BAL_T, 0, s>>>(R[l], nR[l], l, parents, p->balance_full, miss, nmiss, cap);
         count_launch();
         OT_CUDA(cudaGetLastError());
         uint32_t hm = 0;
@@ -356,7 +441,8 @@ ot_status build_tree(const ot_sphere* h_spheres, int nsph, const ot_build_params
         if (l < lmax) {
             if ((st = dalloc(&rank[l], M[l], s)) != OT_OK) return st;
             g.keep(rank[l]);
-            k_rank<<<grid1d(M[l], 256), 256, 0, s>>>(l == lmin ? nullptr : R[l - 1], M[l], R[l], nR[l], rank[l]);
+            const KeySet refined = key_set(R[l], nR[l], l, tab, s);
+            k_rank<<<grid1d(M[l], 256), 256, 0, s>>>(l == lmin ? nullptr : R[l - 1], M[l], refined, rank[l]);
             count_launch();
         }
         if ((st = dalloc(&cnt[l], M[l], s)) != OT_OK) return st;
