@@ -59,8 +59,9 @@ __device__ bool box_near_surface(const double lo[3], double h, const ot_sphere& 
 
 // The same test in FP32: 1 or -1 when its distance is farther from the shell width than the
 // rounding can have moved it, 0 when the FP64 test has to decide (a few cells in a thousand; the
-// FP64 pipe was most of the refinement's time, 497 -> 154 us for 17.3M leaves).  Rounding: positions, radii and distances carry at most
-// 2^-23 of the magnitudes involved each, some 6 of them; the margin is 4e-6 of their sum.
+// FP64 pipe was most of the refinement's time, 497 -> 154 us for 17.3M leaves).  Rounding: positions,
+// radii and distances carry at most 2^-23 of the magnitudes involved each, some 6 of them; the
+// margin is 4e-6 of their sum.
 __device__ __forceinline__ int near_surface_f32(const float lo[3], float h, const ot_sphere& s) {
     float near2 = 0.0f, far2 = 0.0f, mag = 1.0f;
 #pragma unroll
@@ -80,7 +81,8 @@ __device__ __forceinline__ int near_surface_f32(const float lo[3], float h, cons
 // Candidate cells of level l: the 8^l cells (parent == null, l == lmin) or the children of the
 // refined parents; flag[j] = criterion, cand[j] = key.  With the sphere bins (l >= Lb), only the
 // spheres listed for the cell's bin of level Lb are tested: a bin lists every sphere whose
-// centre is within (r + shell) + margin of it, a superset of those near any cell inside it, so the result is the same as testing every sphere.
+// centre is within (r + shell) + margin of it, a superset of those near any cell inside it, so the
+// result is the same as testing every sphere.
 __global__ void k_refine(const uint64_t* __restrict__ parent, int64_t ncand, int l, const ot_sphere* __restrict__ sph,
                          int nsph, const int* __restrict__ bin_off, const int* __restrict__ bin_sph, int Lb,
                          uint64_t* __restrict__ cand, uint32_t* __restrict__ flag) {

@@ -230,8 +230,8 @@ __device__ __forceinline__ uint32_t bits_of(float v) { return __float_as_uint(v)
 __device__ __forceinline__ uint32_t bits_of(double v) { return (uint32_t)__double_as_longlong(v); }
 constexpr uint32_t OFF_NONE = 0x404040u;  // a marker that reaches no tile
 
-// Records in home-tile order (F null: the forces come later), and the runs: a warp takes 32 consecutive markers, finds the first of
-// each run, its end (for the last one of the warp a 32-ary search over the markers that follow)
+// Records in home-tile order (F null: the forces come later), and the runs: a warp takes 32
+// consecutive markers, finds the first of each run, its end (for the last one of the warp a 32-ary search over the markers that follow)
 // and enters it in the table and the list of runs (whose order does not matter; one atomic
 // per block's 256 markers).
 constexpr int REC_T = 256;
