@@ -281,8 +281,9 @@ ot_status ot_spread_workspace_size(const ot_octree* t, int kernel, int64_t n, si
  *     stencils reach it, in a fixed order of these and in marker order within each:
  *     bit-identical run to run and for any launch shape.
  *     Needs d_workspace of ot_spread_workspace_size bytes (16-byte aligned); nothing is
- *     allocated.
- *   OT_ATOMIC: float atomics; order varies run to run.  d_workspace may be NULL. */
+ *     allocated.  d_f may start at any float.
+ *   OT_ATOMIC: float atomics; order varies run to run.  d_workspace may be NULL; d_f 16-byte
+ *     aligned (four-float atomics). */
 ot_status ot_spread(const ot_octree* t, int kernel, int mode, const double* d_x, const double* d_y,
                     const double* d_z, const float* d_F, const float* d_dV, int64_t n, float* d_f,
                     void* d_workspace, size_t ws_bytes, void* stream);

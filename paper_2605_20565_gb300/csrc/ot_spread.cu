@@ -391,11 +391,16 @@ template <typename T> struct Acc3 {
 __device__ __forceinline__ bool is_finite(float v) { return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u; }
 __device__ __forceinline__ bool is_finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
+// (f may start anywhere, a view into a larger buffer say: wide accesses where it allows them)
 __device__ __forceinline__ void add_leaf(float* f, int leaf, const Acc3<float>& a) {
     float* p = f + 4 * (size_t)leaf;
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    *reinterpret_cast<float2*>(p) = make_float2(v.x + a.x, v.y + a.y);
-    p[2] = v.z + a.z;
+    if (((uintptr_t)f & 15) == 0) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        *reinterpret_cast<float2*>(p) = make_float2(v.x + a.x, v.y + a.y);
+        p[2] = v.z + a.z;
+    } else {
+        p[0] += a.x, p[1] += a.y, p[2] += a.z;
+    }
 }
 __device__ __forceinline__ void add_leaf(double* f, int leaf, const Acc3<double>& a) {
     double* p = f + 4 * (size_t)leaf;
