@@ -120,8 +120,10 @@ ot_status ot_octree_copy_leaves(const ot_octree* t, uint64_t* d_keys, uint8_t* d
  * each cell of that level the map holds the leaf at the cell's anchor, so a point in a cell
  * covered by one leaf is located with one table read, and any other point is searched only
  * among its cell's leaves.  8^level * 20 bytes of device memory (the map and the cells' subtree
- * descriptors).  Octrees are created with min(lmax, 7), or 8 when lmax > 10 (a level-map cell's subtree descriptor resolves leaves up
- * to 3 levels below it).  Synchronises the stream. */
+ * descriptors); a change holds the old and the new ones at once, and without memory for the new
+ * ones (OT_ERR_OOM) the octree keeps its level.  Octrees are created with min(lmax, 7), or 8 when
+ * lmax > 10 (a level-map cell's subtree descriptor resolves leaves up to 3 levels below it).
+ * Synchronises the stream. */
 ot_status ot_octree_set_map_level(ot_octree* t, int level, void* stream);
 /* The current level-map level. */
 ot_status ot_octree_get_map_level(const ot_octree* t, int* level);

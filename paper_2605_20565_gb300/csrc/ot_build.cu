@@ -663,37 +663,42 @@ ot_status finish_tree(ot_octree* t, cudaStream_t s, int map_level) {
         ot_status st = build_node_lists(t, s);
         if (st != OT_OK) return st;
     }
-    // (a change of the map level: work on other streams may still read the old map)
-    if (t->d_lmap || t->d_desc) OT_CUDA(cudaDeviceSynchronize());
-    if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);
-    t->d_lmap = nullptr;
-    if (L == Lp) {
-        t->d_lmap = t->d_pmap;
-    } else {
-        const int64_t ncell = (int64_t)1 << (3 * L);
-        OT_CUDA(pool_malloc((void**)&t->d_lmap, sizeof(uint32_t) * ncell, s));
-        k_lmap<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_key, (int)t->n, L, ncell, t->d_lmap);
+    // the new map beside the old one, which stays in place when there is no memory for another
+    const int64_t ncell = (int64_t)1 << (3 * L);
+    uint32_t* lmap = t->d_pmap;
+    uint4* desc = nullptr;
+    auto fail = [&](cudaError_t e) {
+        if (lmap && lmap != t->d_pmap) cudaFreeAsync(lmap, s);
+        if (desc) cudaFreeAsync(desc, s);
+        return cuda_status(e);
+    };
+    cudaError_t e;
+    if (L != Lp) {
+        if ((e = pool_malloc((void**)&lmap, sizeof(uint32_t) * ncell, s)) != cudaSuccess) return fail(e);
+        k_lmap<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_key, (int)t->n, L, ncell, lmap);
         count_launch();
     }
-    t->lmap_level = L;
-    if (t->d_desc) cudaFree(t->d_desc);
-    t->d_desc = nullptr;
-    const int64_t ncell = (int64_t)1 << (3 * L);
-    OT_CUDA(pool_malloc((void**)&t->d_desc, sizeof(uint4) * ncell, s));
-    k_desc_cells<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_level, (int)t->n, t->d_lmap, ncell, t->d_desc);
+    if ((e = pool_malloc((void**)&desc, sizeof(uint4) * ncell, s)) != cudaSuccess) return fail(e);
+    k_desc_cells<<<grid1d(ncell, 256), 256, 0, s>>>(t->d_level, (int)t->n, lmap, ncell, desc);
     count_launch();
     if (L + 2 <= t->lmax) {
         k_desc_leaves<<<grid1d(t->n, 256), 256, 0, s>>>(t->d_key, t->d_level, (int)t->n, L,
-                                                       reinterpret_cast<uint32_t*>(t->d_desc));
+                                                       reinterpret_cast<uint32_t*>(desc));
         count_launch();
     }
     if (!t->d_err) {
-        OT_CUDA(pool_malloc((void**)&t->d_err, 64, s));
-        OT_CUDA(cudaMemsetAsync(t->d_err, 0, 64, s));
+        if ((e = pool_malloc((void**)&t->d_err, 64, s)) != cudaSuccess) return fail(e);
+        if ((e = cudaMemsetAsync(t->d_err, 0, 64, s)) != cudaSuccess) return fail(e);
         t->d_fallbacks = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(t->d_err) + 8);
     }
-    OT_CUDA(cudaGetLastError());
-    OT_CUDA(cudaStreamSynchronize(s));
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e);
+    // (a change of the map level: work on other streams may still read the old map)
+    if (t->d_desc) wait_device(t->device);
+    if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);
+    if (t->d_desc) cudaFree(t->d_desc);
+    t->d_lmap = lmap;
+    t->d_desc = desc;
+    t->lmap_level = L;
     return OT_OK;
 }
 

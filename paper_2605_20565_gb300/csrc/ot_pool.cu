@@ -56,7 +56,9 @@ cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s) {
         }
         pool = g_pools[dev].pool;
     }
-    return cudaMallocFromPoolAsync(p, bytes, pool, s);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e != cudaSuccess) cudaGetLastError();  // returned here; the next call's launches do not report it again
+    return e;
 }
 
 void pool_octree(int dev, int change) {

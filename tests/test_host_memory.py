@@ -1,0 +1,67 @@
+"""The library's host side against failing allocations, without a GPU: the CUDA runtime's memory calls are
+those of fake_cudart.c (kernels do nothing), preloaded in a child process."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PROLOGUE = """
+import ctypes as C, sys
+fake = C.CDLL(sys.argv[1])
+lib = C.CDLL(sys.argv[2])
+fake.fake_fail_from.argtypes = [C.c_size_t]
+lib.ot_octree_build.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+lib.ot_octree_destroy.argtypes = [C.c_void_p]
+MALLOC, POOL, OOM = 1, 2, -3
+def build(level):
+    h = C.c_void_p()
+    prm = (C.c_int * 3)(level, level, 1)
+    return lib.ot_octree_build(None, 0, prm, None, C.byref(h)), h
+def destroy(h):
+    assert lib.ot_octree_destroy(h) == 0
+def map_level(h):
+    v = C.c_int(-1)
+    assert lib.ot_octree_get_map_level(h, C.byref(v)) == 0
+    return v.value
+"""
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    from paper_2605_20565_gb300 import _build
+    lib = _build.build()
+    fake = str(tmp_path_factory.mktemp("fake") / "fake_cudart.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-w", "-o", fake, os.path.join(HERE, "fake_cudart.c")], check=True)
+
+    def run(script):
+        env = dict(os.environ, LD_PRELOAD=fake)
+        r = subprocess.run([sys.executable, "-c", PROLOGUE + script, fake, lib], env=env, cwd=ROOT, timeout=120,
+                           capture_output=True, text=True)
+        assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
+    return run
+
+
+@pytest.mark.parametrize("level,bytes_", [(1, 1), (1, 8 * 16), (3, 1), (0, 16)])
+def test_a_map_level_without_memory_leaves_the_octree_as_it_was(child, level, bytes_):
+    """Either allocation of ot_octree_set_map_level fails (bytes_: from which size on): the call reports it, the
+    level stays, and nothing that the octree holds was freed; with memory again the same call succeeds."""
+    child(f"""
+st, h = build(3)
+assert st == 0 and map_level(h) == 3
+assert lib.ot_octree_set_map_level(h, 2, None) == 0
+live = fake.fake_live(POOL), fake.fake_live(MALLOC)
+for _ in range(3):
+    fake.fake_fail_from({bytes_})
+    assert lib.ot_octree_set_map_level(h, {level}, None) == OOM
+    assert map_level(h) == 2 and (fake.fake_live(POOL), fake.fake_live(MALLOC)) == live
+fake.fake_fail_from(1 << 62)
+assert lib.ot_octree_set_map_level(h, {level}, None) == 0 and map_level(h) == {level}
+assert lib.ot_octree_set_map_level(h, 2, None) == 0 and map_level(h) == 2
+assert (fake.fake_live(POOL), fake.fake_live(MALLOC)) == live
+destroy(h)
+assert fake.fake_live(POOL) == 0
+""")
