@@ -230,7 +230,7 @@ ot_status ot_octree_build(const ot_sphere* h_spheres, int n, const ot_build_para
     ot_octree* t = new (std::nothrow) ot_octree();
     if (!t) return OT_ERR_OOM;
     cudaGetDevice(&t->device);
-    pool_octree(t->device, 1);
+    t->context = pool_octree_made(t->device);
     cudaStream_t s = (cudaStream_t)stream;
     ot_status st = build_tree(h_spheres, n, p, s, t);
     if (st == OT_OK) st = finish_tree(t, s);
@@ -254,7 +254,7 @@ ot_status ot_octree_from_leaves(const uint64_t* d_keys, const uint8_t* d_levels,
     ot_octree* t = new (std::nothrow) ot_octree();
     if (!t) return OT_ERR_OOM;
     cudaGetDevice(&t->device);
-    pool_octree(t->device, 1);
+    t->context = pool_octree_made(t->device);
     cudaError_t e = pool_malloc((void**)&t->d_key, sizeof(uint64_t) * n, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&t->d_level, n, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(t->d_key, d_keys, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s);
@@ -345,7 +345,7 @@ ot_status ot_octree_destroy(ot_octree* t) {
     if (t->d_mids) cudaFree(t->d_mids);
     if (t->d_root) cudaFree(t->d_root);
     if (t->d_err) cudaFree(t->d_err);
-    pool_octree(t->device, -1);
+    pool_octree_left(t->device, t->context);
     delete t;
     return OT_OK;
 }

@@ -11,6 +11,7 @@
 
 struct ot_octree {
     int device = 0;
+    unsigned long long context = 0;  // that its memory belongs to
     int64_t n = 0;
     int lmin = 0, lmax = 0;
     uint64_t* d_key = nullptr;
@@ -68,9 +69,12 @@ int num_sms();
 int blocks_per_sm(const void* fn, int block, size_t smem);
 
 // Stream-ordered device memory from the library's pool (ot_pool.cu); freed with cudaFreeAsync, or
-// with cudaFree once no work uses it.  pool_octree: an octree was made on (1) or left (-1) dev.
+// with cudaFree once no work uses it.  An octree was made on the current device dev (returns its
+// context); the octree was destroyed.
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s);
-void pool_octree(int dev, int change);
+unsigned long long pool_octree_made(int dev);
+void pool_octree_left(int dev, unsigned long long context);
+unsigned long long current_context_id();
 void wait_device(int dev);  // until the device's work is done, whichever device is current
 
 TreeView tree_view(const ot_octree* t);

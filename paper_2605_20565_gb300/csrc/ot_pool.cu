@@ -8,9 +8,13 @@
 // POOL_KEEP bytes while octrees live on the device and gives everything back when the last one is
 // destroyed.  Memory pools are safe to use from several threads and streams: a block is handed
 // out again only after the work before its release, in stream order.
+#include <cuda.h>  // driver types only: the two driver calls below are reached through the runtime
+
 #include <map>
 #include <mutex>
+#include <new>
 #include <tuple>
+#include <utility>
 
 #include "ot_internal.h"
 
@@ -26,7 +30,9 @@ struct Pool {
     int octrees = 0;
 };
 std::mutex g_pool_mu;
-Pool g_pools[MAX_DEVICES];
+// by device and context: a pool dies with the context that it was made in, and the octrees that
+// were left in it no longer count
+std::map<std::pair<int, unsigned long long>, Pool> g_pools;
 
 cudaError_t create_pool(int dev, cudaMemPool_t* out) {
     cudaMemPoolProps p{};
@@ -39,34 +45,88 @@ cudaError_t create_pool(int dev, cudaMemPool_t* out) {
     return cudaMemPoolSetAttribute(*out, cudaMemPoolAttrReleaseThreshold, &keep);
 }
 
+// The current context's identity, made first if there is none yet.
+unsigned long long made_context() {
+    unsigned long long id = current_context_id();
+    if (id == 0) {
+        cudaFree(nullptr);
+        id = current_context_id();
+    }
+    return id;
+}
+
 } // namespace
+
+// Identity of the current CUDA context (0 when the driver does not say).  A context that was
+// destroyed and created again -- cudaDeviceReset, for instance -- has a new identity; what the
+// library keeps per device (memory pools, the address of its device array) belongs to one.
+unsigned long long current_context_id() {
+    using GetCurrent = CUresult (*)(CUcontext*);
+    using GetId = CUresult (*)(CUcontext, unsigned long long*);
+    static GetCurrent get_current = nullptr;
+    static GetId get_id = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get_current = reinterpret_cast<GetCurrent>(f);
+        f = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get_id = reinterpret_cast<GetId>(f);
+    });
+    CUcontext ctx = nullptr;
+    unsigned long long id = 0;
+    if (get_current && get_id && get_current(&ctx) == CUDA_SUCCESS && ctx && get_id(ctx, &id) == CUDA_SUCCESS)
+        return id;
+    return 0;
+}
 
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s) {
     *p = nullptr;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= MAX_DEVICES) return cudaMallocAsync(p, bytes, s);
+    const unsigned long long context = made_context();
     cudaMemPool_t pool;
-    {
+    try {
         std::lock_guard<std::mutex> lock(g_pool_mu);
-        if (!g_pools[dev].pool && (e = create_pool(dev, &g_pools[dev].pool)) != cudaSuccess) {
-            g_pools[dev].pool = nullptr;
+        Pool& q = g_pools[{dev, context}];
+        if (!q.pool && (e = create_pool(dev, &q.pool)) != cudaSuccess) {
+            q.pool = nullptr;
             return e;
         }
-        pool = g_pools[dev].pool;
+        pool = q.pool;
+    } catch (const std::bad_alloc&) {
+        return cudaErrorMemoryAllocation;
     }
     e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e != cudaSuccess) cudaGetLastError();  // returned here; the next call's launches do not report it again
     return e;
 }
 
-void pool_octree(int dev, int change) {
-    if (dev < 0 || dev >= MAX_DEVICES) return;
+unsigned long long pool_octree_made(int dev) {
+    const unsigned long long context = made_context();
+    try {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        ++g_pools[{dev, context}].octrees;
+    } catch (const std::bad_alloc&) {  // not counted: the pool is given back with the others
+    }
+    return context;
+}
+
+void pool_octree_left(int dev, unsigned long long context) {
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    Pool& q = g_pools[dev];
-    q.octrees += change;
-    if (change < 0 && q.octrees == 0 && q.pool) cudaMemPoolTrimTo(q.pool, 0);
+    const auto it = g_pools.find({dev, context});
+    if (it == g_pools.end() || --it->second.octrees > 0 || !it->second.pool) return;
+    int cur = dev;
+    cudaGetDevice(&cur);
+    if (cur != dev) cudaSetDevice(dev);
+    // (a pool of another context than the device's may no longer exist)
+    if (current_context_id() == context) cudaMemPoolTrimTo(it->second.pool, 0);
+    if (cur != dev) cudaSetDevice(cur);
 }
 
 void wait_device(int dev) {

@@ -65,3 +65,29 @@ assert (fake.fake_live(POOL), fake.fake_live(MALLOC)) == live
 destroy(h)
 assert fake.fake_live(POOL) == 0
 """)
+
+
+@pytest.mark.parametrize("old_first", [False, True])
+def test_pools_end_with_their_context(child, old_first):
+    """Octrees after a context was destroyed and made again (cudaDeviceReset) take their memory from a
+    pool of the new one, which is given back with its last octree whatever was left in the old one."""
+    child(f"""
+st, a = build(2)
+st2, b = build(1)
+assert st == 0 and st2 == 0
+fake.fake_new_context()
+st, c = build(2)
+assert st == 0 and fake.fake_dead_pool() == 0
+if {old_first}:
+    destroy(a)
+assert fake.fake_trims() == 0
+destroy(c)
+assert fake.fake_trims() == 1 and fake.fake_dead_pool() == 0
+if not {old_first}:
+    destroy(a)
+destroy(b)
+st, d = build(3)
+assert st == 0
+destroy(d)
+assert fake.fake_trims() == 2 and fake.fake_dead_pool() == 0
+""")
