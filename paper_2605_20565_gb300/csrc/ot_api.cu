@@ -331,20 +331,22 @@ ot_status ot_octree_centres(const ot_octree* t, double* d_xyz, void* stream) {
 
 ot_status ot_octree_destroy(ot_octree* t) {
     if (!t) return OT_OK;
-    // pool memory is handed out again without a wait: the work that reads it has to be done
-    wait_device(t->device);
-    if (t->d_key) cudaFree(t->d_key);
-    if (t->d_level) cudaFree(t->d_level);
-    if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);
-    if (t->d_pmap) cudaFree(t->d_pmap);
-    if (t->d_nodes) cudaFree(t->d_nodes);
-    if (t->d_desc) cudaFree(t->d_desc);
-    if (t->d_mates && t->mates_owned) cudaFree(t->d_mates);
-    if (t->d_need_flags) cudaFree(t->d_need_flags);
-    if (t->d_models) cudaFree(t->d_models);
-    if (t->d_mids) cudaFree(t->d_mids);
-    if (t->d_root) cudaFree(t->d_root);
-    if (t->d_err) cudaFree(t->d_err);
+    // pool memory is handed out again without a wait: the work that reads it has to be done (left
+    // allocated when that cannot be known: while the whole process captures a stream)
+    if (wait_device(t->device)) {
+        if (t->d_key) cudaFree(t->d_key);
+        if (t->d_level) cudaFree(t->d_level);
+        if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);
+        if (t->d_pmap) cudaFree(t->d_pmap);
+        if (t->d_nodes) cudaFree(t->d_nodes);
+        if (t->d_desc) cudaFree(t->d_desc);
+        if (t->d_mates && t->mates_owned) cudaFree(t->d_mates);
+        if (t->d_need_flags) cudaFree(t->d_need_flags);
+        if (t->d_models) cudaFree(t->d_models);
+        if (t->d_mids) cudaFree(t->d_mids);
+        if (t->d_root) cudaFree(t->d_root);
+        if (t->d_err) cudaFree(t->d_err);
+    }
     pool_octree_left(t->device, t->context);
     delete t;
     return OT_OK;

@@ -693,7 +693,7 @@ ot_status finish_tree(ot_octree* t, cudaStream_t s, int map_level) {
     }
     if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e);
     // (a change of the map level: work on other streams may still read the old map)
-    if (t->d_desc) wait_device(t->device);
+    if (t->d_desc && !wait_device(t->device)) return fail(cudaErrorUnknown);
     if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);
     if (t->d_desc) cudaFree(t->d_desc);
     t->d_lmap = lmap;

@@ -194,8 +194,7 @@ bool mates_fit(const ot_octree* t) {
 // Frees the flags (pool memory, whose release does not wait for work that may still read it).
 void drop_need_flags(ot_octree* t) {
     if (!t->d_need_flags) return;
-    wait_device(t->device);
-    cudaFree(t->d_need_flags);
+    if (wait_device(t->device)) cudaFree(t->d_need_flags);
     t->d_need_flags = nullptr;
 }
 

@@ -28,6 +28,7 @@ constexpr int MAX_DEVICES = 64;
 struct Pool {
     cudaMemPool_t pool = nullptr;
     int octrees = 0;
+    void* neighbour = nullptr;  // see wait_device
 };
 std::mutex g_pool_mu;
 // by device and context: a pool dies with the context that it was made in, and the octrees that
@@ -129,12 +130,27 @@ void pool_octree_left(int dev, unsigned long long context) {
     if (cur != dev) cudaSetDevice(cur);
 }
 
-void wait_device(int dev) {
+// Until the work that the device has is done.  By cudaFree, which waits for every stream: unlike
+// cudaDeviceSynchronize it is allowed while another thread captures a stream in its own mode or the
+// relaxed one (that call is refused then and ends the capture).  (cudaFree of pool memory does not wait.)
+// false when it could not be waited for.
+bool wait_device(int dev) {
     int cur = dev;
     cudaGetDevice(&cur);
     if (cur != dev) cudaSetDevice(dev);
-    cudaDeviceSynchronize();
+    const unsigned long long context = made_context();
+    try {  // a neighbour that stays, so that the block freed below is not mapped and unmapped each time
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        Pool& q = g_pools[{dev, context}];
+        if (!q.neighbour && cudaMalloc(&q.neighbour, 64) != cudaSuccess) q.neighbour = nullptr, cudaGetLastError();
+    } catch (const std::bad_alloc&) {
+    }
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, 64);
+    e = e == cudaSuccess ? cudaFree(p) : cudaDeviceSynchronize();
+    if (e != cudaSuccess || !p) cudaGetLastError();
     if (cur != dev) cudaSetDevice(cur);
+    return e == cudaSuccess;
 }
 
 int num_sms() {

@@ -91,3 +91,20 @@ assert st == 0
 destroy(d)
 assert fake.fake_trims() == 2 and fake.fake_dead_pool() == 0
 """)
+
+
+def test_memory_is_released_after_a_wait_that_captures_allow(child):
+    """Destroying an octree, changing its map and dropping its tables wait for the device before pool
+    memory is released, without cudaDeviceSynchronize (an error while a stream is captured anywhere)."""
+    child("""
+st, h = build(3)
+assert st == 0
+for level in (2, 1, 3):
+    assert lib.ot_octree_set_map_level(h, level, None) == 0
+for enable in (1, 1, 0, 1):
+    assert lib.ot_octree_build_mates(h, enable, None) == 0
+st, g = build(2)
+destroy(h)
+destroy(g)
+assert fake.fake_unwaited() == 0 and fake.fake_device_syncs() == 0 and fake.fake_live(POOL) == 0
+""")
