@@ -248,13 +248,18 @@ ot_status ot_octree_from_leaves(const uint64_t* d_keys, const uint8_t* d_levels,
     if (n > OT_MAX_LEAVES) return OT_ERR_LIMIT;
     *out = nullptr;
     cudaStream_t s = (cudaStream_t)stream;
-    int lmin = 0, lmax = 0;
-    ot_status st = validate_leaves(d_keys, d_levels, n, balance_full ? 1 : 0, s, &lmin, &lmax);
-    if (st != OT_OK) return st;
     ot_octree* t = new (std::nothrow) ot_octree();
     if (!t) return OT_ERR_OOM;
     cudaGetDevice(&t->device);
     t->context = pool_octree_made(t->device);
+    int lmin = 0, lmax = 0;
+    ot_status st = validate_leaves(d_keys, d_levels, n, balance_full ? 1 : 0, s, &lmin, &lmax);
+    if (st != OT_OK) {
+        cudaStreamSynchronize(s);  // the validation's memory is back in the pool, which may be given back
+        pool_octree_left(t->device, t->context);
+        delete t;
+        return st;
+    }
     cudaError_t e = pool_malloc((void**)&t->d_key, sizeof(uint64_t) * n, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&t->d_level, n, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(t->d_key, d_keys, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s);

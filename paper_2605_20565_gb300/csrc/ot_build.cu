@@ -559,10 +559,11 @@ __global__ void k_check_balance(const uint64_t* __restrict__ key, const uint8_t*
 
 ot_status validate_leaves(const uint64_t* d_key, const uint8_t* d_level, int64_t n, int full, cudaStream_t s, int* lmin,
                           int* lmax) {
-    unsigned* bad = nullptr;
-    int* lr = nullptr;
-    OT_CUDA(pool_malloc((void**)&bad, 2 * sizeof(unsigned), s));
-    OT_CUDA(pool_malloc((void**)&lr, 2 * sizeof(int), s));
+    unsigned* bad = nullptr;  // two counts, then the level range
+    Guard g{s, {}};
+    OT_CUDA(pool_malloc((void**)&bad, 2 * sizeof(unsigned) + 2 * sizeof(int), s));
+    g.keep(bad);
+    int* lr = reinterpret_cast<int*>(bad + 2);
     int init[2] = {1 << 20, -1};
     OT_CUDA(cudaMemsetAsync(bad, 0, 2 * sizeof(unsigned), s));
     OT_CUDA(cudaMemcpyAsync(lr, init, sizeof(init), cudaMemcpyHostToDevice, s));
@@ -583,8 +584,6 @@ ot_status validate_leaves(const uint64_t* d_key, const uint8_t* d_level, int64_t
         OT_CUDA(cudaStreamSynchronize(s));
         if (hb[1] != 0) st = OT_ERR_UNBALANCED;
     }
-    cudaFreeAsync(bad, s);
-    cudaFreeAsync(lr, s);
     *lmin = hr[0];
     *lmax = hr[1];
     OT_CUDA(cudaGetLastError());

@@ -108,3 +108,32 @@ destroy(h)
 destroy(g)
 assert fake.fake_unwaited() == 0 and fake.fake_device_syncs() == 0 and fake.fake_live(POOL) == 0
 """)
+
+
+@pytest.mark.parametrize("why", ["leaves", "memory"])
+def test_refused_leaves_leave_no_memory(child, why):
+    """ot_octree_from_leaves that is refused, for its leaves or for want of memory, gives the pool's memory back when no
+    octree lives, and only then."""
+    child(f"""
+lib.ot_octree_from_leaves.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_int, C.c_void_p, C.c_void_p]
+keys, levels = (C.c_uint64 * 8)(), (C.c_uint8 * 8)()
+def refused():
+    if {why == "leaves"}:
+        fake.fake_copy_word(1, 1)  # the count of leaves out of place
+        want = -4
+    else:
+        fake.fake_fail_from(1)
+        want = OOM
+    h = C.c_void_p(1)
+    assert lib.ot_octree_from_leaves(keys, levels, 8, 1, None, C.byref(h)) == want and not h.value
+    fake.fake_copy_word(0, 0)
+    fake.fake_fail_from(1 << 62)
+refused()
+assert fake.fake_live(POOL) == 0 and fake.fake_trims() == 1
+st, h = build(2)
+live = fake.fake_live(POOL)
+refused()
+assert fake.fake_live(POOL) == live and fake.fake_trims() == 1
+destroy(h)
+assert fake.fake_live(POOL) == 0 and fake.fake_trims() == 2
+""")
