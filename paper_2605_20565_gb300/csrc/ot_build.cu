@@ -12,6 +12,7 @@
 //      leaf counts bottom-up and offsets top-down place every leaf at its rank without a
 //      global sort.
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <vector>
 
@@ -61,7 +62,8 @@ __device__ bool box_near_surface(const double lo[3], double h, const ot_sphere& 
 // rounding can have moved it, 0 when the FP64 test has to decide (a few cells in a thousand; the
 // FP64 pipe was most of the refinement's time, 497 -> 154 us for 17.3M leaves).  Rounding: positions,
 // radii and distances carry at most 2^-23 of the magnitudes involved each, some 6 of them; the
-// margin is 4e-6 of their sum.
+// margin is 4e-6 of their sum.  Centres whose squared distances overflow FP32 (from 1.8e19 on) are
+// left to FP64 too.
 __device__ __forceinline__ int near_surface_f32(const float lo[3], float h, const ot_sphere& s) {
     float near2 = 0.0f, far2 = 0.0f, mag = 1.0f;
 #pragma unroll
@@ -75,6 +77,7 @@ __device__ __forceinline__ int near_surface_f32(const float lo[3], float h, cons
     const float r = (float)s.r, w = (float)s.shell;
     const float dist = fmaxf(fmaxf(sqrtf(near2) - r, r - sqrtf(far2)), 0.0f);
     const float margin = 4e-6f * (mag + r + w);
+    if (!(near2 <= FLT_MAX && far2 <= FLT_MAX)) return 0;
     return dist > w + margin ? -1 : dist < w - margin ? 1 : 0;
 }
 
