@@ -545,7 +545,8 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
     std::vector<Launch> launches;
     NodeGrid grid{};
     // min_pts: while there are fewer tiles than warps, the tiles are halved down to this many points
-    // (11,000 points in tiles of 128 would keep 86 of thousands of warps busy)
+    // (11,000 points in tiles of 128 would keep 86 of thousands of warps busy), to a multiple of it: the
+    // trilinear kernels take rows of 32 and would read an odd half row's points into the next tile's
     auto add_launch = [&](void* fn, BatchArgs args, int cap, int min_pts, size_t dsmem = 0) -> cudaError_t {
         int per_sm = 0;
         cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, dsmem);
@@ -554,7 +555,7 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
         per_sm = std::max(per_sm, 1);
         const int64_t warps = (int64_t)num_sms() * per_sm * (block / 32);
         while (args.ntiles < warps && args.pts / 2 >= min_pts) {
-            args.pts /= 2;
+            args.pts = args.pts / 2 / min_pts * min_pts;
             args.ntiles = 0;
             for (int k = 0; k < args.ng; ++k) {
                 args.g[k].tile0 = args.ntiles;

@@ -137,3 +137,41 @@ assert fake.fake_live(POOL) == live and fake.fake_trims() == 1
 destroy(h)
 assert fake.fake_live(POOL) == 0 and fake.fake_trims() == 2
 """)
+
+
+@pytest.mark.parametrize("mates", [False, True])
+@pytest.mark.parametrize("tile", [1, 2, 3, 4, 5, 7, 48, 64])
+def test_tiles_of_a_small_batch(child, tile, mates):
+    """With fewer tiles than warps the tiles get smaller: the trilinear kernels' stay whole rows of 32 points (a
+    tile that ends within a row would be done twice from there on), the delta kernels' at least 4
+    points, and the tiles cover the points once."""
+    child(f"""
+class Group(C.Structure):
+    _fields_ = [("kernel", C.c_int), ("x", C.c_void_p), ("y", C.c_void_p), ("z", C.c_void_p), ("n", C.c_int64),
+                ("u", C.c_void_p), ("host", C.c_void_p)]
+st, h = build(3)
+if {mates}:
+    assert lib.ot_octree_build_mates(h, 1, None) == 0
+for n in (1, 31, 300, 1000, 6000):
+    fake.fake_forget_batches()
+    x = (C.c_double * n)()
+    u = (C.c_float * (3 * n))()
+    p = [C.addressof(a) for a in (x, x, x, u)]
+    kinds = (2, 1) if {mates} else (1,)
+    groups = (Group * len(kinds))(*(Group(k, *p[:3], n, p[3], None) for k in kinds))
+    launch = (C.c_int * 7)(0, {tile}, 0, 0, 0, 0, -1)
+    b = C.c_void_p()
+    lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+    assert lib.ot_batch_create(h, groups, len(kinds), u, 0, launch, None, C.byref(b)) == 0
+    assert fake.fake_batch_launches() == len(kinds)
+    for i, kind in enumerate(kinds):
+        pts, tiles = fake.fake_batch_pts(i), fake.fake_batch_tiles(i)
+        assert fake.fake_batch_kernel(i) == kind and tiles == -(-n // pts)
+        assert pts <= 32 * {tile} and pts % (32 if kind == 1 else 4) == 0
+        # as small as it may be while there are fewer tiles than the 32 warps of the fake's 4 SMs
+        assert tiles >= 32 or pts < 2 * (32 if kind == 1 else 4)
+    lib.ot_batch_destroy.argtypes = [C.c_void_p]
+    assert lib.ot_batch_destroy(b) == 0
+destroy(h)
+assert fake.fake_live(POOL) == 0
+""")
