@@ -396,12 +396,19 @@ bool wide_cells(const ot_octree* t) { return t->n >= (int64_t)1 << 28; }
 
 // Cells' entries, node list and record buffer of a batch (synchronises the legacy stream; batch
 // creation is not stream-ordered work).  Leaves b->n_rec = 0, without an error, when no leaf is hot
-// or the records' grids (up to 1.9 GB at hot level 8) find no memory: the rows serve then.
+// or one of them (the records' grids: up to 1.9 GB at hot level 8) finds no memory: the rows serve then.
 ot_status build_hot_records(const ot_octree* t, int hot_l, const NodeGrid& grid, ot_batch* b) {
     const size_t n_node = grid.off[hot_l + 1], seen_bytes = ((n_node + 31) / 32) * 4;
     uint32_t* seen = nullptr;  // the bits, then the count
     auto done = [&](cudaError_t e) {
         if (seen) cudaFree(seen);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            if (b->d_rec) cudaFree(b->d_rec);
+            if (b->d_nodes) cudaFree(b->d_nodes);
+            b->d_rec = nullptr, b->d_nodes = nullptr;
+            return OT_OK;
+        }
         return e == cudaSuccess ? OT_OK : cuda_status(e);
     };
     cudaStream_t s = nullptr;
@@ -417,11 +424,7 @@ ot_status build_hot_records(const ot_octree* t, int hot_l, const NodeGrid& grid,
         if (pass == 1) break;
         if ((e = cudaMemcpy(&count, d_count, sizeof(count), cudaMemcpyDeviceToHost)) != cudaSuccess) return done(e);
         if (count == 0) return done(cudaSuccess);
-        if (cudaMalloc(&b->d_rec, sizeof(float) * REC_FLOATS * n_node) != cudaSuccess) {
-            cudaGetLastError();
-            b->d_rec = nullptr;
-            return done(cudaSuccess);
-        }
+        if ((e = cudaMalloc(&b->d_rec, sizeof(float) * REC_FLOATS * n_node)) != cudaSuccess) return done(e);
         if ((e = cudaMalloc(&b->d_nodes, sizeof(uint2) * (size_t)count)) != cudaSuccess) return done(e);
     }
     const bool wide = wide_cells(t);

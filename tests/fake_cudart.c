@@ -14,6 +14,7 @@ static struct {
     int kind;
 } blocks[MAX_BLOCKS];
 static size_t fail_bytes = (size_t)-1;
+static int fail_in = -1;
 static unsigned long long context = 1;
 static unsigned word;
 static int has_word, unwaited, dead_pool, trims, device_syncs;
@@ -23,6 +24,7 @@ struct pool {
 
 /* for the tests */
 void fake_fail_from(size_t bytes) { fail_bytes = bytes; }             /* allocations of that size or more */
+void fake_fail_nth(int n) { fail_in = n; }                              /* the n-th allocation from here */
 void fake_new_context(void) { ++context; }                              /* as cudaDeviceReset does */
 void fake_copy_word(int on, unsigned v) { has_word = on, word = v; }    /* what a 4-byte copy to the host brings */
 int fake_live(int kind) {
@@ -38,7 +40,7 @@ int fake_unwaited(void) { return unwaited; }         /* pool memory released by 
 static int waited;
 static int take(void** p, size_t bytes, int kind) {
     *p = NULL;
-    if (bytes >= fail_bytes) return OOM;
+    if (bytes >= fail_bytes || (fail_in > 0 && --fail_in == 0)) return OOM;
     for (int i = 0; i < MAX_BLOCKS; ++i)
         if (!blocks[i].p) {
             *p = blocks[i].p = aligned_alloc(256, (bytes + 511) / 256 * 256);

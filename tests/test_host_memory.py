@@ -175,3 +175,37 @@ for n in (1, 31, 300, 1000, 6000):
 destroy(h)
 assert fake.fake_live(POOL) == 0
 """)
+
+
+def test_a_batch_without_memory_for_records_is_made_without(child):
+    """Creating a batch with value records takes four allocations for them (the bits and count, the records, the node list, the cells'
+    entries): whichever fails, the batch is made without records and keeps none of the others."""
+    child("""
+class Group(C.Structure):
+    _fields_ = [("kernel", C.c_int), ("x", C.c_void_p), ("y", C.c_void_p), ("z", C.c_void_p), ("n", C.c_int64),
+                ("u", C.c_void_p), ("host", C.c_void_p)]
+st, h = build(3)
+assert lib.ot_octree_build_mates(h, 1, None) == 0
+n = 4096
+x, u = (C.c_double * n)(), (C.c_float * (3 * n))()
+px, pu = C.addressof(x), C.addressof(u)
+groups = (Group * 1)(Group(1, px, px, px, n, pu, None))
+lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+lib.ot_batch_destroy.argtypes = [C.c_void_p]
+before = fake.fake_live(MALLOC)
+def create():
+    b = C.c_void_p()
+    fake.fake_copy_word(1, 5)  # nodes of hot leaves
+    st = lib.ot_batch_create(h, groups, 1, u, 0, None, None, C.byref(b))
+    fake.fake_copy_word(0, 0)
+    held = fake.fake_live(MALLOC) - before
+    assert st == 0 and lib.ot_batch_destroy(b) == 0 and fake.fake_live(MALLOC) == before
+    return held
+assert create() == 5  # the tile counter, the cell means; records, node list, entries
+for k in (3, 4, 5, 6):
+    fake.fake_fail_nth(k)
+    assert create() == 2
+fake.fake_fail_nth(-1)
+assert create() == 5
+destroy(h)
+""")
