@@ -8,7 +8,8 @@ One step = one pass of the hot path over the whole point set:
 value = (markers + particles) / step time, summed over ranks (each rank runs its own
 independent copy of the workload: weak scaling, no data-path collective).
 
-Prints ONE JSON line (rank 0).  ``--impl reference`` times the FP64 CPU oracle on the same
+Prints ONE JSON line (rank 0) on standard output, at most 2.4 KB, and the whole record (every form and
+workload in detail) on standard error.  ``--impl reference`` times the FP64 CPU oracle on the same
 workload instead (bounded samples, host cores).
 """
 from __future__ import annotations
@@ -968,6 +969,56 @@ def compact(d):
     return out
 
 
+LINE_BYTES = 2400  # of the line on standard output: readers keep its last 3 KB
+
+
+def headline(out):
+    """The line printed on standard output: the record's own keys, without the other workloads' details (their
+    throughput and step time stay) and texts cut to a few words, so that it stays short."""
+    def pick(d, keys):
+        return {k: d[k] for k in keys if k in d} if isinstance(d, dict) else d
+
+    def short(v, n):
+        if isinstance(v, dict):
+            return {k: short(x, n) for k, x in v.items()}
+        if isinstance(v, float):
+            return float(f"{v:.7g}")
+        return v[:n] if isinstance(v, str) else v
+
+    line = pick(out, ("metric", "value", "unit", "impl", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+                      "scaling", "vs_baseline", "dtype", "data", "gpu_launches"))
+    metric = line.get("metric")
+    line["config"] = pick(out.get("config"), ("workload", "bubbles", "levels", "leaves", "markers_peskin4",
+                                              "particles_trilinear", "search", "form", "level_mates", "map_level",
+                                              "spread", "particle_order", "l2", "model", "parallelism"))
+    line["roofline"] = pick(out.get("roofline"), ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
+                                                  "peak_kind", "algorithmic_bytes_per_launch",
+                                                  "algorithmic_bytes_per_step"))
+    line["cpu_baseline"] = pick(out.get("cpu_baseline"), ("value", "unit", "cores", "kind"))
+    line["clocks"] = pick(out.get("clocks"), ("sm_mhz", "sm_max_mhz", "reasons", "samples"))
+    line["e2e"] = pick(out.get("e2e"), ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step",
+                                        "steps", "pipeline"))
+    line["parity"] = pick(out.get("parity"), ("all_ok", "tolerance"))
+    line["workloads"] = {k: pick(d, ("error",)) or
+                         {"value": d.get("value"), "ms_per_step": d.get("ms_per_step"),
+                          "e2e": (d.get("e2e") or {}).get("value"), "ok": (d.get("parity") or {}).get("all_ok")}
+                         for k, d in out.get("workloads", {}).items()}
+    line = {k: v for k, v in line.items() if v not in (None, {}) or k == "vs_baseline"}
+    for n in (90, 60, 40, 20):
+        cut = short(line, n)
+        if metric is not None:
+            cut["metric"] = metric
+        if len(json.dumps(cut)) <= LINE_BYTES:
+            break
+    return cut
+
+
+def report(out):
+    """The whole record on standard error, the line on standard output."""
+    print("[bench] record " + json.dumps(out), file=sys.stderr, flush=True)
+    print(json.dumps(headline(out)), flush=True)
+
+
 def run_ours(args):
     import torch
     from paper_2605_20565_gb300 import _build
@@ -1017,7 +1068,7 @@ def run_ours(args):
             print(f"[bench] {name}: {d['wall_s']:.1f} s", file=sys.stderr, flush=True)
             out["workloads"][name] = d
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        report(out)
     if dist:
         dist.destroy_process_group()
     return 0
@@ -1118,7 +1169,7 @@ def run_tracking(args, light=False, ctx=None):
            "step_parts_ms": parts, "gpu_launches": int(launches), "clocks": clk,
            "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "parity": parity}
     if ctx is None:
-        print(json.dumps(out), flush=True)
+        report(out)
     return out
 
 
