@@ -83,18 +83,15 @@ TreeView tree_view(const ot_octree* t);
 // Exclusive scan of n uint32 (in place allowed); returns the total in *d_total if non-null.
 // Temporary storage is allocated stream-ordered and released before return.
 ot_status scan_u32(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* d_total, cudaStream_t s);
-// The same scan with its temporaries in ws (scan_ws_bytes(n) bytes, 4-byte aligned): no allocation.
-size_t scan_ws_bytes(int64_t n);
-ot_status scan_u32_ws(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* d_total, void* ws, cudaStream_t s);
 // Stable LSD radix sort of n uint64 by bits [bit0, bit1) (8-bit digits).  d_tmp: n uint64
 // scratch.  Result in d_keys.  Temporaries (histograms) are stream-ordered allocations.
 ot_status radix_sort_u64(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, cudaStream_t s);
 // The same sort with caller workspace of radix_ws_bytes(n) bytes: nothing is allocated.
-// d_n (nullable): the key count in device memory, at most n.  *result (nullable): the buffer
-// (d_keys or d_tmp) left with the sorted keys; without it they are in d_keys.
+// *result (nullable): the buffer (d_keys or d_tmp) left with the sorted keys; without it they are
+// in d_keys.
 size_t radix_ws_bytes(int64_t n);
 ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
-                            cudaStream_t s, const uint32_t* d_n = nullptr, uint64_t** result = nullptr);
+                            cudaStream_t s, uint64_t** result = nullptr);
 // Exclusive scan of a short row in place by one block; its total to *d_total.
 ot_status scan_row(uint32_t* d_row, int n, uint32_t* d_total, cudaStream_t s);
 // Compaction: out[j] = in[i] for the i with flag[i] != 0, in order; *h_count on the host

@@ -58,7 +58,7 @@ ot_status launch_point_sort(const double* x, const double* y, const double* z, i
     void* rws = tmp + n;
     k_point_keys<<<grid_o(n), 256, 0, s>>>(x, y, z, n, level, ib, pairs);
     count_launch();
-    return radix_sort_u64_ws(pairs, tmp, n, ib, ib + 3 * level, rws, s, nullptr, sorted);
+    return radix_sort_u64_ws(pairs, tmp, n, ib, ib + 3 * level, rws, s, sorted);
 }
 
 } // namespace ot

@@ -87,7 +87,7 @@ static int64_t scan_tile_elems(int64_t n) {
     return total;
 }
 
-size_t scan_ws_bytes(int64_t n) { return (size_t)(scan_tile_elems(n) + 1) * sizeof(uint32_t) + 256; }
+static size_t scan_ws_bytes(int64_t n) { return (size_t)(scan_tile_elems(n) + 1) * sizeof(uint32_t) + 256; }
 
 // The recursive scan with its tile totals in tmp (scan_tile_elems(n) uint32).
 static ot_status scan_levels(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* tmp, cudaStream_t s) {
@@ -106,7 +106,8 @@ static ot_status scan_levels(const uint32_t* d_in, uint32_t* d_out, int64_t n, u
     return OT_OK;
 }
 
-ot_status scan_u32_ws(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* d_total, void* ws, cudaStream_t s) {
+static ot_status scan_u32_ws(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* d_total, void* ws,
+                             cudaStream_t s) {
     if (n <= 0) {
         if (d_total) OT_CUDA(cudaMemsetAsync(d_total, 0, sizeof(uint32_t), s));
         return OT_OK;
@@ -146,13 +147,10 @@ ot_status scan_u32(const uint32_t* d_in, uint32_t* d_out, int64_t n, uint32_t* d
 // ------------------------------------------------------------------------------------------
 constexpr int RT = 256, RI = 16, RTILE = RT * RI, RW = RT / 32;
 
-// d_n (nullable): the element count in device memory, at most n (tiles past it stay empty).
 __global__ void __launch_bounds__(RT) k_radix_hist(const uint64_t* __restrict__ in, int64_t n, int shift,
-                                                   uint32_t mask, uint32_t* __restrict__ hist, int ntiles,
-                                                   const uint32_t* __restrict__ d_n) {
+                                                   uint32_t mask, uint32_t* __restrict__ hist, int ntiles) {
     __shared__ uint32_t cnt[256];
     cnt[threadIdx.x] = 0;
-    if (d_n) n = min(n, (int64_t)*d_n);
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * RTILE;
     if (base + RTILE <= n) {  // a whole tile: every load issued before the first count
@@ -201,8 +199,7 @@ __global__ void __launch_bounds__(ROW_T) k_radix_rows(uint32_t* __restrict__ his
 __global__ void __launch_bounds__(RT) k_radix_scatter(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
                                                       int64_t n, int shift, uint32_t mask,
                                                       const uint32_t* __restrict__ offs, int ntiles,
-                                                      const uint32_t* __restrict__ totals,
-                                                      const uint32_t* __restrict__ d_n) {
+                                                      const uint32_t* __restrict__ totals) {
     __shared__ uint64_t s_key[RTILE];
     __shared__ uint32_t s_cnt[RW][256];  // per warp: digit counts, then the warp's first place per digit
     // per warp and digit, the lanes of the current round (used before the keys are placed)
@@ -210,9 +207,7 @@ __global__ void __launch_bounds__(RT) k_radix_scatter(const uint64_t* __restrict
     __shared__ uint32_t s_base[256];     // digit: its place in out, less its place in the tile
     __shared__ uint32_t s_warp[33];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (d_n) n = min(n, (int64_t)*d_n);
     const int64_t base = (int64_t)blockIdx.x * RTILE;
-    if (base >= n) return;  // block-uniform
     const int cnt = (int)min((int64_t)RTILE, n - base);
     const int first = warp * (RTILE / RW) + lane;
     uint64_t v[RI];
@@ -277,7 +272,7 @@ size_t radix_ws_bytes(int64_t n) {
 }
 
 ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bit0, int bit1, void* ws,
-                            cudaStream_t s, const uint32_t* d_n, uint64_t** result) {
+                            cudaStream_t s, uint64_t** result) {
     if (result) *result = d_keys;
     if (n <= 1 || bit1 <= bit0) return OT_OK;
     const int nt = (int)((n + RTILE - 1) / RTILE);
@@ -288,9 +283,9 @@ ot_status radix_sort_u64_ws(uint64_t* d_keys, uint64_t* d_tmp, int64_t n, int bi
     for (int sh = bit0, passes = (bit1 - bit0 + 7) / 8; passes > 0; --passes) {
         const int nb = (bit1 - sh + passes - 1) / passes;
         const uint32_t mask = (1u << nb) - 1u;
-        k_radix_hist<<<nt, RT, 0, s>>>(src, n, sh, mask, hist, nt, d_n);
+        k_radix_hist<<<nt, RT, 0, s>>>(src, n, sh, mask, hist, nt);
         k_radix_rows<<<256, ROW_T, 0, s>>>(hist, nt, totals);
-        k_radix_scatter<<<nt, RT, 0, s>>>(src, dst, n, sh, mask, hist, nt, totals, d_n);
+        k_radix_scatter<<<nt, RT, 0, s>>>(src, dst, n, sh, mask, hist, nt, totals);
         count_launch(3);
         std::swap(src, dst);
         sh += nb;

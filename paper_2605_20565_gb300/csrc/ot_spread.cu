@@ -802,7 +802,7 @@ ot_status plan_tiles(const ot_octree* t, const double* x, const double* y, const
             auto k = k_tile_keys<K>;
             k<<<grid_for(k, 256, 0, n), 256, 0, s>>>(o, cur, sh, nb, a, pl.rt, pl.n_runs);
             count_launch();
-            if ((st = radix_sort_u64_ws(a, a == pairs ? tmp : pairs, n, ib, ib + nb, rws, s, nullptr, &cur)) != OT_OK)
+            if ((st = radix_sort_u64_ws(a, a == pairs ? tmp : pairs, n, ib, ib + nb, rws, s, &cur)) != OT_OK)
                 return st;
         }
         o.pairs = cur;
