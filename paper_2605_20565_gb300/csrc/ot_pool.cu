@@ -32,8 +32,12 @@ struct Pool {
 };
 std::mutex g_pool_mu;
 // by device and context: a pool dies with the context that it was made in, and the octrees that
-// were left in it no longer count
-std::map<std::pair<int, unsigned long long>, Pool> g_pools;
+// were left in it no longer count.  Never destroyed: an octree may be, by a static object of the
+// caller's, after this library's own statics.
+std::map<std::pair<int, unsigned long long>, Pool>& pools() {
+    static auto* all = new std::map<std::pair<int, unsigned long long>, Pool>();
+    return *all;
+}
 
 cudaError_t create_pool(int dev, cudaMemPool_t* out) {
     cudaMemPoolProps p{};
@@ -94,7 +98,7 @@ cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s) {
     cudaMemPool_t pool;
     try {
         std::lock_guard<std::mutex> lock(g_pool_mu);
-        Pool& q = g_pools[{dev, context}];
+        Pool& q = pools()[{dev, context}];
         if (!q.pool && (e = create_pool(dev, &q.pool)) != cudaSuccess) {
             q.pool = nullptr;
             return e;
@@ -112,7 +116,7 @@ unsigned long long pool_octree_made(int dev) {
     const unsigned long long context = made_context();
     try {
         std::lock_guard<std::mutex> lock(g_pool_mu);
-        ++g_pools[{dev, context}].octrees;
+        ++pools()[{dev, context}].octrees;
     } catch (const std::bad_alloc&) {  // not counted: the pool is given back with the others
     }
     return context;
@@ -120,13 +124,18 @@ unsigned long long pool_octree_made(int dev) {
 
 void pool_octree_left(int dev, unsigned long long context) {
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    const auto it = g_pools.find({dev, context});
-    if (it == g_pools.end() || --it->second.octrees > 0 || !it->second.pool) return;
+    Pool* q = nullptr;
+    try {
+        const auto it = pools().find({dev, context});
+        if (it != pools().end()) q = &it->second;
+    } catch (const std::bad_alloc&) {
+    }
+    if (!q || --q->octrees > 0 || !q->pool) return;
     int cur = dev;
     cudaGetDevice(&cur);
     if (cur != dev) cudaSetDevice(dev);
     // (a pool of another context than the device's may no longer exist)
-    if (current_context_id() == context) cudaMemPoolTrimTo(it->second.pool, 0);
+    if (current_context_id() == context) cudaMemPoolTrimTo(q->pool, 0);
     if (cur != dev) cudaSetDevice(cur);
 }
 
@@ -141,7 +150,7 @@ bool wait_device(int dev) {
     const unsigned long long context = made_context();
     try {  // a neighbour that stays, so that the block freed below is not mapped and unmapped each time
         std::lock_guard<std::mutex> lock(g_pool_mu);
-        Pool& q = g_pools[{dev, context}];
+        Pool& q = pools()[{dev, context}];
         if (!q.neighbour && cudaMalloc(&q.neighbour, 64) != cudaSuccess) q.neighbour = nullptr, cudaGetLastError();
     } catch (const std::bad_alloc&) {
     }
@@ -170,20 +179,21 @@ int num_sms() {
 // once (the query takes longer than a launch).
 int blocks_per_sm(const void* fn, int block, size_t smem) {
     static std::mutex mu;
-    static std::map<std::tuple<const void*, int, size_t, int>, int> known;
+    using Known = std::map<std::tuple<const void*, int, size_t, int>, int>;
+    static auto* known = new (std::nothrow) Known();  // (never destroyed, as above)
     int dev = 0;
     cudaGetDevice(&dev);
     const auto key = std::make_tuple(fn, block, smem, dev);
-    {
+    if (known) {
         std::lock_guard<std::mutex> lock(mu);
-        const auto it = known.find(key);
-        if (it != known.end()) return it->second;
+        const auto it = known->find(key);
+        if (it != known->end()) return it->second;
     }
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, smem) != cudaSuccess || per_sm < 1) return 1;
     try {
         std::lock_guard<std::mutex> lock(mu);
-        known[key] = per_sm;
+        if (known) (*known)[key] = per_sm;
     } catch (...) {  // no memory to keep it: asked for again
     }
     return per_sm;
