@@ -338,7 +338,7 @@ ot_status ot_octree_destroy(ot_octree* t) {
     if (!t) return OT_OK;
     // pool memory is handed out again without a wait: the work that reads it has to be done (left
     // allocated when that cannot be known: while the whole process captures a stream)
-    if (wait_device(t->device)) {
+    if (context_lives(t->device, t->context) && wait_device(t->device)) {
         if (t->d_key) cudaFree(t->d_key);
         if (t->d_level) cudaFree(t->d_level);
         if (t->d_lmap && t->d_lmap != t->d_pmap) cudaFree(t->d_lmap);

@@ -18,6 +18,8 @@
 
 struct ot_batch {
     const ot_octree* tree = nullptr;
+    int device = 0;
+    unsigned long long context = 0;  // the octree's, that its memory and graph belong to
     int n_groups = 0;
     std::vector<void*> bufs;   // per ordered group: point-order workspace and the ordered copies
     cudaGraph_t graph = nullptr;
@@ -484,6 +486,8 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
 
     ot_batch* b = new ot_batch();
     b->tree = t;
+    b->device = t->device;
+    b->context = t->context;
     b->n_groups = n_groups;
     // trilinear groups processed in Morton order of their points' level-order_level cells:
     // per group, the sort workspace and ordered copies of positions and results
@@ -698,6 +702,10 @@ extern "C" ot_status ot_batch_run(ot_batch* b, void* stream) {
 
 extern "C" ot_status ot_batch_destroy(ot_batch* b) {
     if (!b) return OT_OK;
+    if (!context_lives(b->device, b->context)) {
+        delete b;
+        return OT_OK;
+    }
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->d_counter) cudaFree(b->d_counter);

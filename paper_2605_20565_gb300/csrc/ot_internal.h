@@ -75,6 +75,7 @@ cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t s);
 unsigned long long pool_octree_made(int dev);
 void pool_octree_left(int dev, unsigned long long context);
 unsigned long long current_context_id();
+bool context_lives(int dev, unsigned long long context);
 bool wait_device(int dev);  // until the device's work is done, whichever device is current
 
 TreeView tree_view(const ot_octree* t);

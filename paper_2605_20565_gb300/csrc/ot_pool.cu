@@ -139,6 +139,18 @@ void pool_octree_left(int dev, unsigned long long context) {
     if (cur != dev) cudaSetDevice(cur);
 }
 
+// Whether what was made in this context of the device is still there.  (After cudaDeviceReset it is not,
+// and its addresses and handles may be those of something newer.)
+bool context_lives(int dev, unsigned long long context) {
+    if (context == 0) return true;
+    int cur = dev;
+    cudaGetDevice(&cur);
+    if (cur != dev) cudaSetDevice(dev);
+    const bool same = made_context() == context;
+    if (cur != dev) cudaSetDevice(cur);
+    return same;
+}
+
 // Until the work that the device has is done.  By cudaFree, which waits for every stream: unlike
 // cudaDeviceSynchronize it is allowed while another thread captures a stream in its own mode or the
 // relaxed one (that call is refused then and ends the capture).  (cudaFree of pool memory does not wait.)

@@ -17,7 +17,7 @@ static size_t fail_bytes = (size_t)-1;
 static int fail_in = -1;
 static unsigned long long context = 1;
 static unsigned word;
-static int has_word, unwaited, dead_pool, trims, device_syncs;
+static int has_word, unwaited, bad_frees, dead_pool, trims, device_syncs;
 struct pool {
     unsigned long long context;
 };
@@ -25,7 +25,15 @@ struct pool {
 /* for the tests */
 void fake_fail_from(size_t bytes) { fail_bytes = bytes; }             /* allocations of that size or more */
 void fake_fail_nth(int n) { fail_in = n; }                              /* the n-th allocation from here */
-void fake_new_context(void) { ++context; }                              /* as cudaDeviceReset does */
+void fake_new_context(void) {                                           /* as cudaDeviceReset does */
+    ++context;
+    for (int i = 0; i < MAX_BLOCKS; ++i)
+        if (blocks[i].p) {
+            free(blocks[i].p);
+            blocks[i].p = NULL;
+        }
+}
+int fake_bad_frees(void) { return bad_frees; }       /* of addresses that are not allocated */
 void fake_copy_word(int on, unsigned v) { has_word = on, word = v; }    /* what a 4-byte copy to the host brings */
 int fake_live(int kind) {
     int n = 0;
@@ -60,6 +68,7 @@ static int drop(void* p, int plain) {
             blocks[i].p = NULL;
             return OK;
         }
+    ++bad_frees;
     return INVALID;
 }
 int cudaMalloc(void** p, size_t n) { return take(p, n, MALLOC); }

@@ -209,3 +209,33 @@ fake.fake_fail_nth(-1)
 assert create() == 5
 destroy(h)
 """)
+
+
+def test_what_a_reset_took_is_not_freed_again(child):
+    """Octrees (with tables) and batches of a destroyed context are dropped without releasing anything: their addresses are
+    not theirs any more, and may be a newer octree's."""
+    child("""
+class Group(C.Structure):
+    _fields_ = [("kernel", C.c_int), ("x", C.c_void_p), ("y", C.c_void_p), ("z", C.c_void_p), ("n", C.c_int64),
+                ("u", C.c_void_p), ("host", C.c_void_p)]
+lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+lib.ot_batch_destroy.argtypes = [C.c_void_p]
+x, u = (C.c_double * 64)(), (C.c_float * 192)()
+px, pu = C.addressof(x), C.addressof(u)
+def make():
+    st, h = build(3)
+    assert st == 0 and lib.ot_octree_build_mates(h, 1, None) == 0
+    b = C.c_void_p()
+    assert lib.ot_batch_create(h, (Group * 1)(Group(1, px, px, px, 64, pu, None)), 1, u, 0, None, None, C.byref(b)) == 0
+    return h, b
+old, old_batch = make()
+fake.fake_new_context()
+new, new_batch = make()
+live = fake.fake_live(POOL | MALLOC)
+assert lib.ot_batch_destroy(old_batch) == 0
+destroy(old)
+assert fake.fake_live(POOL | MALLOC) == live and fake.fake_bad_frees() == 0
+assert lib.ot_batch_destroy(new_batch) == 0
+destroy(new)
+assert fake.fake_live(POOL) == 0 and fake.fake_bad_frees() == 0
+""")
