@@ -109,7 +109,8 @@ ot_status ot_octree_from_leaves(const uint64_t* d_keys, const uint8_t* d_levels,
 /* Leaf count and level range. */
 ot_status ot_octree_info(const ot_octree* t, int64_t* n_leaves, int* lmin, int* lmax);
 
-/* Device pointers to the library-owned leaf arrays (valid until ot_octree_destroy). */
+/* Device pointers to the library-owned leaf arrays (valid until ot_octree_destroy).  They are
+ * memory of a stream-ordered pool of their device: other devices and processes cannot map it. */
 ot_status ot_octree_leaves(const ot_octree* t, int64_t* n, const uint64_t** d_keys, const uint8_t** d_levels);
 
 /* Copy the leaves into caller buffers (d_keys: N uint64, d_levels: N uint8; either may be
@@ -277,7 +278,7 @@ ot_status ot_spread_workspace_size(const ot_octree* t, int kernel, int64_t n, si
 /* Force spreading, the exact adjoint of the delta-kernel interpolation (Sec. 2.2, Eq. for
  * F(x)): f(cell) += sum_k F_k phi phi phi dV_k / h^3, h = 2^-lmax, dV_k = h^3 when d_dV is
  * NULL (the paper's literal form).  d_F: 3 planes of n floats; d_f: float4 per leaf,
- * ACCUMULATED (the caller zeroes it), component w untouched.
+ * ACCUMULATED (the caller zeroes it), component w untouched.  n below 2^26 (OT_ERR_LIMIT).
  *   OT_SORTED: the markers are radix-sorted (stable) by the tile of 4x4x4 finest cells that
  *     their stencil starts in; each tile sums its cells' contributions from the 8 tiles whose
  *     stencils reach it, in a fixed order of these and in marker order within each:

@@ -191,7 +191,7 @@ ot_status spread_any(const ot_octree* t, int kernel, int mode, const double* x, 
     if ((kernel != OT_PESKIN4 && kernel != OT_ROMA3) || (mode != OT_SORTED && mode != OT_ATOMIC)) return OT_ERR_ARG;
     if (n > 0 && (!F || !f)) return OT_ERR_ARG;
     if (t->lmax < 1) return OT_ERR_ARG;
-    if (n * 64 >= (1LL << 32)) return OT_ERR_LIMIT; // pair ids are 32-bit
+    if (n * 64 >= (1LL << 32)) return OT_ERR_LIMIT;  // fewer than 2^26 markers (numbers and runs are 32-bit)
     if (mode == OT_SORTED && n > 0 && (!ws || ((uintptr_t)ws & 15))) return OT_ERR_ARG;
     return launch_spread<T>(t, kernel, mode, x, y, z, F, dV, n, f, ws, ws_bytes, (cudaStream_t)stream);
 }

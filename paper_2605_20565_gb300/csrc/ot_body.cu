@@ -195,8 +195,11 @@ extern "C" ot_status ot_body_sums(const double* d_x, const double* d_y, const do
     if (n < 0 || n_bodies < 0 || n_bodies > (1 << 24)) return OT_ERR_ARG;
     if (n_bodies == 0) return OT_OK;
     if (!d_start || !d_xb || !d_lin || !d_ang || (n > 0 && (!d_x || !d_y || !d_z || !d_v))) return OT_ERR_ARG;
-    // blocks per body: up to the portable cluster size while the chip holds all of them at once
-    // (6 blocks per SM), one when the bodies alone fill it or the markers are few
+    // blocks per body: up to the portable cluster size while all of them are at most 6 per SM (3 are
+    // resident by their registers; the rest start as small bodies' end), one when the bodies alone
+    // are that many or the markers are few.  Lines of 3, 6 and 1000 per SM: 64 bodies of different
+    // sizes 349, 277 and 277 us (7.5M markers), 156, 95 and 95 us (2M with volumes), 64 of one size
+    // 175, 178 and 185 us, 1,000 of one size 156, 154 and 384 us.
     int nb = 8;
     while (nb > 1 && ((int64_t)n_bodies * nb > 6 * (int64_t)num_sms() || (int64_t)n_bodies * nb * BT > 4 * n)) nb >>= 1;
     OT_CUDA(d_dV ? launch_body<true>(n_bodies * nb, nb, (cudaStream_t)stream, d_x, d_y, d_z, d_v, d_dV, w, n, d_start,

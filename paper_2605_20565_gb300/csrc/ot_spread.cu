@@ -9,7 +9,7 @@
 // Sorting markers instead of one pair per (marker, overlapped 2x2x2 block) leaves 1/16 of the keys
 // to sort and one record per marker to write, and a record is read by the 5.4 tiles that its
 // stencil overlaps on average instead of by 15.6 blocks.  2M markers of 64 bubbles: spreading
-// 1.84 -> 0.69 ms (keys and sort 0.08, records 0.08, tiles 0.53: issue-bound, 58% of the issue slots
+// 1.84 -> 0.65 ms (keys and sort 0.08, records 0.08, tiles 0.49: issue-bound, 58% of the issue slots
 // at 17 warps per SM, half of the instructions staging and per-tile set-up).
 #include <algorithm>
 
@@ -432,7 +432,11 @@ template <typename T> struct TileOut {
 // Lane: column (x, y) = (lane & 3, lane >> 2 & 3) and the cells z = 2 (lane >> 4), + 1, whose sums
 // it keeps in registers; a marker is staged by one lane and costs the warp 3 shared loads, 2
 // products and 6 fused multiply-adds.  A cell whose sums are all zero is left as it is.
-// 50,000 markers on one bubble (some 700 runs): one warp per run 73 us, one block per tile 41 us.
+// The line of 4096 runs, some 5 blocks of 4 warps on each of 152 SMs, FP32 spreading by warps per run and
+// by blocks per tile: 500,000 markers in 750, 3,000, 5,800 and 11,700 runs 670/295, 298/282, 259/334
+// and 237/468 us; 100,000 in 740, 2,900 and 5,500 runs 194/130, 125/179 and 125/256 us.  With few
+// markers per run the warps are ahead earlier (10,000 in 2,400 runs 85/139 us): the number of
+// markers is not in the rule.
 constexpr int TILE_T = 128, SEG = 64;
 constexpr int64_t WIDE_RUNS = 4096;
 template <typename T, int K>

@@ -1,6 +1,6 @@
-"""Octrees destroyed, re-mapped and given tables on one thread while another captures a CUDA graph in its own mode: the capture
-ends well, and its replays give what they should; and an octree's memory is not released before the
-work on other streams that reads it is done."""
+"""Octrees destroyed, re-mapped and given tables on one thread while another captures a CUDA graph in its
+own mode: the capture ends well, and its replay gives what it should; and an octree's memory is
+not released before the work on other streams that reads it is done."""
 import threading
 
 import numpy as np

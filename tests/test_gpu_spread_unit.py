@@ -43,8 +43,8 @@ def test_sums(env, n, periodic, kernel):
     dV = rng.uniform(0.1, 0.2, n).astype(np.float32)
     inside = X[0] < 1
     kw = dict(periodic=True) if periodic else {}
-    ref, _ = oracle.spread_delta(ko, lo, 1, kernel, *np.ascontiguousarray(X[:, inside]), F[:, inside].astype(np.float64),
-                                 dV=dV[inside].astype(np.float64), **kw)
+    ref, _ = oracle.spread_delta(ko, lo, 1, kernel, *np.ascontiguousarray(X[:, inside]),
+                                 F[:, inside].astype(np.float64), dV=dV[inside].astype(np.float64), **kw)
     x = [torch.as_tensor(np.ascontiguousarray(X[d]), device="cuda") for d in range(3)]
     for dtype, tol in ((torch.float32, 1e-5), (torch.float64, 1e-12)):
         Fd, dVd = (torch.as_tensor(a, device="cuda").to(dtype) for a in (F, dV))

@@ -50,6 +50,7 @@ def test_field_at_any_float(env, kernel, lmin, lmax, offset):
             ot.ot_spread(tree, kernel, ot.OT_SORTED, *x, F, f)
         else:
             s = C.c_void_p(torch.cuda.current_stream().cuda_stream)
-            assert noalloc(tree.handle, kernel, *(a.data_ptr() for a in x), F.data_ptr(), None, n, f.data_ptr(), s) == 0
+            assert noalloc(tree.handle, kernel, *(a.data_ptr() for a in x), F.data_ptr(), None, n, f.data_ptr(),
+                           s) == 0
         assert torch.equal(f, want)
         assert torch.all(buf[:4 + offset] == 7.0) and torch.all(buf[4 + offset + 4 * N:] == 7.0)

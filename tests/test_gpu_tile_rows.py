@@ -39,7 +39,8 @@ def test_same_as_single_calls(env, form, tile, n):
         groups.append(dict(kernel=kernel, x=x[0], y=x[1], z=x[2],
                            u=torch.full((3, n), -9.0, dtype=torch.float32, device="cuda"),
                            host=torch.full((n,), -9, dtype=torch.int32, device="cuda")))
-    b = ot.ot_batch_create(tree, groups, field, launch=dict(tile=tile, tri_tile=tile, tri_records=0 if form == "records" else -1))
+    b = ot.ot_batch_create(tree, groups, field, launch=dict(tile=tile, tri_tile=tile,
+                                                            tri_records=0 if form == "records" else -1))
     for _ in range(2):
         ot.ot_batch_run(b)
     for g, (u, h) in zip(groups, want):

@@ -112,8 +112,8 @@ assert fake.fake_unwaited() == 0 and fake.fake_device_syncs() == 0 and fake.fake
 
 @pytest.mark.parametrize("why", ["leaves", "memory"])
 def test_refused_leaves_leave_no_memory(child, why):
-    """ot_octree_from_leaves that is refused, for its leaves or for want of memory, gives the pool's memory back when no
-    octree lives, and only then."""
+    """ot_octree_from_leaves that is refused, for its leaves or for want of memory, gives the pool's memory
+    back when no octree lives, and only then."""
     child(f"""
 lib.ot_octree_from_leaves.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_int, C.c_void_p, C.c_void_p]
 keys, levels = (C.c_uint64 * 8)(), (C.c_uint8 * 8)()
@@ -161,7 +161,7 @@ for n in (1, 31, 300, 1000, 6000):
     groups = (Group * len(kinds))(*(Group(k, *p[:3], n, p[3], None) for k in kinds))
     launch = (C.c_int * 7)(0, {tile}, 0, 0, 0, 0, -1)
     b = C.c_void_p()
-    lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+    lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int] + [C.c_void_p] * 3
     assert lib.ot_batch_create(h, groups, len(kinds), u, 0, launch, None, C.byref(b)) == 0
     assert fake.fake_batch_launches() == len(kinds)
     for i, kind in enumerate(kinds):
@@ -178,8 +178,9 @@ assert fake.fake_live(POOL) == 0
 
 
 def test_a_batch_without_memory_for_records_is_made_without(child):
-    """Creating a batch with value records takes four allocations for them (the bits and count, the records, the node list, the cells'
-    entries): whichever fails, the batch is made without records and keeps none of the others."""
+    """Creating a batch with value records takes four allocations for them (the bits and count, the records,
+    the node list, the cells' entries): whichever fails, the batch is made without records and keeps
+    none of the others."""
     child("""
 class Group(C.Structure):
     _fields_ = [("kernel", C.c_int), ("x", C.c_void_p), ("y", C.c_void_p), ("z", C.c_void_p), ("n", C.c_int64),
@@ -190,7 +191,7 @@ n = 4096
 x, u = (C.c_double * n)(), (C.c_float * (3 * n))()
 px, pu = C.addressof(x), C.addressof(u)
 groups = (Group * 1)(Group(1, px, px, px, n, pu, None))
-lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int] + [C.c_void_p] * 3
 lib.ot_batch_destroy.argtypes = [C.c_void_p]
 before = fake.fake_live(MALLOC)
 def create():
@@ -212,13 +213,13 @@ destroy(h)
 
 
 def test_what_a_reset_took_is_not_freed_again(child):
-    """Octrees (with tables) and batches of a destroyed context are dropped without releasing anything: their addresses are
-    not theirs any more, and may be a newer octree's."""
+    """Octrees (with tables) and batches of a destroyed context are dropped without releasing anything: their
+    addresses are not theirs any more, and may be a newer octree's."""
     child("""
 class Group(C.Structure):
     _fields_ = [("kernel", C.c_int), ("x", C.c_void_p), ("y", C.c_void_p), ("z", C.c_void_p), ("n", C.c_int64),
                 ("u", C.c_void_p), ("host", C.c_void_p)]
-lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int] + [C.c_void_p] * 3
 lib.ot_batch_destroy.argtypes = [C.c_void_p]
 x, u = (C.c_double * 64)(), (C.c_float * 192)()
 px, pu = C.addressof(x), C.addressof(u)
