@@ -512,23 +512,26 @@ extern "C" ot_status ot_batch_create(const ot_octree* t, const ot_group* groups,
         GroupDev& d = a.g[k];
         if (d.kernel != OT_TRILINEAR || d.n < 64 || !order_fits(d.n, order_level)) continue;
         Ordered o{k, d, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-        void* p = nullptr;
-        const size_t bytes = order_ws_bytes(d.n) + 3 * sizeof(double) * (size_t)d.n + 3 * sizeof(float) * (size_t)d.n +
-                             sizeof(int32_t) * (size_t)d.n + 4 * 256;
-        if ((e = cudaMalloc(&p, bytes)) != cudaSuccess) return fail(e);
-        b->bufs.push_back(p);
-        char* c = static_cast<char*>(p);
-        auto take = [&](size_t sz) {
-            char* r = c;
-            c += (sz + 255) & ~(size_t)255;
-            return r;
+        // the pieces from `base`, each on 256 bytes; the bytes they take (base null: only that)
+        auto carve = [&](char* base) {
+            size_t at = 0;
+            auto take = [&](size_t sz) {
+                char* r = base ? base + at : nullptr;
+                at += (sz + 255) & ~(size_t)255;
+                return r;
+            };
+            o.pairs = reinterpret_cast<uint64_t*>(take(order_ws_bytes(d.n)));
+            o.xs = reinterpret_cast<double*>(take(sizeof(double) * d.n));
+            o.ys = reinterpret_cast<double*>(take(sizeof(double) * d.n));
+            o.zs = reinterpret_cast<double*>(take(sizeof(double) * d.n));
+            o.us = reinterpret_cast<float*>(take(3 * sizeof(float) * d.n));
+            if (d.host) o.hs = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * d.n));
+            return at;
         };
-        o.pairs = reinterpret_cast<uint64_t*>(take(order_ws_bytes(d.n)));
-        o.xs = reinterpret_cast<double*>(take(sizeof(double) * d.n));
-        o.ys = reinterpret_cast<double*>(take(sizeof(double) * d.n));
-        o.zs = reinterpret_cast<double*>(take(sizeof(double) * d.n));
-        o.us = reinterpret_cast<float*>(take(3 * sizeof(float) * d.n));
-        o.hs = d.host ? reinterpret_cast<int32_t*>(take(sizeof(int32_t) * d.n)) : nullptr;
+        void* p = nullptr;
+        if ((e = cudaMalloc(&p, carve(nullptr))) != cudaSuccess) return fail(e);
+        b->bufs.push_back(p);
+        carve(static_cast<char*>(p));
         d.x = o.xs, d.y = o.ys, d.z = o.zs, d.u = o.us, d.host = o.hs;
         ordered.push_back(o);
     }

@@ -139,6 +139,28 @@ int cudaLaunchKernel(const void* f, struct dim g, struct dim b, void** a, size_t
     if (n_batch < 8) batch[n_batch++] = *(struct batch_args*)a[1];
     return OK;
 }
+/* bytes from p to the end of the allocation that holds it, as it was asked for; -1: in none */
+static long long room(const void* p) {
+    for (int i = 0; i < MAX_BLOCKS; ++i) {
+        const char* b = blocks[i].p;
+        if (b && (const char*)p >= b && (const char*)p < b + blocks[i].bytes) return b + blocks[i].bytes - (const char*)p;
+    }
+    return -1;
+}
+/* whether group g's arrays of launch i (positions and results) lie within their allocations, apart from one another */
+int fake_batch_fits(int i, int g) {
+    const long long n = batch[i].g[g].n;
+    const char* a[5] = {(const char*)batch[i].g[g].x, (const char*)batch[i].g[g].y, (const char*)batch[i].g[g].z,
+                        (const char*)batch[i].g[g].u, (const char*)batch[i].g[g].host};
+    const long long bytes[5] = {8 * n, 8 * n, 8 * n, 12 * n, 4 * n};
+    for (int k = 0; k < 5; ++k) {
+        if (!a[k]) continue;
+        if (room(a[k]) < bytes[k]) return 0;
+        for (int j = 0; j < k; ++j)
+            if (a[j] && a[k] < a[j] + bytes[j] && a[j] < a[k] + bytes[k]) return 0;
+    }
+    return 1;
+}
 int fake_batch_launches(void) { return n_batch; }
 int fake_batch_kernel(int i) { return batch[i].g[0].kernel; }
 int fake_batch_pts(int i) { return batch[i].pts; }

@@ -240,3 +240,29 @@ assert lib.ot_batch_destroy(new_batch) == 0
 destroy(new)
 assert fake.fake_live(POOL) == 0 and fake.fake_bad_frees() == 0
 """)
+
+
+def test_ordered_copies_fit_their_allocation(child):
+    """The ordered copies of a group's positions and results, for every size modulo their alignment, with hosts and
+    without."""
+    child("""
+class Group(C.Structure):
+    _fields_ = [("kernel", C.c_int), ("x", C.c_void_p), ("y", C.c_void_p), ("z", C.c_void_p), ("n", C.c_int64),
+                ("u", C.c_void_p), ("host", C.c_void_p)]
+lib.ot_batch_create.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int] + [C.c_void_p] * 3
+lib.ot_batch_destroy.argtypes = [C.c_void_p]
+st, h = build(3)
+x, u = (C.c_double * 64)(), (C.c_float * 192)()
+px, pu = C.addressof(x), C.addressof(u)
+launch = (C.c_int * 7)(0, 0, 0, 5, 0, 0, 0)
+wrong = []
+for n in [*range(64, 64 + 513), *range(4090, 4110), 100_003]:
+    groups = (Group * 2)(Group(1, px, px, px, n, pu, pu), Group(1, px, px, px, n, pu, None))
+    fake.fake_forget_batches()
+    b = C.c_void_p()
+    assert lib.ot_batch_create(h, groups, 2, u, 0, launch, None, C.byref(b)) == 0
+    wrong += [n for g in range(2) if not fake.fake_batch_fits(0, g)]
+    assert lib.ot_batch_destroy(b) == 0
+assert not wrong, wrong
+destroy(h)
+""")
