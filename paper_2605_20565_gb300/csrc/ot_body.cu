@@ -70,14 +70,16 @@ __device__ __forceinline__ void add_small_product(Sum3& s, const float r[3], flo
 // markers with a coordinate of 1 or more, closer to their body's centre than the cut at 2^-62
 // allows, or with a value that floats cannot multiply exactly (below 2^-40, above 2^74, not
 // finite) are summed in FP64.
-// DV: marker volumes given.
-template <bool DV>
-__global__ void __launch_bounds__(BT) k_body_sums(const double* __restrict__ x, const double* __restrict__ y,
+// DV: marker volumes given.  MINB: blocks per SM that the registers allow.
+template <bool DV, int MINB>
+__global__ void __launch_bounds__(BT, MINB) k_body_sums(const double* __restrict__ x, const double* __restrict__ y,
                                                   const double* __restrict__ z, const float* __restrict__ v,
                                                   const float* __restrict__ dV, float w, int64_t n,
                                                   const int64_t* __restrict__ start, const double* __restrict__ xb,
                                                   double scale, double* __restrict__ lin, double* __restrict__ ang) {
-    __shared__ double s_warp[6][BT / 32];
+    __shared__ float s_float[6][BT / 32][3];
+    __shared__ double s_double[6][BT / 32];
+    __shared__ bool s_used[BT / 32];
     __shared__ double s_sum[6];
     cg::cluster_group cluster = cg::this_cluster();
     const int nb = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
@@ -86,6 +88,7 @@ __global__ void __launch_bounds__(BT) k_body_sums(const double* __restrict__ x, 
     const double cx = xb[3 * b], cy = xb[3 * b + 1], cz = xb[3 * b + 2];
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     Sum3 sum[6];
+    bool used = false;  // acc
     long long f0, f1, f2;
     bool t0, t1, t2;
     bool centre = to_fixed(cx, f0, t0);
@@ -133,6 +136,7 @@ __global__ void __launch_bounds__(BT) k_body_sums(const double* __restrict__ x, 
         } else {
             const double s0 = (double)w0 * (double)wk, s1 = (double)w1 * (double)wk, s2 = (double)w2 * (double)wk;
             const double r0 = X - cx, r1 = Y - cy, r2 = Z - cz;
+            used = true;
             acc[0] += s0;
             acc[1] += s1;
             acc[2] += s2;
@@ -141,32 +145,58 @@ __global__ void __launch_bounds__(BT) k_body_sums(const double* __restrict__ x, 
             acc[5] = fma(r0, s1, fma(-r1, s0, acc[5]));
         }
     }
-#pragma unroll
-    for (int c = 0; c < 6; ++c) acc[c] += sum[c].value();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t mine = k1 - k0 - rank * BT;  // markers from the block's first on
+    const int nw = mine <= 0 ? 0 : mine < BT ? ((int)mine + 31) / 32 : BT / 32;  // warps with markers
+    if (warp < nw) {
+        // the lanes' sums and then the warps', in three floats still (in FP64 the conversions and the tree were
+        // most of the time of bodies of a few hundred markers: 5,000 of 200 markers 183 -> 105 us)
+        const bool doubles = __any_sync(0xffffffffu, used);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) {
+        for (int c = 0; c < 6; ++c) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-        if (lane == 0) s_warp[c][warp] = acc[c];
+            for (int o = 16; o > 0; o >>= 1) {
+                Sum3 v;
+                v.a = __shfl_down_sync(0xffffffffu, sum[c].a, o);
+                v.b = __shfl_down_sync(0xffffffffu, sum[c].b, o);
+                v.c = __shfl_down_sync(0xffffffffu, sum[c].c, o);
+                sum[c].add(v);
+            }
+            if (doubles)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+            if (lane == 0) {
+                s_float[c][warp][0] = sum[c].a, s_float[c][warp][1] = sum[c].b, s_float[c][warp][2] = sum[c].c;
+                s_double[c][warp] = acc[c];
+            }
+        }
+        if (lane == 0) s_used[warp] = doubles;
     }
     __syncthreads();
     if (threadIdx.x < 6) {
-        double a = 0.0;
-        for (int k = 0; k < BT / 32; ++k) a += s_warp[threadIdx.x][k];
-        s_sum[threadIdx.x] = a;
+        Sum3 a;
+        double d = 0.0;
+        for (int k = 0; k < nw; ++k) {
+            const float* f = s_float[threadIdx.x][k];
+            a.add(f[0]), a.low(f[1]), a.last(f[2]);
+            if (s_used[k]) d += s_double[threadIdx.x][k];
+        }
+        s_sum[threadIdx.x] = d + a.value();
     }
-    cluster.sync();
+    if (nb > 1)
+        cluster.sync();
+    else
+        __syncthreads();
     if (rank == 0 && threadIdx.x < 6) {
         double a = 0.0;
         for (int k = 0; k < nb; ++k) a += *cluster.map_shared_rank(&s_sum[threadIdx.x], k);
         if (!DV) a *= (double)w;
         (threadIdx.x < 3 ? lin : ang)[3 * b + threadIdx.x % 3] = scale * a;
     }
-    cluster.sync();  // the partial sums stay until they are read
+    if (nb > 1) cluster.sync();  // the partial sums stay until they are read
 }
 
-template <bool DV>
+template <bool DV, int MINB>
 cudaError_t launch_body(int blocks, int nb, cudaStream_t s, const double* x, const double* y, const double* z,
                         const float* v, const float* dV, float w, int64_t n, const int64_t* start, const double* xb,
                         double scale, double* lin, double* ang) {
@@ -180,7 +210,7 @@ cudaError_t launch_body(int blocks, int nb, cudaStream_t s, const double* x, con
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_body_sums<DV>, x, y, z, v, dV, w, n, start, xb, scale, lin, ang);
+    return cudaLaunchKernelEx(&cfg, k_body_sums<DV, MINB>, x, y, z, v, dV, w, n, start, xb, scale, lin, ang);
 }
 
 } // namespace
@@ -195,17 +225,21 @@ extern "C" ot_status ot_body_sums(const double* d_x, const double* d_y, const do
     if (n < 0 || n_bodies < 0 || n_bodies > (1 << 24)) return OT_ERR_ARG;
     if (n_bodies == 0) return OT_OK;
     if (!d_start || !d_xb || !d_lin || !d_ang || (n > 0 && (!d_x || !d_y || !d_z || !d_v))) return OT_ERR_ARG;
-    // blocks per body: up to the portable cluster size while all of them are at most 6 per SM (3 are
-    // resident by their registers; the rest start as small bodies' end), one when the bodies alone
-    // are that many or the markers are few.  Lines of 3, 6 and 1000 per SM: 64 bodies of different
+    // blocks per body: up to the portable cluster size while all of them are at most 6 per SM (more than
+    // are resident at once: large bodies get their share as small ones end), one when the bodies
+    // alone are that many or the markers are few.  Lines of 3, 6 and 1000 per SM: 64 bodies of different
     // sizes 349, 277 and 277 us (7.5M markers), 156, 95 and 95 us (2M with volumes), 64 of one size
-    // 175, 178 and 185 us, 1,000 of one size 156, 154 and 384 us.
+    // 175, 178 and 185 us, 1,000 of one size 156, 154 and 384 us
     int nb = 8;
     while (nb > 1 && ((int64_t)n_bodies * nb > 6 * (int64_t)num_sms() || (int64_t)n_bodies * nb * BT > 4 * n)) nb >>= 1;
-    OT_CUDA(d_dV ? launch_body<true>(n_bodies * nb, nb, (cudaStream_t)stream, d_x, d_y, d_z, d_v, d_dV, w, n, d_start,
-                                     d_xb, scale, d_lin, d_ang)
-                 : launch_body<false>(n_bodies * nb, nb, (cudaStream_t)stream, d_x, d_y, d_z, d_v, d_dV, w, n, d_start,
-                                      d_xb, scale, d_lin, d_ang));
+    // registers: 99 to 121 (2 blocks per SM) while the blocks are few and long, 80 (3 blocks) for many,
+    // which are short.  2 and 3 blocks: 64 bodies of 7.5M and 2M markers 379 and 433 us together, 5,000
+    // bodies of 5M 206 and 177, of 1M 105 and 88, of 100,000 86 and 63
+    const int blocks = n_bodies * nb;
+    const bool few = blocks <= 6 * num_sms();
+    const auto launch = d_dV ? (few ? launch_body<true, 2> : launch_body<true, 3>)
+                             : (few ? launch_body<false, 2> : launch_body<false, 3>);
+    OT_CUDA(launch(blocks, nb, (cudaStream_t)stream, d_x, d_y, d_z, d_v, d_dV, w, n, d_start, d_xb, scale, d_lin, d_ang));
     count_launch();
     return OT_OK;
 }

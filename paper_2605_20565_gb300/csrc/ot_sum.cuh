@@ -22,6 +22,7 @@ struct Sum3 {
     // terms some 2^-20 (low) and 2^-40 (last) below the others
     __device__ __forceinline__ void low(float v) { c = __fadd_rn(c, two_sum(b, v)); }
     __device__ __forceinline__ void last(float v) { c = __fadd_rn(c, v); }
+    __device__ __forceinline__ void add(const Sum3& v) { add(v.a), low(v.b), last(v.c); }
     __device__ __forceinline__ double value() const { return ((double)c + (double)b) + (double)a; }
 };
 // v is zero or 2^-40 <= |v| < 2^74: its products with multiples of 2^-62 below 1, and their rounding
