@@ -218,15 +218,17 @@ __device__ __forceinline__ int delta_sum(const TreeView& t, const T* __restrict_
     if (__any_sync(FULLM, search)) {  // no table, or the middle block is not refined to the finest level
         const int lp = t.lmax - 1, np_cells = 1 << lp, shp = MAXLEVEL - lp;
         int* blk = sg.blk[lane >> 3];
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const int k = ch + 8 * s, b[3] = {k % 3, (k / 3) % 3, k / 9};
-            bool inside = search && k < 27;
+        // the blocks that the stencil overlaps, 2 per axis or, for odd first cells of 4, 3: a search per
+        // lane and round (1 to 4 rounds; always 1 for the 3-point stencil)
+        const int n0 = 2 + (W == 4 ? (int)bits & 1 : 0), n1 = 2 + (W == 4 ? (int)(bits >> 1) & 1 : 0);
+        const int cnt = search ? n0 * n1 * (2 + (W == 4 ? (int)(bits >> 2) & 1 : 0)) : 0;
+        for (int i = ch; __any_sync(FULLM, i < cnt); i += 8) {
+            const int r = n0 == 2 ? i >> 1 : i / 3, z = n1 == 2 ? r >> 1 : r / 3;
+            const int b[3] = {i - n0 * r, r - n1 * z, z};
+            bool inside = i < cnt;
             uint64_t q = 0;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                // the stencil overlaps 3 blocks on an axis only for odd first cells of 4
-                inside = inside && (b[d] < 2 || (W == 4 && ((bits >> d) & 1u)));
                 int v = sg.p0[d][m] + b[d];
                 if (t.periodic) v = (v + np_cells) & (np_cells - 1);
                 inside = inside && v >= 0 && v < np_cells;
@@ -234,7 +236,7 @@ __device__ __forceinline__ int delta_sum(const TreeView& t, const T* __restrict_
             }
             int f = -1;
             if (inside) f = find_block<LEARNED>(t, q);
-            if (k < 27) blk[k] = f;
+            if (i < cnt) blk[b[0] + 3 * b[1] + 9 * b[2]] = f;
         }
         __syncwarp();
     }
