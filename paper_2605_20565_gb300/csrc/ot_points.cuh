@@ -135,9 +135,8 @@ __device__ __forceinline__ bool visit_stencil(const TreeView& t, const int i0[3]
 // independent loads, and so are the 8 values, which the marker's lanes read from the same lines (a
 // block's 8 leaves are 128 consecutive bytes in FP32).  A lane per marker walked 8 to 27 blocks in
 // turn with 64 loads, each from a line of its own: bound by L1, and for few markers by that chain.
-// 2M markers 506 -> 301 us, 1M without the table 430 -> 373 us (there a lane's 4 block searches are
-// half of the instructions), 1,000 markers 79 -> 5.5 us.  Forming the weights by 8 lanes per
-// marker too, without the stage: 392 us.
+// 2M markers 506 -> 301 us, 1M without the table (uniform level 6) 537 -> 297 us, 1,000 markers
+// 79 -> 5.5 us.  Forming the weights by 8 lanes per marker too, without the stage: 392 us.
 // The lanes' sums are added in a fixed tree, the same with and without the parent-block table.
 template <typename T>
 struct DeltaStage {
@@ -146,7 +145,24 @@ struct DeltaStage {
     int p0[3][32];     // first block per axis
     uint32_t bits[32]; // parity of the first cell (bits 0-2), host's slot (2 bits each from 4), inside the cube (16)
     int blk[4][28];    // without the table: first leaves of the 27 blocks from p0, of 4 markers
+    T off[sizeof(T) == 8 ? 3 : 1][33];  // FP64: offset from the centre of the finest cell per axis
 };
+
+// FP64: the weights of the stage's first cnt markers, an evaluation per lane and round whatever their
+// number.  By a lane per marker the few markers of a warp cost the FP64 pipe as much as 32: 3,000 and
+// 30,000 3-point markers 35 -> 27 and 89 -> 65 us with the table.  The slots of one branch of the
+// delta function come together.
+template <int K>
+__device__ __forceinline__ void stage_weights(DeltaStage<double>& sg, int cnt) {
+    using S = Stencil<K>;
+    constexpr int W = S::W, INNER = W == 4 ? 2 : 1;  // slots per axis within one cell of the marker
+    for (int i = threadIdx.x & 31; i < 3 * W * cnt; i += 32) {
+        const int j = i / cnt, m = i - j * cnt, o = j - 3 * INNER;
+        const int d = o < 0 ? j / INNER : o >> 1, a = o < 0 ? 1 + j % INNER : (W - 1) * (o & 1);
+        const int hc = (sg.bits[m] >> (4 + 2 * d)) & 3;
+        sg.w[4 * d + a][m] = S::template phi<double>((double)(hc - a) + sg.off[d][m]);
+    }
+}
 
 template <typename T, int K, bool LEARNED>
 __device__ __forceinline__ void delta_stage(const TreeView& t, DeltaStage<T>& sg, bool active, double x, double y,
@@ -161,8 +177,20 @@ __device__ __forceinline__ void delta_stage(const TreeView& t, DeltaStage<T>& sg
     int row = -1;
     if (ok) {
         int i0[3];
-        T w[3][W];
-        stencil_weights<K, T>(t.lmax, X, i0, w);
+        if constexpr (sizeof(T) == 4) {
+            T w[3][W];
+            stencil_weights<K, T>(t.lmax, X, i0, w);
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+#pragma unroll
+                for (int k = 0; k < W; ++k) sg.w[4 * d + k][lane] = w[d][k];
+        } else {  // stage_weights, once all markers are here
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                i0[d] = S::first((int)fix_cell(X[d], t.lmax), fix_upper_half(X[d], t.lmax) ? 1 : 0);
+                sg.off[d][lane] = fix_offset<T>(X[d], t.lmax);
+            }
+        }
         bool inside = true;
         uint64_t q = 0;
 #pragma unroll
@@ -171,8 +199,6 @@ __device__ __forceinline__ void delta_stage(const TreeView& t, DeltaStage<T>& sg
             bits |= (uint32_t)par << d;
             bits |= (uint32_t)((int)fix_cell(X[d], t.lmax) - i0[d]) << (4 + 2 * d);
             sg.p0[d][lane] = p0;
-#pragma unroll
-            for (int k = 0; k < W; ++k) sg.w[4 * d + k][lane] = w[d][k];
             // every block of the stencil lies within one of the middle one
             int qm = p0 + (W == 4 ? par : 0);
             if (t.periodic) qm = (qm + np_cells) & (np_cells - 1);
@@ -188,11 +214,12 @@ __device__ __forceinline__ void delta_stage(const TreeView& t, DeltaStage<T>& sg
     sg.bits[lane] = bits;
 }
 
-// The sum of marker m of the stage by its 8 lanes (m differs between them in the warp); returns the
-// host leaf when want_host and the finest cell that holds the marker is a leaf, else -1.
+// The sum of marker m of the stage by its 8 lanes (m differs between them in the warp): lanes 0 to 2
+// receive its components.  Returns the host leaf when the finest cell that holds the marker is
+// one, else -1.
 template <typename T, int K, bool LEARNED>
 __device__ __forceinline__ int delta_sum(const TreeView& t, const T* __restrict__ field, DeltaStage<T>& sg, int m,
-                                         T out[3]) {
+                                         T& out) {
     using V = Vec4<T>;
     constexpr int W = Stencil<K>::W;
     constexpr unsigned FULLM = 0xffffffffu;
@@ -269,16 +296,18 @@ __device__ __forceinline__ int delta_sum(const TreeView& t, const T* __restrict_
         if (e == eh) host = at;
     }
     if (missing) atomicOr(t.err, (unsigned)OT_DEV_STENCIL);
+    // the 8 lanes' sums, by pairs: after each exchange a lane goes on with its half of the components (4
+    // additions per lane instead of 9, in the same order)
+    T v = (ch & 1) ? s1 : s0;
+    v += __shfl_xor_sync(FULLM, (ch & 1) ? s0 : s1, 1);
+    s2 += __shfl_xor_sync(FULLM, s2, 1);
+    const T give = (ch & 2) ? v : s2;
+    v = (ch & 2) ? s2 : v;
+    v += __shfl_xor_sync(FULLM, give, 2);
+    v += __shfl_xor_sync(FULLM, v, 4);
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        s0 += __shfl_xor_sync(FULLM, s0, o);
-        s1 += __shfl_xor_sync(FULLM, s1, o);
-        s2 += __shfl_xor_sync(FULLM, s2, o);
-        host = max(host, __shfl_xor_sync(FULLM, host, o));
-    }
-    out[0] = ok ? s0 : qnan<T>();
-    out[1] = ok ? s1 : qnan<T>();
-    out[2] = ok ? s2 : qnan<T>();
+    for (int o = 1; o < 8; o <<= 1) host = max(host, __shfl_xor_sync(FULLM, host, o));
+    out = ok ? v : qnan<T>();
     return host;
 }
 
@@ -295,14 +324,18 @@ __device__ __forceinline__ void delta_markers(const TreeView& t, const T* __rest
     if (mine < end) px = x[mine], py = y[mine], pz = z[mine];
     delta_stage<T, K, LEARNED>(t, sg, mine < end, px, py, pz);
     __syncwarp();
+    if constexpr (sizeof(T) == 8) {
+        stage_weights<K>(sg, (int)(end - base));
+        __syncwarp();
+    }
     const bool ok = (sg.bits[lane] >> 16) & 1u;
     if (mine < end && !ok) atomicOr(t.err, (unsigned)OT_DEV_OUTSIDE);
     for (int64_t b = base; b < end; b += 4) {  // warp-uniform
         const int m = (int)(b - base) + (lane >> 3);
-        T o[3];
+        T o;
         const int h = delta_sum<T, K, LEARNED>(t, field, sg, m, o);
         // results in the place of the marker's weights and row, stored by all lanes together below
-        if (ch < 3) sg.w[ch][m] = ch == 0 ? o[0] : ch == 1 ? o[1] : o[2];
+        if (ch < 3) sg.w[ch][m] = o;
         if (ch == 3) sg.row[m] = h;
         __syncwarp();
     }
