@@ -429,8 +429,10 @@ template <typename T> struct TileOut {
 // and summed in segments of SEG list places, each from zero and the segments in order, so that
 // the result does not depend on who sums which: one warp per run takes its tiles whole or, when the
 // runs are too few to fill the chip, one block per tile deals the segments to its warps.
-// Lane: column (x, y) = (lane & 3, lane >> 2 & 3) and the cells z = 2 (lane >> 4), + 1, whose sums
-// it keeps in registers; a marker is staged by one lane and costs the warp 3 shared loads, 2
+// Lane: column (x, y) = (lane & 3, lane >> 2 & 3) and the cells z = 2 (lane >> 4), + 1 (in FP64 z = lane
+// >> 4, + 2: more than half of the stencils reach only the lower or only the upper two layers of a
+// tile, and the products of the other ones, which the FP64 pipe bounds, are left out: 1M 3-point markers
+// at 8 to a cell 2,737 -> 2,165 us, Peskin-4 4,058 -> 3,307 us), whose sums it keeps in registers; a marker is staged by one lane and costs the warp 3 shared loads, 2
 // products and 6 fused multiply-adds.  A cell whose sums are all zero is left as it is.
 // The line of 4096 runs, some 5 blocks of 4 warps on each of 152 SMs, FP32 spreading by warps per run and
 // by blocks per tile: 500,000 markers in 750, 3,000, 5,800 and 11,700 runs 670/295, 298/282, 259/334
@@ -445,6 +447,7 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
                                                         const uint32_t* __restrict__ n_runs,
                                                         const MarkerRec<T>* __restrict__ recs, TileOut<T> out) {
     constexpr int W = Stencil<K>::W, NW = TILE_T / 32;
+    constexpr bool HALVES = sizeof(T) == 8;  // a lane's cells are 2 apart, one in each half of the tile
     constexpr unsigned FULLM = 0xffffffffu;
     __shared__ TileStage<T> s_stage[NW];
     __shared__ T s_part[NW][6][32];
@@ -513,9 +516,17 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
                                                         (uint32_t)(2 * tc[1] + ((s >> 1) & 1)) << shb,
                                                         (uint32_t)(2 * tc[2] + (s >> 2)) << shb));
             const unsigned valid = __ballot_sync(FULLM, a0 >= 0) & 0xffu;
-            const int mine0 = __shfl_sync(FULLM, a0, (cx >> 1) | ((cy >> 1) << 1) | (zh << 2));
-            const int leaf = mine0 + ((cx & 1) | ((cy & 1) << 1));  // and leaf + 4 above it
-            if (mine0 >= 0) {
+            // this lane's two cells: leaf and the one above it in its block, or (HALVES) leaf and leaf1 of the
+            // blocks above one another
+            const int mine0 = __shfl_sync(FULLM, a0, (cx >> 1) | ((cy >> 1) << 1) | (HALVES ? 0 : zh << 2));
+            const int leaf = mine0 + ((cx & 1) | ((cy & 1) << 1) | (HALVES ? zh << 2 : 0));
+            int mine1 = -1, leaf1 = 0;
+            if constexpr (HALVES) {
+                mine1 = __shfl_sync(FULLM, a0, (cx >> 1) | ((cy >> 1) << 1) | 4);
+                leaf1 = mine1 + (leaf - mine0);
+                if (mine0 >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(out.f + 4 * (size_t)leaf));
+                if (mine1 >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(out.f + 4 * (size_t)leaf1));
+            } else if (mine0 >= 0) {
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(out.f + 4 * (size_t)leaf));
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(out.f + 4 * (size_t)(leaf + 4)));
             }
@@ -574,13 +585,29 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
                 }
                 __syncwarp();
                 if (!slow) {
+                    if constexpr (HALVES) {
+                        // (a loop per half: a product that is only predicated off takes the pipe all the same)
+                        const unsigned reach[2] = {__ballot_sync(FULLM, over && rel[2] <= 1),
+                                                   __ballot_sync(FULLM, over && rel[2] + W > 2)};
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+#pragma unroll 2
+                            for (unsigned todo = reach[e]; todo; todo &= todo - 1u) {
+                                const int j = __popc(m & ((todo & (0u - todo)) - 1u));  // its place in the stage
+                                T Fj[4];
+                                load4(sg.F[j], Fj);
+                                acc[e].add(sg.wxy[lane & 15][j] * sg.wz[e][j][zh], Fj[0], Fj[1], Fj[2]);
+                            }
+                        }
+                    } else {
 #pragma unroll 4
-                    for (int j = 0; j < cnt; ++j) {
-                        const T xy = sg.wxy[lane & 15][j];
-                        T Fj[4];
-                        load4(sg.F[j], Fj);
-                        acc[0].add(xy * sg.wz[zh][j][0], Fj[0], Fj[1], Fj[2]);
-                        acc[1].add(xy * sg.wz[zh][j][1], Fj[0], Fj[1], Fj[2]);
+                        for (int j = 0; j < cnt; ++j) {
+                            const T xy = sg.wxy[lane & 15][j];
+                            T Fj[4];
+                            load4(sg.F[j], Fj);
+                            acc[0].add(xy * sg.wz[zh][j][0], Fj[0], Fj[1], Fj[2]);
+                            acc[1].add(xy * sg.wz[zh][j][1], Fj[0], Fj[1], Fj[2]);
+                        }
                     }
                 } else {  // the stencil's own cells only
                     for (int j = 0; j < cnt; ++j) {
@@ -588,8 +615,9 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
                         if ((cover & cells) != cells) continue;
 #pragma unroll
                         for (int e = 0; e < 2; ++e)
-                            if ((cover >> (8 + 2 * zh + e)) & 1u)
-                                acc[e].add(sg.wxy[lane & 15][j] * sg.wz[zh][j][e], sg.F[j][0], sg.F[j][1], sg.F[j][2]);
+                            if ((cover >> (8 + (HALVES ? zh + 2 * e : 2 * zh + e))) & 1u)
+                                acc[e].add(sg.wxy[lane & 15][j] * (HALVES ? sg.wz[e][j][zh] : sg.wz[zh][j][e]),
+                                           sg.F[j][0], sg.F[j][1], sg.F[j][2]);
                     }
                 }
                 __syncwarp();
@@ -622,7 +650,10 @@ __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o,
                 }
                 if (warp != 0) continue;  // every warp has the sums; one writes them
             }
-            if (mine0 >= 0) {
+            if constexpr (HALVES) {
+                if (mine0 >= 0 && !sum[0].zero()) out.add(leaf, sum[0]);
+                if (mine1 >= 0 && !sum[1].zero()) out.add(leaf1, sum[1]);
+            } else if (mine0 >= 0) {
                 if (!sum[0].zero()) out.add(leaf, sum[0]);
                 if (!sum[1].zero()) out.add(leaf + 4, sum[1]);
             }
