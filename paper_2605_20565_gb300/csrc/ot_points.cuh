@@ -227,19 +227,22 @@ __device__ __forceinline__ int delta_sum(const TreeView& t, const T* __restrict_
     const uint32_t bits = sg.bits[m];
     const bool ok = (bits >> 16) & 1u;
     const int row = sg.row[m];
-    int a[3], b0[3];   // this lane's first slot, and its block relative to p0
-    bool two[3];       // slot a + 2 is in the stencil
-    T w[3][2];
-    int eh = 0;        // the host's cell among this lane's, 8 or more: another lane's
+    constexpr bool CELLS = W == 3 && sizeof(T) == 8;  // 27 cells dealt to the lanes, below
+    [[maybe_unused]] int a[3], b0[3];  // this lane's first slot, and its block relative to p0
+    [[maybe_unused]] bool two[3];      // slot a + 2 is in the stencil
+    [[maybe_unused]] T w[3][2];
+    [[maybe_unused]] int eh = 0;       // the host's cell among this lane's, 8 or more: another lane's
+    if constexpr (!CELLS) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const int par = (bits >> d) & 1, cd = (ch >> d) & 1, hc = (bits >> (4 + 2 * d)) & 3;
-        a[d] = cd ^ par;
-        b0[d] = par & ~cd;
-        two[d] = W == 4 || a[d] == 0;
-        w[d][0] = sg.w[4 * d + a[d]][m];
-        w[d][1] = two[d] ? sg.w[4 * d + a[d] + 2][m] : T(0);
-        eh = ((hc ^ a[d]) & 1) ? 8 : eh + (((hc - a[d]) >> 1) << d);
+        for (int d = 0; d < 3; ++d) {
+            const int par = (bits >> d) & 1, cd = (ch >> d) & 1, hc = (bits >> (4 + 2 * d)) & 3;
+            a[d] = cd ^ par;
+            b0[d] = par & ~cd;
+            two[d] = W == 4 || a[d] == 0;
+            w[d][0] = sg.w[4 * d + a[d]][m];
+            w[d][1] = two[d] ? sg.w[4 * d + a[d] + 2][m] : T(0);
+            eh = ((hc ^ a[d]) & 1) ? 8 : eh + (((hc - a[d]) >> 1) << d);
+        }
     }
     const bool search = ok && row < 0;
     if (__any_sync(FULLM, search)) {  // no table, or the middle block is not refined to the finest level
@@ -267,33 +270,66 @@ __device__ __forceinline__ int delta_sum(const TreeView& t, const T* __restrict_
         }
         __syncwarp();
     }
-    int leaf[8];  // by e = ex + 2 ey + 4 ez: the cell's block, -1 when missing, -2 past the stencil
-    const int k0 = b0[0] + 3 * b0[1] + 9 * b0[2];
-    // the table's row starts one block before the middle one
-    const int pm = W == 4 ? (int)bits & 7 : 0;
-    const int kr = k0 + 13 - (pm & 1) - 3 * ((pm >> 1) & 1) - 9 * (pm >> 2);
-    const int* __restrict__ rp = t.pnbr + 32 * (size_t)max(row, 0) + kr;
-    const int* sp = sg.blk[lane >> 3] + k0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
-        const bool in = ok && (!ex || two[0]) && (!ey || two[1]) && (!ez || two[2]);
-        leaf[e] = !in ? -2 : row >= 0 ? __ldg(rp + ex + 3 * ey + 9 * ez) : sp[ex + 3 * ey + 9 * ez];
-    }
     T s0 = T(0), s1 = T(0), s2 = T(0);
     int host = -1;
     bool missing = false;
+    if constexpr (CELLS) {
+        // 27 cells dealt to the lanes in turn, 4 each: by children the fullest lane has 8, and the FP64 pipe
+        // takes as long for one lane as for all (1M markers 1,050 -> 761 us)
+        int leaf[4];  // -1 when missing, -2 past the 27
+        T wt[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        missing = missing || leaf[e] == -1;
-        if (leaf[e] < 0) continue;
-        const int at = leaf[e] + ch;
-        const auto f = V::load(field, at);
-        const T wt = w[0][e & 1] * w[1][(e >> 1) & 1] * w[2][e >> 2];
-        s0 += wt * f.x;
-        s1 += wt * f.y;
-        s2 += wt * f.z;
-        if (e == eh) host = at;
+        for (int r = 0; r < 4; ++r) {
+            const int c = min(ch + 8 * r, 26), cell[3] = {c % 3, (c / 3) % 3, c / 9};
+            int k = 0, child = 0;
+#pragma unroll
+            for (int d = 0, p3 = 1; d < 3; ++d, p3 *= 3) {
+                const int at = (int)((bits >> d) & 1u) + cell[d];
+                k += (at >> 1) * p3;
+                child |= (at & 1) << d;
+            }
+            int first = -2;
+            if (ok && ch + 8 * r < 27)
+                first = row >= 0 ? __ldg(t.pnbr + 32 * (size_t)row + 13 + k) : sg.blk[lane >> 3][k];
+            leaf[r] = first < 0 ? first : first + child;
+            wt[r] = sg.w[cell[0]][m] * sg.w[4 + cell[1]][m] * sg.w[8 + cell[2]][m];
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            missing = missing || leaf[r] == -1;
+            if (leaf[r] < 0) continue;
+            const auto f = V::load(field, leaf[r]);
+            s0 += wt[r] * f.x;
+            s1 += wt[r] * f.y;
+            s2 += wt[r] * f.z;
+            if (ch + 8 * r == 13) host = leaf[r];  // the middle cell
+        }
+    } else {
+        int leaf[8];  // by e = ex + 2 ey + 4 ez: the cell's block, -1 when missing, -2 past the stencil
+        const int k0 = b0[0] + 3 * b0[1] + 9 * b0[2];
+        // the table's row starts one block before the middle one
+        const int pm = W == 4 ? (int)bits & 7 : 0;
+        const int kr = k0 + 13 - (pm & 1) - 3 * ((pm >> 1) & 1) - 9 * (pm >> 2);
+        const int* __restrict__ rp = t.pnbr + 32 * (size_t)max(row, 0) + kr;
+        const int* sp = sg.blk[lane >> 3] + k0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
+            const bool in = ok && (!ex || two[0]) && (!ey || two[1]) && (!ez || two[2]);
+            leaf[e] = !in ? -2 : row >= 0 ? __ldg(rp + ex + 3 * ey + 9 * ez) : sp[ex + 3 * ey + 9 * ez];
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            missing = missing || leaf[e] == -1;
+            if (leaf[e] < 0) continue;
+            const int at = leaf[e] + ch;
+            const auto f = V::load(field, at);
+            const T wt = w[0][e & 1] * w[1][(e >> 1) & 1] * w[2][e >> 2];
+            s0 += wt * f.x;
+            s1 += wt * f.y;
+            s2 += wt * f.z;
+            if (e == eh) host = at;
+        }
     }
     if (missing) atomicOr(t.err, (unsigned)OT_DEV_STENCIL);
     // the 8 lanes' sums, by pairs: after each exchange a lane goes on with its half of the components (4
