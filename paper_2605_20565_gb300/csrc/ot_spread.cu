@@ -12,6 +12,7 @@
 // 1.84 -> 0.65 ms (keys and sort 0.08, records 0.08, tiles 0.49: issue-bound, 58% of the issue slots
 // at 17 warps per SM, half of the instructions staging and per-tile set-up).
 #include <algorithm>
+#include <type_traits>
 
 #include "ot_internal.h"
 #include "ot_points.cuh"
@@ -391,10 +392,11 @@ template <typename T> struct Acc3 {
 __device__ __forceinline__ bool is_finite(float v) { return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u; }
 __device__ __forceinline__ bool is_finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
-// (f may start anywhere, a view into a larger buffer say: wide accesses where it allows them)
+// VEC: f starts on 16 bytes.  It may start at any float, a view into a larger buffer say.
+template <bool VEC>
 __device__ __forceinline__ void add_leaf(float* f, int leaf, const Acc3<float>& a) {
     float* p = f + 4 * (size_t)leaf;
-    if (((uintptr_t)f & 15) == 0) {
+    if constexpr (VEC) {
         const float4 v = *reinterpret_cast<const float4*>(p);
         *reinterpret_cast<float2*>(p) = make_float2(v.x + a.x, v.y + a.y);
         p[2] = v.z + a.z;
@@ -402,6 +404,7 @@ __device__ __forceinline__ void add_leaf(float* f, int leaf, const Acc3<float>& 
         p[0] += a.x, p[1] += a.y, p[2] += a.z;
     }
 }
+template <bool>
 __device__ __forceinline__ void add_leaf(double* f, int leaf, const Acc3<double>& a) {
     double* p = f + 4 * (size_t)leaf;
     p[0] += a.x, p[1] += a.y, p[2] += a.z;
@@ -409,17 +412,17 @@ __device__ __forceinline__ void add_leaf(double* f, int leaf, const Acc3<double>
 
 // Where a tile's sums go: added to f and, scaled, to u when there is one (multi-direct forcing's
 // velocity correction).
-template <typename T> struct TileOut {
+template <typename T, bool VEC> struct TileOut {
     T* f;
     T* u;
     T scale;
     __device__ __forceinline__ void add(int leaf, const Acc3<T>& a) const {
-        add_leaf(f, leaf, a);
+        add_leaf<VEC>(f, leaf, a);
         if constexpr (sizeof(T) == 4) {  // (the forcing is FP32)
             if (!u) return;
             Acc3<T> b;
             b.x = scale * a.x, b.y = scale * a.y, b.z = scale * a.z;
-            add_leaf(u, leaf, b);
+            add_leaf<VEC>(u, leaf, b);
         }
     }
 };
@@ -441,11 +444,11 @@ template <typename T> struct TileOut {
 // markers is not in the rule.
 constexpr int TILE_T = 128, SEG = 64;
 constexpr int64_t WIDE_RUNS = 4096;
-template <typename T, int K>
+template <typename T, int K, bool VEC>
 __global__ void __launch_bounds__(TILE_T) k_tile_reduce(TreeView t, TileOrder o, RunTable rt,
                                                         const uint32_t* __restrict__ runs,
                                                         const uint32_t* __restrict__ n_runs,
-                                                        const MarkerRec<T>* __restrict__ recs, TileOut<T> out) {
+                                                        const MarkerRec<T>* __restrict__ recs, TileOut<T, VEC> out) {
     constexpr int W = Stencil<K>::W, NW = TILE_T / 32;
     constexpr bool HALVES = sizeof(T) == 8;  // a lane's cells are 2 apart, one in each half of the tile
     constexpr unsigned FULLM = 0xffffffffu;
@@ -680,7 +683,7 @@ template <typename T>
 __device__ __forceinline__ void add_unit(T* f, int leaf, T x, T y, T z) {
     Acc3<T> a;
     a.x = x, a.y = y, a.z = z;
-    if (!a.zero()) add_leaf(f, leaf, a);
+    if (!a.zero()) add_leaf<false>(f, leaf, a);
 }
 
 // part (24 sums per block) is not written by a single block, which adds to f.
@@ -849,11 +852,20 @@ ot_status plan_tiles(const ot_octree* t, const double* x, const double* y, const
     return OT_OK;
 }
 
+// Sums to f and, scaled, to u (nullable).  (Whether they allow wide accesses is a template argument: asked
+// per leaf it cost multi-direct forcing on few markers 2%.)
 template <typename T, int K>
-ot_status reduce_tiles(const TreeView& v, const TilePlan<T>& pl, TileOut<T> out, cudaStream_t s) {
-    auto kt = k_tile_reduce<T, K>;
-    kt<<<grid_for(kt, TILE_T, 0, pl.o.n * 8 * TILE_T), TILE_T, 0, s>>>(v, pl.o, pl.rt, pl.runs, pl.n_runs, pl.recs,
-                                                                     out);
+ot_status reduce_tiles(const TreeView& v, const TilePlan<T>& pl, T* f, T* u, T scale, cudaStream_t s) {
+    auto launch = [&](auto vec) {
+        constexpr bool VEC = decltype(vec)::value;
+        auto kt = k_tile_reduce<T, K, VEC>;
+        kt<<<grid_for(kt, TILE_T, 0, pl.o.n * 8 * TILE_T), TILE_T, 0, s>>>(v, pl.o, pl.rt, pl.runs, pl.n_runs, pl.recs,
+                                                                         TileOut<T, VEC>{f, u, scale});
+    };
+    if (sizeof(T) == 8 || (((uintptr_t)f | (uintptr_t)u) & 15) == 0)
+        launch(std::true_type{});
+    else
+        launch(std::bool_constant<sizeof(T) == 8>{});
     count_launch();
     OT_CUDA(cudaGetLastError());
     return OT_OK;
@@ -878,7 +890,7 @@ ot_status spread_sorted(const ot_octree* t, const double* x, const double* y, co
     }
     TilePlan<T> pl;
     const ot_status st = plan_tiles<T, K>(t, x, y, z, F, dV, n, ws, s, pl);
-    return st == OT_OK ? reduce_tiles<T, K>(v, pl, TileOut<T>{f, nullptr, T(0)}, s) : st;
+    return st == OT_OK ? reduce_tiles<T, K>(v, pl, f, nullptr, T(0), s) : st;
 }
 
 // Marker forces of a round of multi-direct forcing, in home-tile order: the velocity interpolated at
@@ -1008,7 +1020,7 @@ ot_status mdf_tiles(const ot_octree* t, const double* x, const double* y, const 
         if (it == n_iter && !slip2) break;  // the last interpolation is for the slip alone
         k<<<grid, REC_T, 0, s>>>(v, pl.o, pl.recs, u, U, dV, 1.0f / dt, per, it < n_iter, slip2 ? slip2 + it : nullptr);
         count_launch();
-        if (it < n_iter) st = reduce_tiles<float, K>(v, pl, TileOut<float>{f, u, dt / rho}, s);
+        if (it < n_iter) st = reduce_tiles<float, K>(v, pl, f, u, dt / rho, s);
     }
     OT_CUDA(cudaGetLastError());
     return st;
