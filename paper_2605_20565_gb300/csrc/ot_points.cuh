@@ -135,7 +135,7 @@ __device__ __forceinline__ bool visit_stencil(const TreeView& t, const int i0[3]
 // independent loads, and so are the 8 values, which the marker's lanes read from the same lines (a
 // block's 8 leaves are 128 consecutive bytes in FP32).  A lane per marker walked 8 to 27 blocks in
 // turn with 64 loads, each from a line of its own: bound by L1, and for few markers by that chain.
-// 2M markers 506 -> 301 us, 1M without the table (uniform level 6) 537 -> 297 us, 1,000 markers
+// 2M markers 506 -> 270 us, 1M without the table (uniform level 6) 537 -> 297 us, 1,000 markers
 // 79 -> 5.5 us.  Forming the weights by 8 lanes per marker too, without the stage: 392 us.
 // The lanes' sums are added in a fixed tree, the same with and without the parent-block table.
 template <typename T>
