@@ -5,8 +5,8 @@
 // default pool, which gives its memory back at every synchronisation (a build has some 25: the
 // sizes of each level), and from cudaMalloc, mapping memory took more than half as long as the
 // build's kernels (17.3M leaves, a re-adaptation 8.68 -> 6.74 ms).  This pool keeps up to
-// POOL_KEEP bytes while octrees live on the device and gives everything back when the last one is
-// destroyed.  Memory pools are safe to use from several threads and streams: a block is handed
+// POOL_KEEP bytes while octrees live on the device and gives them back when the last one is
+// destroyed (one pool per device and context).  Memory pools are safe to use from several threads and streams: a block is handed
 // out again only after the work before its release, in stream order.
 #include <cuda.h>  // driver types only: the two driver calls below are reached through the runtime
 
